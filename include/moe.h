@@ -263,7 +263,8 @@ moe_status moe_expert_ffn_bwd(const moe_config* cfg, const void* x_perm, const i
  *   dx_router[t] = dlogits[t] W_r[p(t)]  (the router's share of the input gradient)
  *                                                               [T,d] dtype out or NULL
  * aux_coef may be NULL (no aux term). bf16: the two products run on the tensor cores
- * with dlogits rounded to bf16 as their operand (fp32 accumulation); fp32: CUDA cores.
+ * with dlogits rounded to bf16 as their operand (fp32 accumulation); fp32: dW_r on the CUDA
+ * cores, dx_router on the split fp32 GEMM.
  * Deterministic: partial sums go to the workspace and are reduced in a fixed order.
  */
 moe_status moe_route_bwd(const moe_config* cfg, const void* x, const void* w_router,

@@ -1,0 +1,622 @@
+// fp32 grouped GEMMs on the tensor cores, for the fp32 configuration: all six expert
+// contractions, the router logits of pools over 64 experts and the router's input
+// gradient. Same argument meaning as the bf16 kernels (moe_internal.h).
+//
+// A TF32 product, or a two-way split, would not hold fp32 results. Here every fp32 operand
+// value is split exactly into three bf16 values, x = h + m + l (each the bf16 nearest to
+// what the ones before left: 3 x 8 bits of significand cover fp32's 24), and a product is
+// the sum of the six bf16 products hh, hm, mh, mm, hl, lh; the three left out are below
+// 2^-25 of it. The tensor core's fp32 accumulator truncates, which over a long contraction
+// loses more than an FFMA chain does, so an accumulator holds only 32 contraction terms
+// (the smallest products first) and is then added to fp32 registers with round-to-nearest.
+// Measured against 64 bits, the worst tensor of a whole fp32 step is 2.4e-7 (512 tokens,
+// d = 256, F = 512) and 5.7e-7 (1501 tokens, d = 1000, F = 1366) off; the FFMA kernels that
+// this replaces were 7.1e-7 and 1.5e-6 off, and accumulators of 64 terms (1.5% faster)
+// 8.3e-7 and 1.1e-6.
+//
+// Roles (one persistent CTA per SM, 128 x BN tiles): 16 producer warps copy fp32 into
+// shared memory up to three stages ahead (cp.async), split it and write three swizzled bf16
+// planes per operand into a ring of two 32-deep stages; one warp issues the 12 MMAs of a
+// stage into one of four TMEM accumulators; 8 warps add the accumulators into registers and
+// run the epilogue. cp.async and not TMA because lines need only 4-byte alignment (any d_ff).
+//
+// What bounds it: shared-memory bandwidth. A 32-deep stage of a 128 x 128 tile is 32 KB of
+// fp32 written and read, 48 KB of planes written, and 96 KB of operand reads by the MMAs;
+// the counters show the LSU pipe at 41% and the tensor pipe's reads at 47% (accumulating an
+// eighth as often, or issuing one MMA of six, changed the time by 10% and 4%). Whole fp32 steps:
+// 1501 tokens, d = 1000, F = 1366, E = 6, k = 3: 5.44 -> 1.35 ms (20 -> 82 TFLOP/s);
+// 512 tokens, d = 256, F = 512, E = 8, k = 2: 494 -> 177 us.
+//
+// An infinite or NaN operand makes 0 * inf terms in the split, so an output element that is
+// not finite is computed again by a plain fp32 FMA chain, which gives IEEE results.
+#include <algorithm>
+#include <type_traits>
+
+#include "moe_internal.h"
+#include "tc_ptx.cuh"
+
+namespace moe {
+namespace f32 {
+
+using namespace tc;
+
+constexpr int FK = 32;                // contraction terms per stage (and per accumulator)
+constexpr int PROD_WARPS = 16, EPI_W = 8;
+constexpr int EPI_WARP0 = PROD_WARPS, MMA_WARP = PROD_WARPS + EPI_W;
+// whole warpgroups, whose registers are split by role: 16 x 64 + 8 x 112 + 4 x 24 registers
+// a lane is exactly the 28 x 72 of the launch (the warps after the MMA warp are idle)
+constexpr int NTHREADS = 32 * (PROD_WARPS + EPI_W + 4);
+constexpr int REG_PROD = 64, REG_EPI = 112, REG_MMA = 24;
+template <int R>
+__device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R)); }
+template <int R>
+__device__ __forceinline__ void reg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R)); }
+constexpr int NBUF = 4;               // TMEM accumulators in flight
+constexpr int FMAX_GROUPS = 256;
+constexpr int ST_FLOATS = 32 * 32;    // transposition buffer per epilogue warp
+
+struct Params {
+    GroupRows rows;
+    int G;
+    const int32_t* gexp;
+    const float* a;
+    const float* b;
+    int64_t b_group_elems;
+    int M, N, K;  // M: output rows per group (K-variable); K: contraction (M-variable)
+    float* out0;
+    float* out1;
+    const float* aux;
+    uint64_t wait_ns;
+    int vec_a, vec_b;  // floats per copy along a contiguous line of each operand (4, 2 or 1)
+};
+
+constexpr uint32_t plane_a() { return BM * FK * 2; }
+constexpr uint32_t plane_b(int bn) { return (uint32_t)bn * FK * 2; }
+constexpr uint32_t stage_bytes(int bn) { return 3 * (plane_a() + plane_b(bn)); }
+constexpr int NST = 2;                // bf16 stages (the MMAs of one, the split into the other)
+constexpr int NRAW = 3;               // fp32 stages: copies in flight ahead of the split
+constexpr uint32_t raw_bytes() { return PROD_WARPS * 2048; }  // a block of each operand per warp
+constexpr uint32_t smem_bytes(int bn) {
+    return 1024 + NST * stage_bytes(bn) + NRAW * raw_bytes() + EPI_W * ST_FLOATS * 4;
+}
+static_assert(smem_bytes(128) + 2048 <= 227 * 1024, "shared memory of one SM");
+
+struct Tile {
+    int g, we, m0, n0, mrows, klen;
+    int64_t a0, b0, o0;
+};
+
+// Asynchronous copy of W floats from global to shared memory, of which the first `bytes`
+// are read and the rest are zero-filled (bytes = 0: nothing is read).
+template <int W>
+__device__ __forceinline__ void cp_async(uint32_t dst, const float* src, int bytes) {
+    if constexpr (W == 4)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;" ::"r"(dst), "l"(src), "r"(bytes), "n"(4 * W)
+                     : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// 8 values -> the three bf16 planes of x = h + m + l, 16 bytes each
+__device__ __forceinline__ void split8(const float* v, uint4* h, uint4* m, uint4* l) {
+    uint32_t* hp = reinterpret_cast<uint32_t*>(h);
+    uint32_t* mp = reinterpret_cast<uint32_t*>(m);
+    uint32_t* lp = reinterpret_cast<uint32_t*>(l);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 hh = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+        const uint32_t hu = *reinterpret_cast<const uint32_t*>(&hh);
+        const float r0 = v[2 * i] - __uint_as_float(hu << 16), r1 = v[2 * i + 1] - __uint_as_float(hu & 0xffff0000u);
+        const __nv_bfloat162 mm = __floats2bfloat162_rn(r0, r1);
+        const uint32_t mu = *reinterpret_cast<const uint32_t*>(&mm);
+        const __nv_bfloat162 ll =
+            __floats2bfloat162_rn(r0 - __uint_as_float(mu << 16), r1 - __uint_as_float(mu & 0xffff0000u));
+        hp[i] = hu;
+        mp[i] = mu;
+        lp[i] = *reinterpret_cast<const uint32_t*>(&ll);
+    }
+}
+
+// One output element by a plain FMA chain (outputs that the split made non-finite).
+__device__ float dot_plain(const float* a, int64_t sa, const float* b, int64_t sb, int K) {
+    float s = 0.f;
+    for (int k = 0; k < K; ++k) s = fmaf(a[k * sa], b[k * sb], s);
+    return s;
+}
+
+template <bool A_MN, bool B_MN, bool VAR_K, int EPI, int BN>
+__global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_constant__ Params p) {
+    pdl_begin();
+    static_assert(BN == 64 || BN == 128, "tile widths");
+    constexpr uint32_t STAGE = stage_bytes(BN);
+    constexpr int CW = BN / 4;       // an epilogue warp owns CW columns of each half of the tile
+    constexpr int B_BLOCKS = BN * FK / 256;  // blocks of 256 values of B per stage
+    static_assert(BM * FK / 256 == PROD_WARPS && B_BLOCKS <= PROD_WARPS, "one block of each operand per warp");
+    constexpr uint32_t IDESC = instr_desc<BN, false, false, BM>();
+
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t bars[2 * NST + 2 * NBUF + 1];
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_abort;
+    __shared__ int s_tile_start[FMAX_GROUPS + 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    volatile int* abort_flag = &s_abort;
+    const uint32_t raw_u32 = smem_u32(smem_raw);
+    const uint32_t ring = raw_u32 + ((1024u - (raw_u32 & 1023u)) & 1023u);
+    uint8_t* ring_ptr = smem_raw + (ring - raw_u32);
+    const uint32_t bar0 = smem_u32(&bars[0]);
+    auto full_bar = [&](int s) { return bar0 + 8u * s; };
+    auto empty_bar = [&](int s) { return bar0 + 8u * (NST + s); };
+    auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * NST + b); };
+    auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * NST + NBUF + b); };
+    const uint32_t drain_bar = bar0 + 8u * (2 * NST + 2 * NBUF);
+
+    const int F = EPI == EPI_SWIGLU_FWD ? p.N / 2 : p.N;
+    const int tiles_n = EPI == EPI_SWIGLU_FWD ? (F + BN / 2 - 1) / (BN / 2) : (p.N + BN - 1) / BN;
+    auto group_rows = [&](int g) { return p.rows.offsets ? p.rows.offsets[g + 1] - p.rows.offsets[g] : p.rows.rows; };
+    if (warp == 0) {  // tiles before each group
+        int run = 0;
+        for (int g0 = 0; g0 < p.G; g0 += 32) {
+            const int g = g0 + lane;
+            int n = 0;
+            if (g < p.G) n = (VAR_K ? (p.M + BM - 1) / BM : (max(group_rows(g), 0) + BM - 1) / BM) * tiles_n;
+            int inc = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += u;
+            }
+            if (g < p.G) s_tile_start[g] = run + inc - n;
+            run += __shfl_sync(0xffffffffu, inc, 31);
+        }
+        if (lane == 0) s_tile_start[p.G] = run;
+    } else if (warp == MMA_WARP) {
+        if (lane == 0) {
+            s_abort = 0;
+            for (int s = 0; s < NST; ++s) {
+                mbar_init(full_bar(s), PROD_WARPS);
+                mbar_init(empty_bar(s), 1);
+            }
+            for (int b = 0; b < NBUF; ++b) {
+                mbar_init(tfull_bar(b), 1);
+                mbar_init(tempty_bar(b), EPI_W);
+            }
+            mbar_init(drain_bar, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        __syncwarp();
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(NBUF * BN)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem_base = s_tmem;
+    const int total = s_tile_start[p.G];
+
+    // bounded wait of a whole warp (inlined: a call would spill the accumulators around it)
+    auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
+        bool ok = mbar_try(bar, parity);
+        if (!ok) {
+            const uint64_t t0 = gtimer();
+            while (!(ok = mbar_try(bar, parity)) && !*abort_flag) {
+                if (gtimer() - t0 > p.wait_ns) {
+                    *abort_flag = 1;
+                    record_status(MOE_ERR_TIMEOUT);
+                }
+            }
+        }
+        return __all_sync(0xffffffffu, ok);
+    };
+    // M-tiles innermost: the CTAs of a round share the tile columns of B
+    auto tile_at = [&](int t) -> Tile {
+        int lo = 0, hi = p.G - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (s_tile_start[mid] <= t) lo = mid;
+            else hi = mid - 1;
+        }
+        Tile ti;
+        ti.g = lo;
+        ti.we = p.gexp ? p.gexp[lo] : lo;
+        const int local = t - s_tile_start[lo], mt = (s_tile_start[lo + 1] - s_tile_start[lo]) / tiles_n;
+        ti.m0 = (local % mt) * BM;
+        ti.n0 = (local / mt) * (EPI == EPI_SWIGLU_FWD ? BN / 2 : BN);
+        const int rows = group_rows(lo);
+        if (p.rows.offsets) {
+            ti.a0 = ti.b0 = ti.o0 = p.rows.offsets[lo];
+        } else {
+            ti.a0 = (int64_t)lo * p.rows.a_stride;
+            ti.b0 = (int64_t)lo * p.rows.b_stride;
+            ti.o0 = (int64_t)lo * p.rows.out_stride;
+        }
+        ti.mrows = VAR_K ? p.M : rows;
+        ti.klen = VAR_K ? max(rows, 0) : p.K;
+        return ti;
+    };
+    auto a_base = [&](const Tile& ti) { return p.a + ti.a0 * (VAR_K ? p.M : p.K); };
+    auto b_base = [&](const Tile& ti) { return VAR_K ? p.b + ti.b0 * p.N : p.b + (int64_t)ti.we * p.b_group_elems; };
+    // weight row of tile column c (SwiGLU forward: BN / 2 gate features, then their up rows)
+    auto b_row = [&](const Tile& ti, int c) -> int {
+        if (EPI == EPI_SWIGLU_FWD) return c < BN / 2 ? ti.n0 + c : F + ti.n0 + c - BN / 2;
+        return ti.n0 + c;
+    };
+
+    if (warp < PROD_WARPS) {
+        // ------------------------------------------------------------ producers
+        // A warp moves one block of 256 values of each operand per stage, 8 outer x 32 inner
+        // (inner: the dimension that is contiguous in memory, k or the operand rows), with
+        // cp.async into its own part of the fp32 ring, up to NRAW stages ahead, and splits it
+        // when it has landed: lane l then holds 8 consecutive k of one operand row (MN: row
+        // l of 32, else row l / 4 of 8).
+        reg_dec<REG_PROD>();
+        const bool has_b = warp < B_BLOCKS;
+        const uint32_t raw = ring + NST * STAGE + warp * 2048;
+        const uint8_t* raw_ptr = ring_ptr + NST * STAGE + warp * 2048;
+        // the block's first operand row and first k
+        const int arow = A_MN ? 32 * (warp % (BM / 32)) : 8 * warp, ak = A_MN ? 8 * (warp / (BM / 32)) : 0;
+        const int brow = B_MN ? 32 * (warp % (BN / 32)) : 8 * warp, bk = B_MN ? 8 * (warp / (BN / 32)) : 0;
+        const int64_t lda = A_MN ? p.M : p.K, ldb = B_MN ? p.N : p.K;
+        const int per_a = 32 / p.vec_a, per_b = 32 / p.vec_b;  // lanes per contiguous line
+        const int oa = lane / per_a, ia = (lane % per_a) * p.vec_a, ob = lane / per_b, ib = (lane % per_b) * p.vec_b;
+        int t = (int)blockIdx.x - (int)gridDim.x, left = 0;
+        const float *src_a = nullptr, *src_b = nullptr;  // this lane's first element of the block
+        int lim_a = 0, lim_b = 0;  // outer lines with data past the lane's (K-contiguous), or whether the column has any
+        auto seek = [&]() -> bool {  // the next stage: of this tile, or of the next one with work
+            if ((left -= FK) > 0) {
+                src_a += A_MN ? FK * lda : FK;
+                src_b += B_MN ? FK * ldb : FK;
+                return true;
+            }
+            while ((t += gridDim.x) < total) {
+                const Tile ti = tile_at(t);
+                left = ti.klen;
+                if (left <= 0) continue;
+                const int ra = ti.m0 + arow + (A_MN ? ia : oa);
+                lim_a = A_MN ? (ra < ti.mrows ? 1 : 0) : ti.mrows - ra;
+                src_a = a_base(ti) + (A_MN ? (ak + oa) * lda + ra : ra * lda + ia);
+                if (has_b) {
+                    const int c = brow + (B_MN ? ib : ob);
+                    const int rb = b_row(ti, c), end = EPI == EPI_SWIGLU_FWD ? (c < BN / 2 ? F : 2 * F) : p.N;
+                    lim_b = B_MN ? (rb < end ? 1 : 0) : end - rb;
+                    src_b = b_base(ti) + (B_MN ? (bk + ob) * ldb + rb : rb * ldb + ib);
+                }
+                return true;
+            }
+            return false;
+        };
+        // copy one block, W floats a copy: outer lines o0, o0 + 32 / PER, ...
+        auto copy_block = [&](auto mnc, auto wc, const float* src, int64_t ld, int o, int in, int k0, int lim, uint32_t dst) {
+            constexpr bool MN = decltype(mnc)::value;
+            constexpr int W = decltype(wc)::value, STEP = W;  // 32 / (32 / W) lines per copy
+            // K-contiguous lines are swizzled so that the 32-byte reads below spread over the banks
+            dst += o * 128 + in * 4;
+            const int nk = MN ? left - k0 - o : 4 * max(0, min(W, left - in));
+#pragma unroll
+            for (int o0 = 0; o0 < 8; o0 += STEP) {
+                const int n = MN ? (lim && o0 < nk ? 4 * W : 0) : (o0 < lim ? nk : 0);
+                const uint32_t at = dst + o0 * 128;
+                cp_async<W>(MN ? at : at ^ (((o + o0) & 1) << 4), n ? src + o0 * ld : p.a, n);
+            }
+        };
+        auto copy_op = [&](auto mnc, int vec, const float* src, int64_t ld, int o, int in, int k0, int lim, uint32_t dst) {
+            if (vec == 4) copy_block(mnc, std::integral_constant<int, 4>{}, src, ld, o, in, k0, lim, dst);
+            else if (vec == 2) copy_block(mnc, std::integral_constant<int, 2>{}, src, ld, o, in, k0, lim, dst);
+            else copy_block(mnc, std::integral_constant<int, 1>{}, src, ld, o, in, k0, lim, dst);
+        };
+        auto issue = [&](int slot) {
+            const uint32_t dst = raw + slot * raw_bytes();
+            copy_op(std::integral_constant<bool, A_MN>{}, p.vec_a, src_a, lda, oa, ia, ak, lim_a, dst);
+            if (has_b) copy_op(std::integral_constant<bool, B_MN>{}, p.vec_b, src_b, ldb, ob, ib, bk, lim_b, dst + 1024);
+        };
+        // split one landed block into the three planes at d
+        auto split_block = [&](auto mnc, const uint8_t* q, uint8_t* d, uint32_t plane) {
+            float v[8];
+            if constexpr (decltype(mnc)::value) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = *reinterpret_cast<const float*>(q + u * 128 + lane * 4);
+            } else {
+                const uint8_t* ln = q + (lane >> 2) * 128;
+                const int w = (lane & 3) * 32, x = ((lane >> 2) & 1) << 4;
+                Vec<float>::load(reinterpret_cast<const float*>(ln + (w ^ x)), v);
+                Vec<float>::load(reinterpret_cast<const float*>(ln + ((w + 16) ^ x)), v + 4);
+            }
+            uint4 h, m, l;
+            split8(v, &h, &m, &l);
+            *reinterpret_cast<uint4*>(d) = h;
+            *reinterpret_cast<uint4*>(d + plane) = m;
+            *reinterpret_cast<uint4*>(d + 2 * plane) = l;
+        };
+        auto plane_at = [&](int i, int kc) { return i * 64 + ((kc ^ ((i >> 1) & 3)) << 4); };
+        const uint32_t da = plane_at(arow + (A_MN ? lane : lane >> 2), A_MN ? ak >> 3 : lane & 3);
+        const uint32_t db = 3 * plane_a() + plane_at(brow + (B_MN ? lane : lane >> 2), B_MN ? bk >> 3 : lane & 3);
+        bool more = seek();
+        int slot_in = 0, slot = 0, ahead = 0;  // stages copied and not yet split
+        uint32_t phase = 0;
+        int stage = 0;
+        for (;;) {
+            while (more && ahead < NRAW) {
+                issue(slot_in);
+                cp_commit();
+                slot_in = slot_in + 1 == NRAW ? 0 : slot_in + 1;
+                ++ahead;
+                more = seek();
+            }
+            if (!ahead) break;
+            if (ahead == NRAW) cp_wait<NRAW - 1>();
+            else cp_wait<0>();  // the last stages
+            __syncwarp();
+            if (!wait(empty_bar(stage), phase ^ 1u)) break;
+            uint8_t* sa = ring_ptr + (size_t)stage * STAGE;
+            const uint8_t* rp = raw_ptr + slot * raw_bytes();
+            split_block(std::integral_constant<bool, A_MN>{}, rp, sa + da, plane_a());
+            if (has_b) split_block(std::integral_constant<bool, B_MN>{}, rp + 1024, sa + db, plane_b(BN));
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(full_bar(stage));
+            --ahead;
+            slot = slot + 1 == NRAW ? 0 : slot + 1;
+            if (++stage == NST) {
+                stage = 0;
+                phase ^= 1u;
+            }
+        }
+        cp_wait<0>();  // after an abort: copies in flight
+    } else if (warp >= MMA_WARP) {
+        // ------------------------------------------------------------ MMA issuer
+        reg_dec<REG_MMA>();
+        if (warp == MMA_WARP) {
+            int stage = 0, b = 0;
+            uint32_t phase = 0, bphase = 0;
+            bool ok = true, issued = false;
+            for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+                const int kiters = (tile_at(t).klen + FK - 1) / FK;
+                for (int kb = 0; kb < kiters; ++kb) {
+                    ok = wait(tempty_bar(b), bphase ^ 1u) && wait(full_bar(stage), phase);
+                    if (!ok) break;
+                    fence_after();
+                    if (lane == 0) {
+                        const uint32_t sa = ring + stage * STAGE, sb = sa + 3 * plane_a();
+                        constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+    #pragma unroll
+                        for (int q = 0; q < 6; ++q)
+    #pragma unroll
+                            for (int kk = 0; kk < FK / 16; ++kk)
+                                mma_bf16(tmem_base + b * BN, smem_desc_sw64(sa + pa[q] * plane_a() + kk * 32),
+                                         smem_desc_sw64(sb + pb[q] * plane_b(BN) + kk * 32), IDESC, (q | kk) ? 1u : 0u);
+                        mma_commit(empty_bar(stage));
+                        mma_commit(tfull_bar(b));
+                    }
+                    issued = true;
+                    __syncwarp();
+                    if (++stage == NST) {
+                        stage = 0;
+                        phase ^= 1u;
+                    }
+                    if (++b == NBUF) {
+                        b = 0;
+                        bphase ^= 1u;
+                    }
+                }
+            }
+            if ((!ok || *abort_flag) && lane == 0 && issued) {
+                // every MMA issued has completed before TMEM is released
+                mma_commit(drain_bar);
+                const uint64_t limit = p.wait_ns > 200000000ull ? p.wait_ns : 200000000ull, t0 = gtimer();
+                while (!mbar_try(drain_bar, 0) && gtimer() - t0 < limit) {
+                }
+            }
+            __syncwarp();
+        }
+    } else {
+        // ------------------------------------------------------------ accumulate, epilogue
+        reg_inc<REG_EPI>();
+        const int q = warp & 3, hc = (warp - EPI_WARP0) >> 2;  // TMEM lane quarter, column half
+        float* st = reinterpret_cast<float*>(ring_ptr + NST * STAGE + NRAW * raw_bytes()) + (warp - EPI_WARP0) * ST_FLOATS;
+        int b = 0;
+        uint32_t bphase = 0;
+        for (int t = blockIdx.x; t < total; t += gridDim.x) {
+            const Tile ti = tile_at(t);
+            const int kiters = (ti.klen + FK - 1) / FK;
+            float acc[2][CW];
+#pragma unroll
+            for (int c = 0; c < CW; ++c) acc[0][c] = acc[1][c] = 0.f;
+            bool ok = true;
+            for (int kb = 0; kb < kiters; ++kb) {
+                ok = wait(tfull_bar(b), bphase);
+                if (!ok) break;
+                fence_after();
+                const uint32_t tb = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN + hc * CW);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    float v[CW];
+                    if constexpr (CW == 32) tmem_ld32(tb + u * (BN / 2), v);
+                    else tmem_ld16(tb + u * (BN / 2), v);
+#pragma unroll
+                    for (int c = 0; c < CW; ++c) acc[u][c] += v[c];
+                }
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(tempty_bar(b));
+                if (++b == NBUF) {
+                    b = 0;
+                    bphase ^= 1u;
+                }
+            }
+            if (!ok) break;
+            // transpose through shared memory (32 rows x 32 columns at a time): lanes then run
+            // along the columns, so that loads and stores are coalesced
+            auto put = [&](int at, float v) { st[lane * 32 + (at ^ lane)] = v; };
+            auto get = [&](int r, int at) { return st[r * 32 + (at ^ r)]; };
+            auto redo = [&](float v, int m, int n) -> float {
+                if (fabsf(v) <= 3.402823466e38f) return v;
+                const float* A = a_base(ti) + (A_MN ? (int64_t)m : (int64_t)m * p.K);
+                const float* B = b_base(ti) + (B_MN ? (int64_t)n : (int64_t)n * p.K);
+                return dot_plain(A, A_MN ? p.M : 1, B, B_MN ? p.N : 1, ti.klen);
+            };
+            const int mrow = ti.m0 + q * 32;
+            if constexpr (EPI == EPI_SWIGLU_FWD) {
+                // 16 gate columns beside the 16 up columns of the same features; a half-warp per row
+#pragma unroll
+                for (int c0 = 0; c0 < CW; c0 += 16) {
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        put(i, acc[0][c0 + i]);
+                        put(16 + i, acc[1][c0 + i]);
+                    }
+                    __syncwarp();
+                    const int c = lane & 15, f = ti.n0 + hc * CW + c0 + c;
+#pragma unroll 4
+                    for (int i = 0; i < 16; ++i) {
+                        const int r = 2 * i + (lane >> 4), m = mrow + r;
+                        if (f >= F || m >= ti.mrows) continue;
+                        const float G = redo(get(r, c), m, f), U = redo(get(r, 16 + c), m, F + f);
+                        const int64_t row = ti.o0 + m;
+                        p.out0[row * 2 * F + f] = G;
+                        p.out0[row * 2 * F + F + f] = U;
+                        p.out1[row * F + f] = G * sigmoidf_(G) * U;
+                    }
+                }
+            } else {
+                // 32 columns at a time: one half's (CW = 32), or both halves' (CW = 16)
+#pragma unroll
+                for (int u = 0; u < CW / 16; ++u) {
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) put(i, CW == 32 ? acc[u][i % CW] : acc[i / CW][i % CW]);
+                    __syncwarp();
+                    const int n = ti.n0 + hc * CW + (CW == 32 ? u * (BN / 2) + lane : (lane >> 4) * (BN / 2) + (lane & 15));
+#pragma unroll 4
+                    for (int r = 0; r < 32; ++r) {
+                        const int m = mrow + r;
+                        if (n >= p.N || m >= ti.mrows) continue;
+                        const float v = redo(get(r, lane), m, n);
+                        if constexpr (EPI == EPI_SWIGLU_BWD) {  // v = dA[row, n], N = F
+                            const int64_t row = (ti.o0 + m) * 2 * F;
+                            const float G = p.aux[row + n], U = p.aux[row + F + n];
+                            const float s = sigmoidf_(G);
+                            p.out0[row + F + n] = v * G * s;
+                            p.out0[row + n] = v * U * s * (1.f + G * (1.f - s));
+                        } else {
+                            const int64_t row = VAR_K ? (int64_t)ti.we * p.M + m : ti.o0 + m;
+                            p.out0[row * p.N + n] = v;
+                        }
+                    }
+                }
+            }
+        }
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (warp == MMA_WARP)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(NBUF * BN)
+                     : "memory");
+}
+
+// ------------------------------------------------------------------------ host side
+static int sm_count() {
+    static int n = 0;
+    if (!n) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        if (n <= 0) n = 148;
+    }
+    return n;
+}
+
+// floats per copy that the lines of an operand allow: their length, the distance of its
+// groups and its address are multiples of it
+static int vec_of(const void* base, int64_t ld, int64_t group = 0) {
+    for (int w = 4; w > 1; w /= 2)
+        if (ld % w == 0 && group % w == 0 && (uintptr_t)base % (4 * w) == 0) return w;
+    return 1;
+}
+
+template <bool A_MN, bool B_MN, bool VAR_K, int EPI, int BN>
+static cudaError_t launch_bn(const Params& p, int64_t tiles, cudaStream_t s) {
+    auto kern = gemm_f32_kernel<A_MN, B_MN, VAR_K, EPI, BN>;
+    constexpr size_t smem = smem_bytes(BN);
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        // the roles' register shares must not exceed the launch's (setmaxnreg would wait forever)
+        cudaFuncAttributes fa;
+        if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
+        if (fa.numRegs * NTHREADS < 32 * (PROD_WARPS * REG_PROD + EPI_W * REG_EPI + 4 * REG_MMA))
+            return cudaErrorInvalidConfiguration;
+        attr = true;
+    }
+    const unsigned grid = (unsigned)std::min<int64_t>(tiles, sm_count());
+    (void)launch_pdl(kern, dim3(grid), dim3(NTHREADS), smem, s, p);
+    return cudaGetLastError();
+}
+
+template <bool A_MN, bool B_MN, bool VAR_K, int EPI>
+static cudaError_t launch(const Params& p, int64_t mt, cudaStream_t s) {
+    const int cols = EPI == EPI_SWIGLU_FWD ? p.N / 2 : p.N, per = EPI == EPI_SWIGLU_FWD ? 2 : 1;
+    const int64_t wide = mt * ((cols + 128 / per - 1) / (128 / per));
+    if (wide <= 0) return cudaSuccess;
+    // 128-wide tiles once they fill the SMs; under that, twice as many 64-wide ones
+    if (wide >= sm_count()) return launch_bn<A_MN, B_MN, VAR_K, EPI, 128>(p, wide, s);
+    return launch_bn<A_MN, B_MN, VAR_K, EPI, 64>(p, mt * ((cols + 64 / per - 1) / (64 / per)), s);
+}
+
+}  // namespace f32
+
+cudaError_t launch_gemm_m_f32(const GemmMArgs& g, cudaStream_t s) {
+    using namespace f32;
+    if (g.G > FMAX_GROUPS) return cudaErrorInvalidValue;
+    Params p{};
+    p.rows = g.rows;
+    p.G = g.G;
+    p.gexp = g.group_expert;
+    p.a = (const float*)g.a;
+    p.b = (const float*)g.b;
+    p.b_group_elems = g.b_group_elems;
+    p.N = g.N;
+    p.K = g.K;
+    p.out0 = (float*)g.out0;
+    p.out1 = (float*)g.out1;
+    p.aux = (const float*)g.aux;
+    p.wait_ns = wait_limit_ns();
+    p.vec_a = vec_of(g.a, g.K);
+    p.vec_b = vec_of(g.b, g.b_kmajor ? g.K : g.N, g.b_group_elems);
+    // upper bound of the M-tiles: OFFSETS groups may each end in a partial one
+    const int64_t mt = g.rows.offsets ? ((int64_t)g.rows.rows + BM - 1) / BM + g.G
+                                      : (int64_t)g.G * ((g.rows.rows + BM - 1) / BM);
+    if (g.epi == EPI_SWIGLU_FWD) return launch<false, false, false, EPI_SWIGLU_FWD>(p, mt, s);
+    if (g.epi == EPI_SWIGLU_BWD) return launch<false, true, false, EPI_SWIGLU_BWD>(p, mt, s);
+    if (g.b_kmajor) return launch<false, false, false, EPI_STORE>(p, mt, s);
+    return launch<false, true, false, EPI_STORE>(p, mt, s);
+}
+
+cudaError_t launch_gemm_k_f32(const GemmKArgs& g, cudaStream_t s) {
+    using namespace f32;
+    if (g.G > FMAX_GROUPS) return cudaErrorInvalidValue;
+    Params p{};
+    p.rows = g.rows;
+    p.G = g.G;
+    p.gexp = g.group_expert;
+    p.a = (const float*)g.a;
+    p.b = (const float*)g.b;
+    p.M = g.M;
+    p.N = g.N;
+    p.out0 = (float*)g.out;
+    p.wait_ns = wait_limit_ns();
+    p.vec_a = vec_of(g.a, g.M);
+    p.vec_b = vec_of(g.b, g.N);
+    return launch<true, true, true, EPI_STORE>(p, (int64_t)g.G * ((g.M + BM - 1) / BM), s);
+}
+
+cudaError_t f32_status(cudaStream_t s, int* code) { return tu_status_read_clear(s, code); }
+
+}  // namespace moe

@@ -11,17 +11,14 @@
 // the fused epilogue. Every mbarrier wait is bounded in time; on a timeout the CTA
 // records MOE_ERR_TIMEOUT, drains its in-flight copies and MMAs, frees TMEM and
 // returns.
-#include <cuda.h>
-
 #include <algorithm>
 
-#include "moe_common.cuh"
 #include "moe_internal.h"
+#include "tc_ptx.cuh"
 
 namespace moe {
 namespace tc {
 
-constexpr int BM = 128;
 constexpr int BK = 64;  // 64 bf16 = 128 bytes = one 128B-swizzle row
 // Contraction rows per k-block: BK, except for CTA-pair K-variable tiles (weight
 // gradients), whose operands are both MN-major (64-element TMA boxes): 128-row boxes
@@ -78,249 +75,6 @@ struct Params {
     // short batch spread over every SM (each CTA streams its rows at a per-CTA rate)
     int tile_rows;
 };
-
-// ------------------------------------------------------------------------ PTX helpers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ uint64_t gtimer() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// One poll: the thread sleeps until the phase completes or at most ~20 us have passed.
-constexpr uint32_t kSuspendHintNs = 20000;
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(kSuspendHintNs)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait. Returns false when the CTA is aborting (another role gave up) or when
-// this wait ran past `limit_ns` (then it raises the abort flag and records TIMEOUT).
-__device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                       uint64_t limit_ns) {
-    if (mbar_try(bar, parity)) return true;
-    const uint64_t t0 = gtimer();
-    for (;;) {
-        if (mbar_try(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if (gtimer() - t0 > limit_ns) {
-            *abort_flag = 1;
-            record_status(MOE_ERR_TIMEOUT);
-            return false;
-        }
-    }
-}
-// --- CTA-pair (cta_group::2) helpers
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// shared::cluster address of the same shared-memory offset in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(kSuspendHintNs)
-        : "memory");
-    return ok != 0;
-}
-// TMA load into this CTA's shared memory whose completion is counted on a barrier
-// that may live in the peer CTA of the pair (the leader's "full" barrier)
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map,
-                                                 uint32_t cluster_bar, int c0, int c1) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
-        "[%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
-        "l"((uint64_t)map), "r"(cluster_bar), "r"(c0), "r"(c1)
-        : "memory");
-}
-__device__ __forceinline__ void mma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
-                                              uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// commit the pair's MMAs to the barrier at this offset in every CTA of `mask`
-__device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint16_t mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 "
-        "[%0], %1;" ::"r"(bar),
-        "h"(mask)
-        : "memory");
-}
-// credit `bytes` of expected transactions to a barrier in another CTA of the cluster, as
-// if that many bytes had arrived there (no arrival)
-__device__ __forceinline__ void mbar_complete_tx_remote(uint32_t cluster_bar, uint32_t bytes) {
-    asm volatile("mbarrier.complete_tx.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(cluster_bar), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
-                     : "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
-                                            int c0, int c1) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-        "[%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
-        "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1)
-        : "memory");
-}
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int c0, int c1) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
-                     (uint64_t)map),
-                 "r"(src), "r"(c0), "r"(c1)
-                 : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read0() {
-    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-// wait until at most N of this thread's bulk groups are still reading shared memory
-template <int N>
-__device__ __forceinline__ void bulk_wait_read() {
-    asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ void bulk_wait0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void fence_proxy_async() {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-// 32 fp32 values -> 32 bf16 (64 bytes) at dst (16-byte aligned; shared or global)
-__device__ __forceinline__ void store_row32(__nv_bfloat16* dst, const float* v) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) Vec<__nv_bfloat16>::store(dst + 8 * i, v + 8 * i);
-}
-
-// One 64-byte row (32 bf16) of a staging box in the 64B-swizzled layout the TMA store
-// map uses: 16-byte chunk c of row r sits at chunk c ^ ((r >> 1) & 3).
-__device__ __forceinline__ void store_row32_sw64(uint8_t* row_base, int r, const float* v) {
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-        Vec<__nv_bfloat16>::store(reinterpret_cast<__nv_bfloat16*>(row_base + ((c ^ ((r >> 1) & 3)) << 4)),
-                                  v + 8 * c);
-}
-
-__device__ __forceinline__ void fence_before() {
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void fence_after() {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-        : "memory");
-}
-// 32 lanes x 32 consecutive fp32 columns of the accumulator
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-          "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
-          "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
-          "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// 32 lanes x 16 consecutive fp32 columns of the accumulator
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-          "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-// 16-byte read-only load (the buffer is not written while the kernel runs)
-__device__ __forceinline__ uint4 ldg_nc(const __nv_bfloat16* ptr) {
-    uint4 r;
-    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
-                 : "l"(ptr));
-    return r;
-}
-__device__ __forceinline__ void unpack8(uint4 u, float* v) {
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float2 f = __bfloat1622float2(h[i]);
-        v[2 * i] = f.x;
-        v[2 * i + 1] = f.y;
-    }
-}
-
-// Shared-memory matrix descriptor, 128B swizzle, sm_100 family layout:
-// start>>4 [0,14), LBO>>4 [16,30), SBO>>4 [32,46), version 1 [46,48), swizzle 2 [61,64).
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-// Instruction descriptor of kind::f16: fp32 D [4,6), bf16 A [7,10), bf16 B [10,13),
-// A major [15], B major [16] (1 = MN-major), N>>3 [17,23), M>>4 [24,29).
-template <int BN, bool A_MN, bool B_MN, int M = BM>
-__host__ __device__ constexpr uint32_t instr_desc() {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((A_MN ? 1u : 0u) << 15) |
-           ((B_MN ? 1u : 0u) << 16) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
 
 // Pipeline depth: as many operand stages as fit beside the epilogue's shared memory
 // (staging boxes, or the router's histogram), at most 12. OCC CTAs share one SM (OCC = 2:
@@ -1450,6 +1204,7 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
 }  // namespace tc
 
 void set_wait_limit_ns(uint64_t ns) { tc::g_wait_ns = ns ? ns : 1; }
+uint64_t wait_limit_ns() { return tc::g_wait_ns; }
 void set_gemm_pairs(int mode) { tc::g_pairs = mode; }
 
 // Pair tiles where they fill at least four rounds of the SMs (the last, partly empty
@@ -1487,7 +1242,7 @@ bool gemm_k_uses_pairs(const GemmKArgs& g) {
 
 // M-variable grouped GEMM (forward, dA, dX).
 cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s) {
-    if (!bf16) return launch_gemm_m_simt(g, s);
+    if (!bf16) return launch_gemm_m_f32(g, s);
     using namespace tc;
     if (g.G > MAX_GROUPS) return cudaErrorInvalidValue;
     Params p{};
@@ -1566,7 +1321,7 @@ cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s) {
 
 // K-variable grouped GEMM (dW1, dW2).
 cudaError_t launch_gemm_k(const GemmKArgs& g, bool bf16, cudaStream_t s) {
-    if (!bf16) return launch_gemm_k_simt(g, s);
+    if (!bf16) return launch_gemm_k_f32(g, s);
     using namespace tc;
     if (g.G > MAX_GROUPS) return cudaErrorInvalidValue;
     Params p{};

@@ -541,7 +541,7 @@ moe_status moe_expert_ffn_bwd(const moe_config* cfg, const void* x_perm, const i
     // Each M-variable GEMM runs with its weight gradient in one persistent launch (one
     // tail instead of two, and no two persistent grids contending for SMs): dA then dW2
     // (which needs only dY and A), dX then dW1 (which needs dH). A GEMM that runs as
-    // CTA-pair tiles, and the CUDA-core path, instead put the weight gradient on a side
+    // CTA-pair tiles, and the fp32 path, instead put the weight gradient on a side
     // stream: dW2 alongside dA, dW1 alongside dX once dH exists.
     const bool fuse_a = bf16 && !gemm_m_uses_pairs(a);
     const bool fuse_b = bf16 && !gemm_m_uses_pairs(b);  // the same rule as moe_expert_ffn_bwd_kernels
@@ -768,7 +768,7 @@ moe_status moe_device_status(moe_stream_t stream, int32_t* code) {
     if ((e = route_status(s, &c[0])) != cudaSuccess) return cuda_status(e, "status");
     if ((e = dispatch_status(s, &c[1])) != cudaSuccess) return cuda_status(e, "status");
     if ((e = gemm_status(s, &c[2])) != cudaSuccess) return cuda_status(e, "status");
-    if ((e = simt_status(s, &c[3])) != cudaSuccess) return cuda_status(e, "status");
+    if ((e = f32_status(s, &c[3])) != cudaSuccess) return cuda_status(e, "status");
     *code = 0;
     for (int i = 0; i < 4; ++i)
         if (c[i] && !*code) *code = c[i];

@@ -150,11 +150,12 @@ bool gemm_k_uses_pairs(const GemmKArgs& g);
 void set_wait_limit_ns(uint64_t ns);
 void set_gemm_pairs(int mode);  // MOE_PAIRS_*
 cudaError_t gemm_status(cudaStream_t s, int* code);
-cudaError_t simt_status(cudaStream_t s, int* code);
+cudaError_t f32_status(cudaStream_t s, int* code);
 
-// fp32 SIMT versions (the fp32 configuration); same argument meaning.
-cudaError_t launch_gemm_m_simt(const GemmMArgs& g, cudaStream_t s);
-cudaError_t launch_gemm_k_simt(const GemmKArgs& g, cudaStream_t s);
+// the fp32 configuration (gemm_f32.cu); same argument meaning
+cudaError_t launch_gemm_m_f32(const GemmMArgs& g, cudaStream_t s);
+cudaError_t launch_gemm_k_f32(const GemmKArgs& g, cudaStream_t s);
+uint64_t wait_limit_ns();
 
 // training step around the layer (train.cu)
 cudaError_t launch_sgd_update(void* w, const void* dw, float* master, int64_t n_groups, int64_t group_elems,

@@ -582,10 +582,9 @@ static cudaError_t launch_route_t(const RouteArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// E > 64 on the CUDA cores (fp32): the router's products x W_r[p]^T by the grouped SIMT
-// GEMM into `logits` (groups = parties), then the gating pass reads them back, adds the
+// E > 64, fp32: the router's products x W_r[p]^T by the grouped fp32 GEMM into `logits` (groups = parties), then the gating pass reads them back, adds the
 // bias and overwrites them with the biased logits.
-static cudaError_t launch_route_wide_simt(const RouteArgs& a, cudaStream_t s) {
+static cudaError_t launch_route_wide_f32(const RouteArgs& a, cudaStream_t s) {
     GemmMArgs m{};
     m.G = (a.po && a.P > 1) ? a.P : 1;
     m.rows = (a.po && a.P > 1) ? GroupRows{a.po, (int)a.T, 0, 0, 0} : GroupRows{nullptr, (int)a.T, 0, 0, 0};
@@ -597,7 +596,7 @@ static cudaError_t launch_route_wide_simt(const RouteArgs& a, cudaStream_t s) {
     m.K = a.d;
     m.epi = EPI_STORE;
     m.out0 = a.logits;
-    cudaError_t e = launch_gemm_m_simt(m, s);
+    cudaError_t e = launch_gemm_m_f32(m, s);
     if (e != cudaSuccess) return e;
     RouteArgs b = a;
     b.logits_in = a.logits;
@@ -613,7 +612,7 @@ cudaError_t launch_route(const RouteArgs& a, bool bf16, bool from_logits, cudaSt
         return launch_route_t<float, true>(b, s);
     }
     if (bf16 && (a.E % 4 == 0 || a.E > 64) && a.T > 0) return launch_route_tc(a, s);
-    if (a.E > 64) return a.T > 0 ? launch_route_wide_simt(a, s) : cudaSuccess;
+    if (a.E > 64) return a.T > 0 ? launch_route_wide_f32(a, s) : cudaSuccess;
     return bf16 ? launch_route_t<__nv_bfloat16, false>(a, s) : launch_route_t<float, false>(a, s);
 }
 
@@ -674,7 +673,7 @@ static cudaError_t launch_dlogits(const RouteBwdArgs& a, __nv_bfloat16* dz16, in
     return cudaGetLastError();
 }
 
-// fp32: dlogits, CUDA-core partials and reduce, dx_router on the CUDA-core GEMM
+// fp32: dlogits, CUDA-core partials and reduce, dx_router on the fp32 GEMM
 static cudaError_t launch_route_bwd_simt(const RouteBwdArgs& a, void* ws, cudaStream_t s) {
     using T = float;
     const int64_t nch = (a.T + RB_CH - 1) / RB_CH + a.P;
@@ -715,7 +714,7 @@ static cudaError_t launch_route_bwd_simt(const RouteBwdArgs& a, void* ws, cudaSt
         m.K = a.E;
         m.epi = EPI_STORE;
         m.out0 = a.dx_router;
-        return launch_gemm_m_simt(m, s);
+        return launch_gemm_m_f32(m, s);
     }
     return cudaSuccess;
 }

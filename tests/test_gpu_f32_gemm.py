@@ -1,0 +1,94 @@
+"""The fp32 grouped GEMMs (three-way bf16 split on the tensor cores) at the edges of their
+tiles and copies: contractions around the 32-term stage, lines
+of 4-, 8- and 16-byte alignment, row counts around the 128-row tile, empty experts, one and
+several tiles per CTA; and infinities, NaN and the largest finite values.
+
+Bound per element of a contraction c = sum a_i b_i: the split leaves out terms below
+3 * 2^-25 |a_i b_i|; each of the 12 accumulation steps per 32 terms and each register
+addition rounds a partial sum no larger than S = sum |a_i b_i| by at most 2^-23 (truncation),
+so |err| <= (12 + K / 32 + 3) * 2^-23 S is a safe worst case."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import moe_oracle as mo
+from synth import moe_inputs as mi
+from tests.gpu_util import cfg_of, dev, empty, need_gpu, status
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    return need_gpu()
+
+
+def close(name, got, ref, mag, K):
+    err = np.abs(got.double().cpu().numpy() - ref)
+    bound = (16 + K / 32) * 2.0 ** -23 * mag + 1e-38
+    assert (err <= bound).all(), (name, float((err / bound).max()))
+
+
+def run(L, rows, d, F, seed, x=None):
+    """fwd + bwd of experts with the given row counts; returns buffers and inputs."""
+    E, TK = len(rows), int(sum(rows))
+    off = np.concatenate([[0], np.cumsum(rows)]).astype(np.int32)
+    rng = np.random.default_rng(seed)
+    f = lambda *s: rng.standard_normal(s).astype(np.float32)  # noqa: E731
+    x = f(TK, d) if x is None else x
+    w1, w2, dy = f(E, 2 * F, d) * np.float32(0.1), f(E, d, F) * np.float32(0.1), f(TK, d)
+    sh = mi.MoEShape("f", TK, d, E, F, 1, "f32")
+    g = {n: empty(s, torch.float32) for n, s in dict(h=(TK, 2 * F), a=(TK, F), y=(TK, d), dh=(TK, 2 * F), dx=(TK, d),
+                                                     dw1=(E, 2 * F, d), dw2=(E, d, F)).items()}
+    t = {n: dev(v, torch.float32) for n, v in dict(x=x, w1=w1, w2=w2, dy=dy).items()}
+    offd = dev(off, torch.int32)
+    L.moe_expert_ffn_fwd(cfg_of(L, sh), t["x"], offd, t["w1"], t["w2"], g["h"], g["a"], g["y"])
+    L.moe_expert_ffn_bwd(cfg_of(L, sh), t["x"], offd, t["w1"], t["w2"], g["h"], g["a"], t["dy"], g["dh"], g["dx"],
+                         g["dw1"], g["dw2"])
+    assert status(L) == 0
+    return g, off, x, w1, w2, dy
+
+
+@pytest.mark.parametrize("rows,d,F", [
+    ((1, 0, 127, 128, 129), 32, 33),       # 4-byte lines (F odd), one stage, tile edges, an empty expert
+    ((31, 32, 33, 63, 64, 65), 64, 62),    # 8-byte lines; weight gradients ending around a stage
+    ((5,), 28, 1),                          # less than one stage, one feature
+    ((300, 2, 700), 132, 100),              # 16-byte lines, 4 past a stage
+    ((2000, 900), 516, 388),                # 128-wide tiles, several per CTA
+])
+def test_contractions_at_the_edges(L, rows, d, F):
+    g, off, x, w1, w2, dy = run(L, rows, d, F, seed=d + F)
+    x, w1, w2, dy = (v.astype(np.float64) for v in (x, w1, w2, dy))
+    h, a, dh = (g[n].double().cpu().numpy() for n in ("h", "a", "dh"))
+    for e in range(len(rows)):
+        r = slice(off[e], off[e + 1])
+        close("h", g["h"][r], x[r] @ w1[e].T, np.abs(x[r]) @ np.abs(w1[e]).T, d)
+        close("y", g["y"][r], a[r] @ w2[e].T, np.abs(a[r]) @ np.abs(w2[e]).T, F)
+        close("dx", g["dx"][r], dh[r] @ w1[e], np.abs(dh[r]) @ np.abs(w1[e]), 2 * F)
+        close("dw1", g["dw1"][e], dh[r].T @ x[r], np.abs(dh[r]).T @ np.abs(x[r]), rows[e])
+        close("dw2", g["dw2"][e], dy[r].T @ a[r], np.abs(dy[r]).T @ np.abs(a[r]), rows[e])
+        G, U = h[r, :F], h[r, F:]
+        s = mo.sigmoid(G)
+        dA, mag = dy[r] @ w2[e], np.abs(dy[r]) @ np.abs(w2[e])
+        close("dG", g["dh"][r, :F], dA * U * s * (1 + G * (1 - s)), mag * np.abs(U) * (1 + np.abs(G)), d)
+        close("dU", g["dh"][r, F:], dA * G * s, mag * np.abs(G), d)
+
+
+def test_non_finite_values_follow_ieee(L):
+    """A row of x holding an infinity, a NaN or the largest finite value gives what an fp32
+    FMA chain gives there, and leaves the other rows alone."""
+    rng = np.random.default_rng(3)
+    rows, d, F = (40, 90), 96, 70
+    x = rng.standard_normal((130, d)).astype(np.float32)
+    clean = run(L, rows, d, F, seed=9, x=x.copy())[0]["h"].cpu()
+    big = np.float32(3.4028235e38)
+    x[3, 5], x[50, 7], x[51, 40], x[129, 95] = np.inf, -np.inf, np.nan, -big
+    g, off, _, w1, _, _ = run(L, rows, d, F, seed=9, x=x)
+    h = g["h"].cpu()
+    assert torch.isinf(h[3]).all() and (torch.sign(h[3]) == torch.sign(torch.from_numpy(w1[0][:, 5]))).all()
+    assert torch.isinf(h[50]).all() and (torch.sign(h[50]) == -torch.sign(torch.from_numpy(w1[1][:, 7]))).all()
+    assert torch.isnan(h[51]).all()
+    want = -big.astype(np.float64) * w1[1][:, 95].astype(np.float64)
+    assert np.allclose(h[129].double().numpy(), want, rtol=1e-6, atol=0)
+    rest = [i for i in range(130) if i not in (3, 50, 51, 129)]
+    assert torch.equal(h[rest], clean[rest])
