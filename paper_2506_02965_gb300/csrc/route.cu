@@ -1,5 +1,5 @@
 // Gating function of the MoE layer (Alg. 7) and its backward, plus the per-party
-// load-balancing loss. Memory-bound SIMT kernels: x is read once with 16-byte
+// load-balancing loss. SIMT kernels: x is read once with 16-byte
 // vector loads, logits are reduced with warp shuffles, top-k is a warp argmax.
 #include <cfloat>
 
@@ -99,21 +99,156 @@ __device__ void softmax_topk_token(const float (&z)[NV], int lane, int E, int k,
 }
 
 // ----------------------------------------------------------------------------- router fwd
-// One warp handles a group of up to TPW consecutive tokens of one party. Lane l
-// accumulates the dot products of its 16-byte column chunks for every expert, then
-// the partial sums are combined with a butterfly (identical bits on every lane).
-// FROM_LOGITS: the logits come from logits_in instead ([T,E] fp32); with a bias they
-// are the router's raw products (E > 64, computed by a GEMM): the bias is added here
-// and the biased logits are written back to `logits` (which may be logits_in).
-// The per-(party, expert) counts go through a shared-memory histogram when P E fits
-// (HIST_SMEM), else straight to the global counts.
-constexpr int HIST_SMEM = 4096;
-template <typename T, int EMAX, int TPW, bool FROM_LOGITS>
-__global__ void __launch_bounds__(256) route_kernel(
+// Router logits and gating on the CUDA cores: the fp32 configuration, and bf16 pools whose
+// size is not a multiple of 4 (up to 64 experts). One CTA takes TB consecutive tokens of
+// one party and all experts (padded to EP): chunks of RD_KC columns of x and W_r are staged
+// in shared memory as fp32 (the next chunk's global loads are in flight meanwhile), and
+// thread (ks, tg, eg) multiplies TB/4 tokens by 4 experts over the columns of its slice ks.
+// A chunk's products are summed on their own before they join the running sum, so no chain
+// of additions is longer than about d / 128 + 32. The KS slices of a logit are then added
+// through shared memory and each warp gates its tokens.
+//
+// What bounds it: with large pools the shared-memory reads (12 wavefronts per 64 FMAs of a
+// warp), with small ones the latency of the d / 128 chunk steps. The kernel that it replaces
+// (a warp per 1 to 8 tokens, W_r read from L2 by every warp) took 588 us for 3805 bf16 tokens
+// of d = 3072 with E = 63, now 108; 93 -> 27 us for 2157 of 3072 with E = 6; 51 -> 13.6 us for
+// 1003 of 1152 with E = 13; fp32: 19 -> 4.8 us for 512 of 256 with E = 8.
+constexpr int RD_KC = 128;         // columns per chunk
+constexpr int RD_LD = RD_KC + 4;   // row pitch in shared memory: rows start 16 bytes apart in the banks
+constexpr int RD_THREADS = 256;
+
+template <typename T, int EP, int TB>
+__global__ void __launch_bounds__(RD_THREADS, 2) route_dot_kernel(
     const T* __restrict__ x, const T* __restrict__ wr, const float* __restrict__ bias,
-    const float* logits_in, const int32_t* __restrict__ po, int P, int64_t Tn,
-    int d, int E, int k, int normalize, float* logits, float* probs, int32_t* topk_idx,
-    float* topk_w, int32_t* counts) {
+    const int32_t* __restrict__ po, int P, int64_t Tn, int d, int E, int k, int normalize, float* logits,
+    float* probs, int32_t* topk_idx, float* topk_w, int32_t* counts) {
+    pdl_begin();
+    constexpr int NV = (EP + 31) / 32, VN = Vec<T>::N;
+    constexpr int EG = EP / 4, TM = TB / 4, KS = RD_THREADS / EP;  // 4 EG tiles of TM x 4, KS slices
+    constexpr int ROWV = RD_KC / VN;                               // vectors per staged row
+    constexpr int XV = (TB * ROWV + RD_THREADS - 1) / RD_THREADS, WV = (EP * ROWV + RD_THREADS - 1) / RD_THREADS;
+    extern __shared__ float s_dyn[];  // two buffers of [TB + EP][RD_LD]; then the slices' sums
+    __shared__ int s_hist[EP];
+    const int tid = threadIdx.x;
+    // the CTA's tokens: group blockIdx.x of TB tokens, enumerated party by party
+    int party = -1, n = 0;
+    int64_t t0 = 0, g = blockIdx.x;
+    for (int q = 0; q < P && party < 0; ++q) {
+        const int64_t a = po ? po[q] : 0, b = po ? po[q + 1] : Tn;
+        const int64_t ng = b > a ? (b - a + TB - 1) / TB : 0;
+        if (g < ng) {
+            party = q;
+            t0 = a + g * TB;
+            n = (int)min64(TB, b - t0);
+        }
+        g -= ng;
+    }
+    if (party < 0) return;
+    if (tid < EP) s_hist[tid] = 0;
+    const T* W = wr + (int64_t)party * E * d;
+    uint4 xr[XV], wv[WV];
+    auto fetch = [&](int c0) {
+#pragma unroll
+        for (int i = 0; i < XV; ++i) {
+            const int v = tid + i * RD_THREADS, r = v / ROWV, c = c0 + (v % ROWV) * VN;
+            xr[i] = r < n && c < d ? Vec<T>::raw_load(x + (t0 + r) * d + c) : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int i = 0; i < WV; ++i) {
+            const int v = tid + i * RD_THREADS, r = v / ROWV, c = c0 + (v % ROWV) * VN;
+            wv[i] = r < E && c < d ? Vec<T>::raw_load(W + (int64_t)r * d + c) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    auto put = [&](float* buf) {
+#pragma unroll
+        for (int i = 0; i < XV + WV; ++i) {
+            const int v = tid + (i < XV ? i : i - XV) * RD_THREADS, r = v / ROWV;
+            if (r >= (i < XV ? TB : EP)) continue;
+            float f[VN];
+            unpack_vec<T>(i < XV ? xr[i < XV ? i : 0] : wv[i < XV ? 0 : i - XV], f);
+            float* dst = buf + ((i < XV ? 0 : TB) + r) * RD_LD + (v % ROWV) * VN;
+#pragma unroll
+            for (int h = 0; h < VN; h += 4) Vec<float>::store(dst + h, f + h);
+        }
+    };
+    const int eg = tid % EG, tg = (tid / EG) % 4, ks = tid / (4 * EG);
+    float acc[TM][4];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    fetch(0);
+    put(s_dyn);
+    __syncthreads();
+    int cur = 0;
+    for (int c0 = 0; c0 < d; c0 += RD_KC) {
+        const bool more = c0 + RD_KC < d;
+        if (more) fetch(c0 + RD_KC);
+        const float* xs = s_dyn + cur * (TB + EP) * RD_LD + tg * RD_LD;
+        const float* ws = s_dyn + cur * (TB + EP) * RD_LD + (TB + eg) * RD_LD;
+        float part[TM][4];
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) part[i][j] = 0.f;
+#pragma unroll 2
+        for (int q = ks; q < RD_KC / 4; q += KS) {
+            float xv[TM][4], wq[4][4];
+#pragma unroll
+            for (int i = 0; i < TM; ++i) Vec<float>::load(xs + 4 * i * RD_LD + 4 * q, xv[i]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) Vec<float>::load(ws + EG * j * RD_LD + 4 * q, wq[j]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int i = 0; i < TM; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) part[i][j] = fmaf(xv[i][u], wq[j][u], part[i][j]);
+        }
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] += part[i][j];
+        if (more) put(s_dyn + (cur ^ 1) * (TB + EP) * RD_LD);
+        __syncthreads();
+        cur ^= 1;
+    }
+    // [KS][TB][EP] slice sums (token tg + 4 i, expert eg + EG j)
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s_dyn[(ks * TB + tg + 4 * i) * EP + eg + EG * j] = acc[i][j];
+    __syncthreads();
+    const int lane = tid & 31;
+    for (int tt = tid >> 5; tt < n; tt += RD_THREADS / 32) {
+        float z[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int e = lane + 32 * v;
+            float s4[4] = {0.f, 0.f, 0.f, 0.f};
+            if (e < E) {
+#pragma unroll
+                for (int q = 0; q < KS; ++q) s4[q & 3] += s_dyn[(q * TB + tt) * EP + e];
+            }
+            z[v] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+            if (bias && e < E) z[v] += bias[party * E + e];
+        }
+        softmax_topk_token<NV>(z, lane, E, k, normalize, t0 + tt, 0, logits, probs, topk_idx, topk_w, s_hist);
+    }
+    __syncthreads();
+    if (tid < E && s_hist[tid]) atomicAdd(&counts[party * E + tid], s_hist[tid]);
+}
+
+// Gating alone, on logits that exist ([T,E] fp32), one warp per group of up to TPW
+// consecutive tokens of one party. With a bias they are the router's raw products (E > 64,
+// computed by a GEMM): the bias is added here and the biased logits are written back to
+// `logits` (which may be logits_in). The per-(party, expert) counts go through a
+// shared-memory histogram when P E fits (HIST_SMEM), else straight to the global counts.
+constexpr int HIST_SMEM = 4096;
+template <int EMAX, int TPW>
+__global__ void __launch_bounds__(256) route_kernel(
+    const float* __restrict__ bias, const float* logits_in, const int32_t* __restrict__ po, int P, int64_t Tn,
+    int E, int k, int normalize, float* logits, float* probs, int32_t* topk_idx, float* topk_w, int32_t* counts) {
     pdl_begin();
     constexpr int NV = (EMAX + 31) / 32;
     extern __shared__ int s_hist_dyn[];  // [P*E] when it fits
@@ -123,11 +258,8 @@ __global__ void __launch_bounds__(256) route_kernel(
         for (int i = threadIdx.x; i < P * E; i += blockDim.x) s_hist[i] = 0;
     }
     __syncthreads();
-    using V = Vec<T>;
-    constexpr int VN = V::N;
     const int lane = threadIdx.x & 31;
     const int warps_total = gridDim.x * (blockDim.x >> 5);
-    const int64_t nvec = d / VN;
     // groups are enumerated party by party
     int64_t total_groups = 0;
     for (int p = 0; p < P; ++p) {
@@ -146,68 +278,19 @@ __global__ void __launch_bounds__(256) route_kernel(
         }
         const int n = (int)min64(TPW, tend - t0);
         float z[TPW][NV];
-        if constexpr (FROM_LOGITS) {
 #pragma unroll
-            for (int i = 0; i < TPW; ++i)
+        for (int i = 0; i < TPW; ++i)
 #pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    const int e = lane + 32 * v;
-                    z[i][v] = (i < n && e < E) ? logits_in[(t0 + i) * E + e] : 0.f;
-                    if (bias && e < E) z[i][v] += bias[party * E + e];
-                }
-        } else {
-            float acc[TPW][EMAX];
-#pragma unroll
-            for (int i = 0; i < TPW; ++i)
-#pragma unroll
-                for (int e = 0; e < EMAX; ++e) acc[i][e] = 0.f;
-            const T* W = wr + (int64_t)party * E * d;
-            for (int64_t v = lane; v < nvec; v += 32) {
-                float xv[TPW][VN];
-#pragma unroll
-                for (int i = 0; i < TPW; ++i) {
-                    if (i < n) V::load(x + (t0 + i) * d + v * VN, xv[i]);
-                    else {
-#pragma unroll
-                        for (int q = 0; q < VN; ++q) xv[i][q] = 0.f;
-                    }
-                }
-#pragma unroll
-                for (int e = 0; e < EMAX; ++e) {
-                    if (e < E) {
-                        float wv[VN];
-                        V::load(W + (int64_t)e * d + v * VN, wv);
-#pragma unroll
-                        for (int i = 0; i < TPW; ++i)
-#pragma unroll
-                            for (int q = 0; q < VN; ++q) acc[i][e] = fmaf(xv[i][q], wv[q], acc[i][e]);
-                    }
-                }
+            for (int v = 0; v < NV; ++v) {
+                const int e = lane + 32 * v;
+                z[i][v] = (i < n && e < E) ? logits_in[(t0 + i) * E + e] : 0.f;
+                if (bias && e < E) z[i][v] += bias[party * E + e];
             }
-#pragma unroll
-            for (int i = 0; i < TPW; ++i) {
-#pragma unroll
-                for (int v = 0; v < NV; ++v) z[i][v] = 0.f;
-#pragma unroll
-                for (int e = 0; e < EMAX; ++e) {
-                    float s = warp_sum(acc[i][e]);
-#pragma unroll
-                    for (int v = 0; v < NV; ++v)
-                        if (e == lane + 32 * v) z[i][v] = s;
-                }
-                if (bias) {
-#pragma unroll
-                    for (int v = 0; v < NV; ++v)
-                        if (lane + 32 * v < E) z[i][v] += bias[party * E + lane + 32 * v];
-                }
-            }
-        }
 #pragma unroll
         for (int i = 0; i < TPW; ++i)
             if (i < n)
-                softmax_topk_token<NV>(z[i], lane, E, k, normalize, t0 + i, party,
-                                       (FROM_LOGITS && !bias) ? nullptr : logits, probs, topk_idx,
-                                       topk_w, s_hist);
+                softmax_topk_token<NV>(z[i], lane, E, k, normalize, t0 + i, party, bias ? logits : nullptr, probs,
+                                       topk_idx, topk_w, s_hist);
     }
     __syncthreads();
     if (hist_smem) {
@@ -552,34 +635,51 @@ static int num_sms() {
     return n;
 }
 
-template <typename T, bool FROM>
-static cudaError_t launch_route_t(const RouteArgs& a, cudaStream_t s) {
+// gating of logits in a.logits_in
+static cudaError_t launch_gating(const RouteArgs& a, cudaStream_t s) {
     const int E = a.E;
     const size_t smem = a.P * E <= HIST_SMEM ? (size_t)a.P * E * sizeof(int) : 0;
     const int64_t groups_ub = a.T + a.P;  // upper bound with TPW = 1
     int blocks = (int)min64((groups_ub + 7) / 8, (int64_t)num_sms() * 8);
     if (blocks < 1) blocks = 1;
-    const T* x = (const T*)a.x;
-    const T* wr = (const T*)a.w_router;
-#define MOE_ROUTE_CASE(EM, TP)                                                                   \
-    (void)launch_pdl(route_kernel<T, EM, TP, FROM>, dim3(blocks), dim3(256), smem, s,                                       \
-        x, wr, a.bias, a.logits_in, a.po, a.P, a.T, a.d, E, a.k, a.normalize, a.logits, a.probs, \
-        a.topk_idx, a.topk_w, a.counts)
-    if constexpr (FROM) {
-        if (E <= 64) MOE_ROUTE_CASE(64, 4);
-        else if (E <= 128) MOE_ROUTE_CASE(128, 2);
-        else MOE_ROUTE_CASE(256, 1);
-    } else if (E <= 8) {
-        MOE_ROUTE_CASE(8, 8);
-    } else if (E <= 16) {
-        MOE_ROUTE_CASE(16, 4);
-    } else if (E <= 32) {
-        MOE_ROUTE_CASE(32, 2);
-    } else {
-        MOE_ROUTE_CASE(64, 1);
-    }
-#undef MOE_ROUTE_CASE
+#define MOE_GATE(EM, TP)                                                                              \
+    (void)launch_pdl(route_kernel<EM, TP>, dim3(blocks), dim3(256), smem, s, a.bias, a.logits_in, a.po, \
+                     a.P, a.T, E, a.k, a.normalize, a.logits, a.probs, a.topk_idx, a.topk_w, a.counts)
+    if (E <= 64) MOE_GATE(64, 4);
+    else if (E <= 128) MOE_GATE(128, 2);
+    else MOE_GATE(256, 1);
+#undef MOE_GATE
     return cudaGetLastError();
+}
+
+template <typename T, int EP, int TB>
+static cudaError_t launch_route_dot_t(const RouteArgs& a, cudaStream_t s) {
+    auto kern = route_dot_kernel<T, EP, TB>;
+    constexpr size_t smem = std::max<size_t>(2 * (size_t)(TB + EP) * RD_LD, (size_t)RD_THREADS * TB) * sizeof(float);
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr = true;
+    }
+    const unsigned blocks = (unsigned)((a.T + TB - 1) / TB + (a.po ? a.P : 0));
+    (void)launch_pdl(kern, dim3(blocks), dim3(RD_THREADS), smem, s, (const T*)a.x, (const T*)a.w_router, a.bias, a.po,
+                     a.P, a.T, a.d, a.E, a.k, a.normalize, a.logits, a.probs, a.topk_idx, a.topk_w, a.counts);
+    return cudaGetLastError();
+}
+
+// E <= 64. 16 tokens per CTA, 8 while those would not give every SM two CTAs (the weights
+// of a CTA are staged for its tokens alone, so fewer tokens cost more shared-memory traffic)
+template <typename T>
+static cudaError_t launch_route_dot(const RouteArgs& a, cudaStream_t s) {
+    if (a.T == 0) return cudaSuccess;
+    const bool few = a.T < 2 * 16 * (int64_t)num_sms();
+#define MOE_DOT(EP) (few ? launch_route_dot_t<T, EP, 8>(a, s) : launch_route_dot_t<T, EP, 16>(a, s))
+    if (a.E <= 8) return MOE_DOT(8);
+    if (a.E <= 16) return MOE_DOT(16);
+    if (a.E <= 32) return MOE_DOT(32);
+    return MOE_DOT(64);
+#undef MOE_DOT
 }
 
 // E > 64, fp32: the router's products x W_r[p]^T by the grouped fp32 GEMM into `logits` (groups = parties), then the gating pass reads them back, adds the
@@ -600,7 +700,7 @@ static cudaError_t launch_route_wide_f32(const RouteArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     RouteArgs b = a;
     b.logits_in = a.logits;
-    return launch_route_t<float, true>(b, s);
+    return launch_gating(b, s);
 }
 
 cudaError_t launch_route(const RouteArgs& a, bool bf16, bool from_logits, cudaStream_t s) {
@@ -609,11 +709,11 @@ cudaError_t launch_route(const RouteArgs& a, bool bf16, bool from_logits, cudaSt
     if (from_logits) {
         RouteArgs b = a;
         b.bias = nullptr;  // the caller's logits are final
-        return launch_route_t<float, true>(b, s);
+        return launch_gating(b, s);
     }
     if (bf16 && (a.E % 4 == 0 || a.E > 64) && a.T > 0) return launch_route_tc(a, s);
     if (a.E > 64) return a.T > 0 ? launch_route_wide_f32(a, s) : cudaSuccess;
-    return bf16 ? launch_route_t<__nv_bfloat16, false>(a, s) : launch_route_t<float, false>(a, s);
+    return bf16 ? launch_route_dot<__nv_bfloat16>(a, s) : launch_route_dot<float>(a, s);
 }
 
 cudaError_t launch_aux_loss(const float* probs, const int32_t* counts, const int32_t* po, int P,
