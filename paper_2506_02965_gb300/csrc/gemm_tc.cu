@@ -699,10 +699,10 @@ __global__ void __launch_bounds__(THREADS, OCC)
                 // group. Only K=16 steps that contain valid rows are issued, and inside the
                 // last of them the A rows past the group's end are zeroed (A alone suffices:
                 // their products with any finite B row vanish).
-                int ksteps = KB * KPS / 16;
                 const bool dwt = DW2 && ti.dw;
-                if ((VAR_K || dwt) && kb == ti.k_iters - 1 && ti.last_rows < KB) {
-                    ksteps = (ti.last_rows + 15) / 16;
+                const bool part = (VAR_K || dwt) && kb == ti.k_iters - 1 && ti.last_rows < KB;
+                const int ksteps = part ? (ti.last_rows + 15) / 16 : KB * KPS / 16;
+                if (part) {
                     const int zr0 = ti.last_rows, zr1 = ksteps * 16;
                     if (zr1 > zr0) {
                         uint8_t* base = ring_ptr + (size_t)stage * STAGE_BYTES;
@@ -718,9 +718,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
                 }
                 fence_after();
                 if (lane == 0) {
-#pragma unroll
-                    for (int kk = 0; kk < KB * KPS / 16; ++kk) {
-                        if (kk >= ksteps) break;
+                    auto step = [&](int kk) {
                         uint64_t ad, bd;
                         if (!A_MN && !dwt) ad = smem_desc(sa + (kk / (KB / 16)) * A_BOX + (kk % (KB / 16)) * 32, 16, 1024);
                         else ad = smem_desc(sa + (kk / (KB / 16)) * A_BOX + (kk % (KB / 16)) * 2048, ATOM, 1024);
@@ -728,6 +726,15 @@ __global__ void __launch_bounds__(THREADS, OCC)
                         else bd = smem_desc(sb + (kk / (KB / 16)) * B_BOX + (kk % (KB / 16)) * 2048, ATOM, 1024);
                         if constexpr (PAIR) mma_bf16_pair(tmem_d, ad, bd, IDESC, (kb | kk) ? 1u : 0u);
                         else mma_bf16(tmem_d, ad, bd, dwt ? IDESC_DW : IDESC, (kb | kk) ? 1u : 0u);
+                    };
+                    // whole k-blocks without a check per step (with one, the issuing thread
+                    // held back the weight-gradient launches by up to 20%)
+                    if (!part) {
+#pragma unroll
+                        for (int kk = 0; kk < KB * KPS / 16; ++kk) step(kk);
+                    } else {
+#pragma unroll 1
+                        for (int kk = 0; kk < ksteps; ++kk) step(kk);
                     }
                     if constexpr (PAIR) mma_commit_pair(empty_bar(stage), 3);  // both producers
                     else mma_commit(empty_bar(stage));
@@ -794,7 +801,10 @@ __global__ void __launch_bounds__(THREADS, OCC)
                             }
                             __syncwarp();
                             if (lane == 0) {
-                                asm volatile("fence.acq_rel.cluster;" ::: "memory");
+                                // release of the zeroed shared memory only: a full cluster
+                                // fence waits for all of the SM's memory traffic (14-18% of
+                                // the weight-gradient launches at 512 and 768 rows an expert)
+                                fence_release_smem_cluster();
                                 mbar_complete_tx_remote(map_to_rank(full_bar(st2), 0), STAGE_BYTES);
                             }
                             __syncwarp();
@@ -1030,7 +1040,12 @@ __global__ void __launch_bounds__(THREADS, OCC)
             fence_before();
             __syncwarp();
             if (lane == 0) {
-                if constexpr (PAIR) mbar_arrive_remote(map_to_rank(tempty_bar(acc), 0));
+                if constexpr (PAIR) {
+                    // (a release at cluster scope of everything the warp wrote would wait for
+                    // its output too: 3-5% of a launch with short contractions)
+                    fence_release_smem_cluster();
+                    mbar_arrive_remote(map_to_rank(tempty_bar(acc), 0));
+                }
                 else mbar_arrive(tempty_bar(acc));
             }
             if (++acc == 2) {
