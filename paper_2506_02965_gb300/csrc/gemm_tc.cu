@@ -103,7 +103,22 @@ struct Tile {
     bool dw;            // a tile of the second (K-variable) problem of a fused launch
     int we;             // expert whose weights (M-variable) or weight gradient (K-variable)
                         // the tile uses: group_expert[g], or g
+    int ntok;           // swapped tile (below): its rows rounded up to 16, else 0
 };
+
+// Swapped tiles of the M-variable pairs. An expert's last tile holds 1 to 256 of its rows,
+// but a pair's MMA always computes 256: at 512 rows an expert a fifth of all MMAs multiply
+// other experts' rows that are never stored. With at most SWAP_ROWS rows the operands are
+// exchanged: the weights are the MMA's 256-row operand (128 features per CTA, already laid
+// out like that in shared memory) and the rows its N dimension, which goes in steps of 16.
+// The accumulator is then transposed (lane = feature, column = row) and the epilogue writes
+// 32 features of a row at a time straight from registers.
+// Up to 128 rows: above, little is saved and the register epilogue costs more (dA with
+// tiles of up to 240 rows: 245 -> 429 us). Measured at 768 rows an expert (d = 2048, F = 1408):
+// dX 373 -> 350 us, GEMM2 196 -> 188, dA 249 -> 241; at 6 rows GEMM2 70 -> 65. Not in GEMM1:
+// gate and up of a feature meet in one lane only with 16-row weight boxes, whose TMA rate
+// costs more than the MMAs saved (389 -> 414 us; at 6 rows 135 -> 150).
+constexpr int SWAP_ROWS = 128;
 
 // ------------------------------------------------------------------------ router epilogue
 // Gating of Alg. 7 for the token of this TMEM lane: the thread holds all BN >= E
@@ -279,6 +294,87 @@ __device__ __forceinline__ void route_epilogue_wide(const Params& p, const Tile&
     }
 }
 
+// ------------------------------------------------------------------------ swapped tiles
+// Lane l of warp q of CTA `rank` holds one feature, its columns the tile's rows. Two rows
+// j, j + 1 at a time, neighbouring lanes exchange values so that each lane holds two features
+// of one of the two rows, and a warp's 32 lanes move 64 contiguous bytes of both.
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+// (a: row j, b: row j + 1) of this lane's feature -> the bf16 pair of features (l & ~1,
+// l | 1) of row j + (l & 1)
+__device__ __forceinline__ uint32_t pair_up(float a, float b, int lane) {
+    const float other = __shfl_xor_sync(0xffffffffu, (lane & 1) ? a : b, 1);
+    return (lane & 1) ? pack_bf16(other, b) : pack_bf16(a, other);
+}
+// the inverse for loads: u = the pair of row j + (l & 1) -> this feature's values of j, j + 1
+__device__ __forceinline__ void pair_down(uint32_t u, int lane, float* a, float* b) {
+    const float lo = __uint_as_float(u << 16), hi = __uint_as_float(u & 0xffff0000u);
+    const float other = __shfl_xor_sync(0xffffffffu, (lane & 1) ? lo : hi, 1);
+    *a = (lane & 1) ? other : lo;
+    *b = (lane & 1) ? hi : other;
+}
+
+template <int EPI>
+__device__ __forceinline__ void swapped_epilogue(const Params& p, const Tile& ti, int rank, int q, int lane, uint32_t tbase) {
+    const int v = ti.mvalid - ti.m0;       // rows of the tile
+    const int64_t row0 = ti.out_row + ti.m0;
+    const int F = p.F;
+    const int n = ti.n0 + rank * 128 + q * 32 + (lane & ~1);  // this lane's pair of features
+    if (n >= p.N) return;                                      // (a ragged last tile: whole CTAs)
+#pragma unroll 1
+    for (int c = 0; c < v; c += 32) {
+        if constexpr (EPI == EPI_STORE) {
+            float y[32];
+            tmem_ld32(tbase + c, y);
+            __nv_bfloat16* out = (__nv_bfloat16*)p.out0 + (row0 + c) * (int64_t)p.N + n;
+#pragma unroll
+            for (int i = 0; i < 32; i += 2) {
+                const uint32_t u = pair_up(y[i], y[i + 1], lane);
+                const int j = i + (lane & 1);
+                if (c + j < v) *reinterpret_cast<uint32_t*>(out + j * (int64_t)p.N) = u;
+            }
+        } else {  // SwiGLU backward: y = dA
+            const __nv_bfloat16* gu = (const __nv_bfloat16*)p.aux + (row0 + c) * (int64_t)(2 * F) + n;
+            __nv_bfloat16* dh = (__nv_bfloat16*)p.out0 + (row0 + c) * (int64_t)(2 * F) + n;
+#pragma unroll 1
+            for (int h = 0; h < 32 && c + h < v; h += 16) {
+                uint32_t gr[8], ur[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int j = h + 2 * i + (lane & 1);
+                    gr[i] = ur[i] = 0;
+                    if (c + j < v) {
+                        gr[i] = *reinterpret_cast<const uint32_t*>(gu + j * (int64_t)(2 * F));
+                        ur[i] = *reinterpret_cast<const uint32_t*>(gu + j * (int64_t)(2 * F) + F);
+                    }
+                }
+                float y[16];
+                tmem_ld16(tbase + c + h, y);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    float G[2], U[2], dg[2], du[2];
+                    pair_down(gr[i], lane, &G[0], &G[1]);
+                    pair_down(ur[i], lane, &U[0], &U[1]);
+#pragma unroll
+                    for (int w = 0; w < 2; ++w) {
+                        const float sg = __fdividef(1.0f, 1.0f + __expf(-G[w])), d = y[2 * i + w];
+                        du[w] = d * G[w] * sg;
+                        dg[w] = d * U[w] * sg * (1.0f + G[w] * (1.0f - sg));
+                    }
+                    const uint32_t dgu = pair_up(dg[0], dg[1], lane), duu = pair_up(du[0], du[1], lane);
+                    const int j = h + 2 * i + (lane & 1);
+                    if (c + j < v) {
+                        *reinterpret_cast<uint32_t*>(dh + j * (int64_t)(2 * F)) = dgu;
+                        *reinterpret_cast<uint32_t*>(dh + j * (int64_t)(2 * F) + F) = duu;
+                    }
+                }
+            }
+        }
+    }
+}
+
 // ------------------------------------------------------------------------ the kernel
 // PAIR: the two CTAs of a cluster compute one 256 x BN tile with tcgen05 cta_group::2
 // MMAs issued by CTA 0: each CTA holds 128 rows of A and BN/2 rows of B in its own
@@ -294,7 +390,8 @@ __global__ void __launch_bounds__(THREADS, OCC)
     grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                         const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmO0,
-                        const __grid_constant__ CUtensorMap tmO1, const Params p,
+                        const __grid_constant__ CUtensorMap tmO1,
+                        const __grid_constant__ CUtensorMap tmAs, const Params p,
                         const __grid_constant__ CUtensorMap tmA2,
                         const __grid_constant__ CUtensorMap tmB2,
                         const __grid_constant__ CUtensorMap tmO2, const Params p2) {
@@ -302,6 +399,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
     static_assert(!DW2 || (B_MN && !VAR_K && !PAIR && BN == 256), "fused: M-variable, MN-major B");
     static_assert(OCC == 1 || (!PAIR && !DW2 && 2 * BN * OCC <= 512), "shared SMs: single-CTA tiles, TMEM for all");
     constexpr bool A_MN = VAR_K;
+    constexpr bool SWAP = PAIR && !VAR_K && EPI != EPI_SWIGLU_FWD;  // swapped tiles possible
     constexpr int NPAIR = PAIR ? 2 : 1;
     constexpr int BNL = BN / NPAIR;  // B rows held by this CTA
     constexpr int BMP = BM * NPAIR;  // rows of one (pair) tile
@@ -406,6 +504,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
     auto tile_at = [&](int t) -> Tile {
         Tile ti;
         ti.dw = false;
+        ti.ntok = 0;
         if constexpr (DW2) {
             if (t >= s_total1) {  // second problem: K-variable, rows of group g
                 const int per = (p2.Mout / BM) * (p2.N / BN);
@@ -473,6 +572,13 @@ __global__ void __launch_bounds__(THREADS, OCC)
             ti.out_row = o0;
             ti.k_iters = p.K / (BK * KPS);
             ti.last_rows = BK;
+            if constexpr (SWAP) {
+                const int v = (int)nrows - mt * BMP;
+                if (v <= SWAP_ROWS) {
+                    ti.ntok = (v + 15) / 16 * 16;
+                    ti.m0 = mt * BMP;  // both CTAs hold features of the same rows
+                }
+            }
         }
         return ti;
     };
@@ -570,6 +676,10 @@ __global__ void __launch_bounds__(THREADS, OCC)
             };
             for (int t = tile0; t < total_tiles && ok; t += tile_step) {
                 const Tile ti = tile_at(t);
+                // a swapped tile's rows: half in each CTA, in boxes of 32
+                const int trows = SWAP ? ti.ntok / 2 : 0;
+                uint32_t tile_bytes = NPAIR * STAGE_BYTES;  // per stage, both CTAs of a pair
+                if (SWAP && trows) tile_bytes = NPAIR * (B_BYTES + (uint32_t)((trows + 31) / 32) * (32u * 128u * KPS));
                 for (int kb = 0; kb < ti.k_iters; ++kb) {
                     if (!wait_bar(empty_bar(stage), phase ^ 1u)) {
                         ok = false;
@@ -590,7 +700,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
                     // peer reuses a stage only after the leader's MMAs released it, so its bytes
                     // always count towards the phase the leader arms.
                     if constexpr (PAIR) {
-                        if (rank == 0) mbar_expect_tx(full_bar(stage), NPAIR * STAGE_BYTES);
+                        if (rank == 0) mbar_expect_tx(full_bar(stage), tile_bytes);
                         else if (part_peer) {
                             mbar_expect_tx(fb, STAGE_BYTES);
                             parmed |= 1u << stage;
@@ -604,8 +714,15 @@ __global__ void __launch_bounds__(THREADS, OCC)
                     const int k0 = kb * KB * KPS;
                     const bool dw = DW2 && ti.dw;
                     if (!A_MN && !dw) {
+                        if (SWAP && trows) {
+                            const int row = (int)(ti.a_row + ti.m0) + (int)rank * trows;
+                            for (int r = 0; r < trows; r += 32)
 #pragma unroll
-                        for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX, &tmA, fb, k0 + KB * i, (int)(ti.a_row + ti.m0));
+                                for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX + r * 128, &tmAs, fb, k0 + KB * i, row + r);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX, &tmA, fb, k0 + KB * i, (int)(ti.a_row + ti.m0));
+                        }
                     } else {
                         const CUtensorMap* mA = dw ? &tmA2 : &tmA;
 #pragma unroll
@@ -682,6 +799,8 @@ __global__ void __launch_bounds__(THREADS, OCC)
         // write both CTAs' TMEM)
         for (int t = tile0; t < total_tiles && ok && rank == 0; t += tile_step) {
             const Tile ti = tile_at(t);
+            // kind::f16 descriptor of a swapped tile: A = weights (M = 256), B = rows (K-major)
+            const uint32_t idesc_s = instr_desc<16, B_MN, false, BMP>() - (2u << 17) + ((uint32_t)(ti.ntok >> 3) << 17);
             if (!wait_bar(tempty_bar(acc), acc_phase ^ 1u)) {
                 ok = false;
                 break;
@@ -718,23 +837,27 @@ __global__ void __launch_bounds__(THREADS, OCC)
                 }
                 fence_after();
                 if (lane == 0) {
-                    auto step = [&](int kk) {
+                    auto step = [&](int kk, bool swapped) {
                         uint64_t ad, bd;
                         if (!A_MN && !dwt) ad = smem_desc(sa + (kk / (KB / 16)) * A_BOX + (kk % (KB / 16)) * 32, 16, 1024);
                         else ad = smem_desc(sa + (kk / (KB / 16)) * A_BOX + (kk % (KB / 16)) * 2048, ATOM, 1024);
                         if (!B_MN) bd = smem_desc(sb + (kk / (KB / 16)) * B_BOX + (kk % (KB / 16)) * 32, 16, 1024);
                         else bd = smem_desc(sb + (kk / (KB / 16)) * B_BOX + (kk % (KB / 16)) * 2048, ATOM, 1024);
-                        if constexpr (PAIR) mma_bf16_pair(tmem_d, ad, bd, IDESC, (kb | kk) ? 1u : 0u);
+                        if (SWAP && swapped) mma_bf16_pair(tmem_d, bd, ad, idesc_s, (kb | kk) ? 1u : 0u);
+                        else if constexpr (PAIR) mma_bf16_pair(tmem_d, ad, bd, IDESC, (kb | kk) ? 1u : 0u);
                         else mma_bf16(tmem_d, ad, bd, dwt ? IDESC_DW : IDESC, (kb | kk) ? 1u : 0u);
                     };
                     // whole k-blocks without a check per step (with one, the issuing thread
                     // held back the weight-gradient launches by up to 20%)
-                    if (!part) {
+                    if (SWAP && ti.ntok) {
 #pragma unroll
-                        for (int kk = 0; kk < KB * KPS / 16; ++kk) step(kk);
+                        for (int kk = 0; kk < KB * KPS / 16; ++kk) step(kk, true);
+                    } else if (!part) {
+#pragma unroll
+                        for (int kk = 0; kk < KB * KPS / 16; ++kk) step(kk, false);
                     } else {
 #pragma unroll 1
-                        for (int kk = 0; kk < ksteps; ++kk) step(kk);
+                        for (int kk = 0; kk < ksteps; ++kk) step(kk, false);
                     }
                     if constexpr (PAIR) mma_commit_pair(empty_bar(stage), 3);  // both producers
                     else mma_commit(empty_bar(stage));
@@ -850,7 +973,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
         if constexpr (EPI == EPI_SWIGLU_BWD) {
             if (tile0 < total_tiles) {
                 const Tile tf = tile_at(tile0);
-                if (!(DW2 && tf.dw)) gu_issue(tf, 0);
+                if (!(DW2 && tf.dw) && !tf.ntok) gu_issue(tf, 0);
             }
         }
         for (int t = tile0; t < total_tiles; t += tile_step) {
@@ -906,6 +1029,10 @@ __global__ void __launch_bounds__(THREADS, OCC)
                     __nv_bfloat16* direct[1] = {out + ti.n0 + c};
                     emit(1, vals, maps, cols, direct);
                 }
+            } else if (SWAP && ti.ntok) {
+                if (!wait_bar(tfull_bar(acc), acc_phase)) break;
+                fence_after();
+                swapped_epilogue<EPI>(p, ti, (int)rank, q, lane, tbase);
             } else if constexpr (EPI == EPI_SWIGLU_BWD) {
                 // dA in TMEM. G and U of each 32-column chunk arrive by TMA in one of two
                 // staging buffers (the next chunk's load is in flight while this one is
@@ -924,7 +1051,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
                     if (c + 1 < nchv) gu_issue(ti, c + 1);
                     else if (t + tile_step < total_tiles) {
                         const Tile tn = tile_at(t + tile_step);
-                        if (!(DW2 && tn.dw)) gu_issue(tn, 0);
+                        if (!(DW2 && tn.dw) && !tn.ntok) gu_issue(tn, 0);
                     }
                     const int b = gu_chunk & 1;
                     if (!gu_wait(b, (gu_chunk >> 1) & 1)) { stop = true; break; }
@@ -1146,11 +1273,12 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
                           const CUtensorMap& mo1, const Params& p, int64_t tiles_ub,
                           cudaStream_t s, const CUtensorMap* ma2 = nullptr,
                           const CUtensorMap* mb2 = nullptr, const CUtensorMap* mo2 = nullptr,
-                          const Params* p2 = nullptr) {
+                          const Params* p2 = nullptr, const CUtensorMap* mas = nullptr) {
     auto kern = grouped_gemm_kernel<BN, B_MN, VAR_K, EPI, PAIR, DW2, OCC>;
     const CUtensorMap& A2 = ma2 ? *ma2 : ma;
     const CUtensorMap& B2 = mb2 ? *mb2 : mb;
     const CUtensorMap& O2 = mo2 ? *mo2 : mo0;
+    const CUtensorMap& AS = mas ? *mas : ma;  // boxes of swapped tiles (M-variable pairs)
     Params P1 = p;
     Params P2 = p2 ? *p2 : p;
     constexpr int NPAIR = PAIR ? 2 : 1;
@@ -1207,11 +1335,11 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 2;
-        return cudaLaunchKernelEx(&cfg, kern, ma, mb, mo0, mo1, P1, A2, B2, O2, P2);
+        return cudaLaunchKernelEx(&cfg, kern, ma, mb, mo0, mo1, AS, P1, A2, B2, O2, P2);
     } else {
         const int grid = (int)std::min<int64_t>(tiles_ub, (int64_t)OCC * sm_count());
         P1.band = P2.band = band_for(grid);
-        (void)launch_pdl(kern, dim3(grid), dim3(THREADS), smem, s, ma, mb, mo0, mo1, P1, A2, B2, O2, P2);
+        (void)launch_pdl(kern, dim3(grid), dim3(THREADS), smem, s, ma, mb, mo0, mo1, AS, P1, A2, B2, O2, P2);
         return cudaGetLastError();
     }
 }
@@ -1288,8 +1416,9 @@ cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s) {
     // output rows in the 2D view of the outputs
     const int64_t o_rows = g.rows.offsets ? (int64_t)g.rows.rows
                                           : std::max<int64_t>(g.rows.rows, (int64_t)(g.G - 1) * g.rows.out_stride + g.rows.rows);
-    CUtensorMap ma, mb, mo0, mo1;
+    CUtensorMap ma, mb, mo0, mo1, mas;  // mas: A in boxes of 32 rows (swapped tiles)
     if (!make_map(&ma, g.a, g.K, a_rows, BM)) return cudaErrorInvalidValue;
+    if (pair && !make_map(&mas, g.a, g.K, a_rows, 32)) return cudaErrorInvalidValue;
     if (g.epi == EPI_SWIGLU_FWD) {
         const int F = g.N / 2;
         p.F = F;
@@ -1305,7 +1434,8 @@ cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s) {
         if (!make_map(&mo0, g.out0, g.N, o_rows, 0, true)) return cudaErrorInvalidValue;
         if (pair) {
             if (!make_map(&mb, g.b, g.K, (int64_t)g.G * g.N, 128)) return cudaErrorInvalidValue;
-            return launch<256, false, false, EPI_STORE, true>(ma, mb, mo0, mo0, p, pt_ub * ((g.N + 255) / 256), s);
+            return launch<256, false, false, EPI_STORE, true>(ma, mb, mo0, mo0, p, pt_ub * ((g.N + 255) / 256), s, nullptr,
+                                                              nullptr, nullptr, nullptr, &mas);
         }
         if (g.N % 256 == 0) {
             if (!make_map(&mb, g.b, g.K, (int64_t)g.G * g.N, 256)) return cudaErrorInvalidValue;
@@ -1322,14 +1452,17 @@ cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s) {
         if (!make_map(&mo0, g.out0, 2 * (int64_t)g.N, o_rows, 0, true)) return cudaErrorInvalidValue;
         if (!make_map(&mo1, g.aux, 2 * (int64_t)g.N, o_rows, 0, true)) return cudaErrorInvalidValue;
         if (pair)
-            return launch<256, true, false, EPI_SWIGLU_BWD, true>(ma, mb, mo0, mo1, p, pt_ub * ((g.N + 255) / 256), s);
+            return launch<256, true, false, EPI_SWIGLU_BWD, true>(ma, mb, mo0, mo1, p, pt_ub * ((g.N + 255) / 256), s,
+                                                                  nullptr, nullptr, nullptr, nullptr, &mas);
         if (g.N % 256 == 0) return launch<256, true, false, EPI_SWIGLU_BWD>(ma, mb, mo0, mo1, p, mt_ub * (g.N / 256), s);
         return launch<128, true, false, EPI_SWIGLU_BWD>(ma, mb, mo0, mo1, p, mt_ub * (g.N / 128), s);
     }
     if (!make_map(&mo0, g.out0, g.N, o_rows, 0, true)) return cudaErrorInvalidValue;
     if (g.slim && g.N % 128 == 0)
         return launch<128, true, false, EPI_STORE, false, false, 2>(ma, mb, mo0, mo0, p, mt_ub * (g.N / 128), s);
-    if (pair) return launch<256, true, false, EPI_STORE, true>(ma, mb, mo0, mo0, p, pt_ub * ((g.N + 255) / 256), s);
+    if (pair)
+        return launch<256, true, false, EPI_STORE, true>(ma, mb, mo0, mo0, p, pt_ub * ((g.N + 255) / 256), s, nullptr, nullptr,
+                                                         nullptr, nullptr, &mas);
     if (g.N % 256 == 0) return launch<256, true, false, EPI_STORE>(ma, mb, mo0, mo0, p, mt_ub * (g.N / 256), s);
     return launch<128, true, false, EPI_STORE>(ma, mb, mo0, mo0, p, mt_ub * (g.N / 128), s);
 }
