@@ -20,18 +20,26 @@ namespace moe {
 namespace tc {
 
 constexpr int BK = 64;  // 64 bf16 = 128 bytes = one 128B-swizzle row
-// Contraction rows per k-block: BK, except for CTA-pair K-variable tiles (weight
-// gradients), whose operands are both MN-major (64-element TMA boxes): 128-row boxes
-// there halve the boxes and stage hand-offs per byte (3 stages of 64 KiB per CTA).
-__host__ __device__ constexpr int kblock_rows(bool var_k, bool pair) { return (var_k && pair) ? 128 : BK; }
+// Contraction rows per k-block: BK, except for the weight gradients' CTA-pair and 128-wide
+// tiles, whose operands are both MN-major (64-element TMA boxes): 128-row boxes there halve
+// the boxes and stage hand-offs per byte (3 stages of 64 KiB per CTA).
+__host__ __device__ constexpr int kblock_rows(bool var_k, bool pair, int epi, int bn) {
+    return (var_k && epi == EPI_STORE && (pair || bn == 128)) ? 128 : BK;
+}
 // k-blocks per operand stage: 2 for the router up to 64 experts (its stream of x is bound
 // by a fixed cost per stage hand-off, so a stage carries two 64-wide boxes of each
-// operand; wider B would leave too few stages) and for the M-variable CTA-pair tiles
+// operand; wider B would leave too few stages), for the M-variable CTA-pair tiles
 // with a store or SwiGLU-forward epilogue (three stages of 64 KiB per CTA instead of six
 // of 32: the same bytes in flight, half the hand-offs, less power per flop under the
-// power cap), else 1 (the SwiGLU-backward pairs measured faster with six stages)
-__host__ __device__ constexpr int kblocks_per_stage(int epi, int bn, bool pair = false, bool var_k = false) {
-    return ((epi == 3 /* EPI_ROUTE */ && bn <= 64) || (pair && !var_k && epi != 2 /* EPI_SWIGLU_BWD */)) ? 2 : 1;
+// power cap) and for the 128-wide single-CTA tiles (three stages of 64 KiB instead of six:
+// dA at d = 3072, F = 640 46 -> 37 us, GEMM2 at d = 384 35 -> 28 us); else 1: the
+// SwiGLU-backward pairs measured faster with six stages, and 256-wide single-CTA tiles lose
+// with two stages of 96 KiB (GEMM1 47 -> 53 us)
+__host__ __device__ constexpr int kblocks_per_stage(int epi, int bn, bool pair, bool var_k, bool dw2, int occ) {
+    if (epi == EPI_ROUTE) return bn <= 64 ? 2 : 1;
+    if (var_k || dw2 || occ > 1) return 1;
+    if (pair) return epi != EPI_SWIGLU_BWD ? 2 : 1;
+    return bn == 128 ? 2 : 1;
 }
 constexpr int EPI_WARPS = 4;
 constexpr int THREADS = 64 + 32 * EPI_WARPS;  // TMA warp, MMA warp, epilogue warps
@@ -403,9 +411,10 @@ __global__ void __launch_bounds__(THREADS, OCC)
     constexpr int NPAIR = PAIR ? 2 : 1;
     constexpr int BNL = BN / NPAIR;  // B rows held by this CTA
     constexpr int BMP = BM * NPAIR;  // rows of one (pair) tile
-    constexpr int KB = kblock_rows(VAR_K, PAIR);  // contraction rows per k-block
-    constexpr uint32_t ATOM = KB * 128;              // bytes of one 64-wide MN-major box
-    constexpr int KPS = kblocks_per_stage(EPI, BN, PAIR, VAR_K);
+    constexpr int KB = kblock_rows(VAR_K, PAIR, EPI, BN);  // contraction rows per k-block
+    constexpr int KPS = kblocks_per_stage(EPI, BN, PAIR, VAR_K, DW2, OCC);
+    constexpr uint32_t ATOM = KB * 128;         // bytes of one 64-wide MN-major box
+    constexpr uint32_t ATOM_B = ATOM * KPS;     // of B's: one box holds all of a stage's k-blocks
     constexpr uint32_t A_BOX = BM * KB * 2;   // one k-block of A
     constexpr uint32_t B_BOX = BNL * KB * 2;  // one k-block of B
     constexpr uint32_t A_BYTES = A_BOX * KPS;
@@ -662,13 +671,13 @@ __global__ void __launch_bounds__(THREADS, OCC)
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
-            int issued_phase[NST];
-            for (int s = 0; s < NST; ++s) issued_phase[s] = -1;
+            uint32_t issued = 0, issued_par = 0;  // stages ever filled, and the parity of their last fill
             // K-variable pair peer: stages whose own barrier was ever armed, and per stage
             // the parity of the next phase to arm
             uint32_t parmed = 0, pnext = 0;
             bool ok = true;
             // every TMA load is counted on the leader's full barrier (CTA 0 of a pair)
+            const uint32_t full0 = PAIR ? map_to_rank(bar0, 0) : bar0;
             bool local_bar = false;  // this stage's copies complete on this CTA's own barrier
             auto load = [&](uint32_t dst, const CUtensorMap* map, uint32_t fb, int c0, int c1) {
                 if (PAIR && !local_bar) tma_load_2d_pair(dst, map, fb, c0, c1);
@@ -676,10 +685,19 @@ __global__ void __launch_bounds__(THREADS, OCC)
             };
             for (int t = tile0; t < total_tiles && ok; t += tile_step) {
                 const Tile ti = tile_at(t);
+                const bool dw = DW2 && ti.dw;
                 // a swapped tile's rows: half in each CTA, in boxes of 32
                 const int trows = SWAP ? ti.ntok / 2 : 0;
                 uint32_t tile_bytes = NPAIR * STAGE_BYTES;  // per stage, both CTAs of a pair
+                if (EPI == EPI_ROUTE) tile_bytes = (uint32_t)p.tile_rows * 128u * KPS + B_BYTES;  // A boxes of tile_rows rows
                 if (SWAP && trows) tile_bytes = NPAIR * (B_BYTES + (uint32_t)((trows + 31) / 32) * (32u * 128u * KPS));
+                // the tile's coordinates: A (first row, or contraction row), B (row, or contraction row)
+                const int arow = (int)ti.a_row + ((A_MN || dw) ? 0 : ti.m0 + (int)rank * trows);
+                int brow;
+                if (VAR_K || dw) brow = (int)ti.b_row;
+                else if (B_MN) brow = (int)((int64_t)ti.we * p.b_group_rows);
+                else brow = (int)((int64_t)ti.we * p.b_group_rows + ti.n0) +
+                            (EPI == EPI_SWIGLU_FWD ? (PAIR && rank ? p.F : 0) : (int)rank * BNL);
                 for (int kb = 0; kb < ti.k_iters; ++kb) {
                     if (!wait_bar(empty_bar(stage), phase ^ 1u)) {
                         ok = false;
@@ -687,76 +705,56 @@ __global__ void __launch_bounds__(THREADS, OCC)
                     }
                     const uint32_t sa = ring + stage * STAGE_BYTES;
                     const uint32_t sb = sa + A_BYTES;
-                    // K-variable pair, peer, partial last k-block: its copies land on its own
-                    // barrier; the MMA warp zeroes the rows past the group's end and then
-                    // credits these bytes to the leader's full barrier
-                    const bool part_peer = PAIR && VAR_K && rank == 1 && kb == ti.k_iters - 1 && ti.last_rows < KB;
-                    const uint32_t fb = part_peer ? pfull_bar(stage)
-                                                  : (PAIR ? map_to_rank(full_bar(stage), 0) : full_bar(stage));
-                    local_bar = part_peer;
+                    uint32_t fb = full0 + 8u * stage;
                     // In a pair only the leader arrives, expecting the bytes of both CTAs: the
                     // peer's copies complete on the leader's barrier without an arrival (a
                     // cluster-scope arrive per stage cost the producers most of their time). The
                     // peer reuses a stage only after the leader's MMAs released it, so its bytes
                     // always count towards the phase the leader arms.
-                    if constexpr (PAIR) {
-                        if (rank == 0) mbar_expect_tx(full_bar(stage), tile_bytes);
-                        else if (part_peer) {
+                    if (!PAIR || rank == 0) mbar_expect_tx(full_bar(stage), tile_bytes);
+                    if constexpr (PAIR && VAR_K) {
+                        // peer, partial last k-block: its copies land on its own barrier; the MMA
+                        // warp zeroes the rows past the group's end and then credits these bytes
+                        // to the leader's full barrier
+                        local_bar = rank == 1 && kb == ti.k_iters - 1 && ti.last_rows < KB;
+                        if (local_bar) {
+                            fb = pfull_bar(stage);
                             mbar_expect_tx(fb, STAGE_BYTES);
                             parmed |= 1u << stage;
                             pnext ^= 1u << stage;
                         }
-                    } else if constexpr (EPI == EPI_ROUTE) {
-                        mbar_expect_tx(fb, (uint32_t)p.tile_rows * 128u * KPS + B_BYTES);  // A boxes of tile_rows rows
-                    } else {
-                        mbar_expect_tx(fb, STAGE_BYTES);
                     }
                     const int k0 = kb * KB * KPS;
-                    const bool dw = DW2 && ti.dw;
                     if (!A_MN && !dw) {
                         if (SWAP && trows) {
-                            const int row = (int)(ti.a_row + ti.m0) + (int)rank * trows;
                             for (int r = 0; r < trows; r += 32)
 #pragma unroll
-                                for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX + r * 128, &tmAs, fb, k0 + KB * i, row + r);
+                                for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX + r * 128, &tmAs, fb, k0 + KB * i, arow + r);
                         } else {
 #pragma unroll
-                            for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX, &tmA, fb, k0 + KB * i, (int)(ti.a_row + ti.m0));
+                            for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX, &tmA, fb, k0 + KB * i, arow);
                         }
                     } else {
                         const CUtensorMap* mA = dw ? &tmA2 : &tmA;
 #pragma unroll
-                        for (int i = 0; i < BM / 64; ++i)
-                            load(sa + i * ATOM, mA, fb, ti.m0 + 64 * i, (int)(ti.a_row + k0));
+                        for (int i = 0; i < BM / 64; ++i) load(sa + i * ATOM, mA, fb, ti.m0 + 64 * i, arow + k0);
                     }
-                    if (EPI == EPI_SWIGLU_FWD) {
-                        // 128 gate rows then 128 up rows of the same features; in a pair the
-                        // leader holds the gate half and the peer the up half
-                        const int64_t r = (int64_t)ti.we * p.b_group_rows + ti.n0;
-                        if constexpr (PAIR) {
+                    if (!B_MN) {
 #pragma unroll
-                            for (int j = 0; j < KPS; ++j)
-                                load(sb + j * B_BOX, &tmB, fb, k0 + KB * j, (int)(r + (rank ? p.F : 0)));
-                        } else {
-                            load(sb, &tmB, fb, k0, (int)r);
-                            load(sb + 128 * 128, &tmB, fb, k0, (int)(r + p.F));
+                        for (int i = 0; i < KPS; ++i) {
+                            load(sb + i * B_BOX, &tmB, fb, k0 + KB * i, brow);
+                            // SwiGLU forward: 128 gate rows, then 128 up rows of the same features
+                            // (in a pair the leader holds the gate half and the peer the up half)
+                            if (EPI == EPI_SWIGLU_FWD && !PAIR) load(sb + i * B_BOX + 128 * 128, &tmB, fb, k0 + KB * i, brow + p.F);
                         }
-                    } else if (!B_MN) {
-#pragma unroll
-                        for (int i = 0; i < KPS; ++i)
-                            load(sb + i * B_BOX, &tmB, fb, k0 + KB * i,
-                                 (int)((int64_t)ti.we * p.b_group_rows + ti.n0 + rank * BNL));
                     } else {
-                        const int64_t krow = (VAR_K || dw) ? (ti.b_row + k0) : ((int64_t)ti.we * p.b_group_rows + k0);
                         const CUtensorMap* mB = dw ? &tmB2 : &tmB;
 #pragma unroll
-                        for (int j = 0; j < KPS; ++j)
-#pragma unroll
-                            for (int i = 0; i < BNL / 64; ++i)
-                                load(sb + j * B_BOX + i * ATOM, mB, fb, ti.n0 + (int)rank * BNL + 64 * i,
-                                     (int)(krow + KB * j));
+                        for (int i = 0; i < BNL / 64; ++i)
+                            load(sb + i * ATOM_B, mB, fb, ti.n0 + (int)rank * BNL + 64 * i, brow + k0);
                     }
-                    issued_phase[stage] = (int)phase;
+                    issued |= 1u << stage;
+                    issued_par = (issued_par & ~(1u << stage)) | (phase << stage);
                     if (++stage == NST) {
                         stage = 0;
                         phase ^= 1u;
@@ -779,9 +777,9 @@ __global__ void __launch_bounds__(THREADS, OCC)
                 // let every copy started into this pair land before the CTAs exit (the
                 // leader's full barriers count the peer's bytes too)
                 for (int s = 0; s < NST; ++s) {
-                    if (issued_phase[s] < 0) continue;
+                    if (!((issued >> s) & 1u)) continue;
                     const uint64_t t0 = gtimer();
-                    while (!mbar_try(full_bar(s), (uint32_t)issued_phase[s]) &&
+                    while (!mbar_try(full_bar(s), (issued_par >> s) & 1u) &&
                            gtimer() - t0 < drain_limit) {
                     }
                 }
@@ -842,7 +840,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
                         if (!A_MN && !dwt) ad = smem_desc(sa + (kk / (KB / 16)) * A_BOX + (kk % (KB / 16)) * 32, 16, 1024);
                         else ad = smem_desc(sa + (kk / (KB / 16)) * A_BOX + (kk % (KB / 16)) * 2048, ATOM, 1024);
                         if (!B_MN) bd = smem_desc(sb + (kk / (KB / 16)) * B_BOX + (kk % (KB / 16)) * 32, 16, 1024);
-                        else bd = smem_desc(sb + (kk / (KB / 16)) * B_BOX + (kk % (KB / 16)) * 2048, ATOM, 1024);
+                        else bd = smem_desc(sb + kk * 2048, ATOM_B, 1024);
                         if (SWAP && swapped) mma_bf16_pair(tmem_d, bd, ad, idesc_s, (kb | kk) ? 1u : 0u);
                         else if constexpr (PAIR) mma_bf16_pair(tmem_d, ad, bd, IDESC, (kb | kk) ? 1u : 0u);
                         else mma_bf16(tmem_d, ad, bd, dwt ? IDESC_DW : IDESC, (kb | kk) ? 1u : 0u);
@@ -1282,8 +1280,8 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
     Params P1 = p;
     Params P2 = p2 ? *p2 : p;
     constexpr int NPAIR = PAIR ? 2 : 1;
-    constexpr int KB = kblock_rows(VAR_K, PAIR);
-    constexpr int STB = (BM * KB * 2 + BN / NPAIR * KB * 2) * kblocks_per_stage(EPI, BN, PAIR, VAR_K);  // bytes of one operand stage
+    constexpr int KB = kblock_rows(VAR_K, PAIR, EPI, BN);
+    constexpr int STB = (BM * KB * 2 + BN / NPAIR * KB * 2) * kblocks_per_stage(EPI, BN, PAIR, VAR_K, DW2, OCC);  // bytes of one operand stage
     constexpr int NST = num_stages((uint32_t)STB, EPI, OCC);
     const int extra_max = EPI == EPI_ROUTE ? 64 * 64 * 4 : EPI_WARPS * epi_stage_bytes(EPI);
     const int extra = EPI == EPI_ROUTE ? p.hist_n * 4 : EPI_WARPS * epi_stage_bytes(EPI);
@@ -1373,14 +1371,20 @@ bool gemm_m_uses_pairs(const GemmMArgs& g) {
 }
 
 // K-variable weight gradients (dW = A^T B over each group's rows) as 256 x 256 CTA-pair
-// tiles: both output dimensions multiples of 256, and (AUTO) at least four rounds of
-// pair tiles.
+// tiles: M a multiple of 256, and (AUTO) no slower by rounds: a launch takes its rounds of
+// tiles times a tile's time per contraction row, measured as 4.9 (pairs), 6.7 (128 x 256) and
+// 4.5 (128 x 128) in the same unit. (Two shared experts of 8192 rows: dW1 in 3 pair rounds
+// where 128 x 256 tiles take 3, dW2 in 2 where 128 x 128 tiles take 3: 166 -> 123 and 157 -> 82 us.)
 bool gemm_k_uses_pairs(const GemmKArgs& g) {
     using namespace tc;
     if (g.epi != EPI_STORE || g.M % 256 != 0 || g.N % 128 != 0) return false;
     if (g_pairs == MOE_PAIRS_ALL) return true;
     if (g_pairs != MOE_PAIRS_AUTO) return false;
-    return (int64_t)g.G * (g.M / 256) * ((g.N + 255) / 256) >= 4 * (int64_t)(sm_count() / 2);
+    const bool wide = g.N % 256 == 0;
+    const int64_t pairs = sm_count() / 2, sms = sm_count();
+    const int64_t tp = (int64_t)g.G * (g.M / 256) * ((g.N + 255) / 256);
+    const int64_t ts = (int64_t)g.G * (g.M / 128) * (wide ? g.N / 256 : g.N / 128);
+    return (tp + pairs - 1) / pairs * 49 <= (ts + sms - 1) / sms * (wide ? 67 : 45);
 }
 
 // M-variable grouped GEMM (forward, dA, dX).
@@ -1446,7 +1450,9 @@ cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s) {
     }
     // MN-major B: weights stored [G*K, N] (or [G*b_rows, N])
     p.b_group_rows = g.b_rows ? g.b_rows : g.K;
-    if (!make_map(&mb, g.b, g.N, (int64_t)g.G * p.b_group_rows, 64)) return cudaErrorInvalidValue;
+    const bool slim = g.slim && g.epi == EPI_STORE && g.N % 128 == 0;
+    const int kps = kblocks_per_stage(g.epi, pair || g.N % 256 == 0 ? 256 : 128, pair, false, false, slim ? 2 : 1);
+    if (!make_map(&mb, g.b, g.N, (int64_t)g.G * p.b_group_rows, BK * kps)) return cudaErrorInvalidValue;
     if (g.epi == EPI_SWIGLU_BWD) {
         p.F = g.N;
         if (!make_map(&mo0, g.out0, 2 * (int64_t)g.N, o_rows, 0, true)) return cudaErrorInvalidValue;
@@ -1458,7 +1464,7 @@ cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s) {
         return launch<128, true, false, EPI_SWIGLU_BWD>(ma, mb, mo0, mo1, p, mt_ub * (g.N / 128), s);
     }
     if (!make_map(&mo0, g.out0, g.N, o_rows, 0, true)) return cudaErrorInvalidValue;
-    if (g.slim && g.N % 128 == 0)
+    if (slim)
         return launch<128, true, false, EPI_STORE, false, false, 2>(ma, mb, mo0, mo0, p, mt_ub * (g.N / 128), s);
     if (pair)
         return launch<256, true, false, EPI_STORE, true>(ma, mb, mo0, mo0, p, pt_ub * ((g.N + 255) / 256), s, nullptr, nullptr,
@@ -1491,7 +1497,7 @@ cudaError_t launch_gemm_k(const GemmKArgs& g, bool bf16, cudaStream_t s) {
                                           : std::max<int64_t>(g.rows.rows, (int64_t)(g.G - 1) * g.rows.b_stride + g.rows.rows);
     CUtensorMap ma, mb, mo;
     const bool pair = g.epi == EPI_STORE && gemm_k_uses_pairs(g);
-    const int kbr = kblock_rows(true, pair);  // box rows of the MN-major operands
+    const int kbr = kblock_rows(true, pair, g.epi, g.N % 256 ? 128 : 256);  // box rows of the MN-major operands
     if (!make_map(&ma, g.a, g.M, rows_a, kbr)) return cudaErrorInvalidValue;
     if (!make_map(&mb, g.b, g.N, rows_b, kbr)) return cudaErrorInvalidValue;
     const int64_t tiles = (int64_t)g.G * (g.M / BM);
