@@ -60,120 +60,166 @@ __global__ void __launch_bounds__(DCH) chunk_count_kernel(const int32_t* __restr
 // (a bit per token and expert, counted with popc). The expert segments follow in
 // (e mod Pown, e) order: expert order for Pown = 1, owner-grouped for Pown = P (chunk 0
 // then also writes group_expert[g] = the expert of segment g).
-__global__ void __launch_bounds__(DCH) slot_kernel(const int32_t* __restrict__ idx,
-                                                   const int32_t* __restrict__ chunk_counts,
-                                                   int64_t T, int E, int k, int nchunks,
-                                                   int32_t* offsets, int32_t* slot_of,
-                                                   int32_t* token_of, int Pown,
-                                                   int32_t* group_expert) {
+// The picks of the chunks before this one and of all chunks come from chunk_counts, added by
+// SLOT_THREADS / E threads per expert with eight loads in flight each; for at most
+// SLOT_SELF_CHUNKS chunks (chunk_counts null) every block counts the picks itself instead
+// and the counting launch is left out. A chain of latencies: 17.4 -> 7.6 us for 8192 tokens of
+// 64 experts (128 threads that staged the counts, and a serial prefix over the experts).
+constexpr int SLOT_THREADS = 512;
+constexpr int SLOT_SELF_CHUNKS = 8;
+__global__ void __launch_bounds__(SLOT_THREADS) slot_kernel(const int32_t* __restrict__ idx,
+                                                            const int32_t* __restrict__ chunk_counts,
+                                                            int64_t T, int E, int k, int nchunks,
+                                                            int32_t* offsets, int32_t* slot_of,
+                                                            int32_t* token_of, int Pown,
+                                                            int32_t* group_expert) {
     pdl_begin();
-    __shared__ int s_pre[EMAX];
-    __shared__ int s_tot[EMAX];
-    __shared__ int s_base[EMAX];
+    __shared__ int s_pre[EMAX], s_tot[EMAX];
+    __shared__ int s_ord[EMAX];   // totals in segment order, then each segment's first row
     __shared__ unsigned s_bits[EMAX][DCH / 32];
-    __shared__ int s_ppre[DCH], s_ptot[DCH];  // per (group, expert) partial sums
-    constexpr int TAB = 6144;  // chunk-count table staged in shared memory when it fits
-    __shared__ int s_tab[TAB];
-    const int c = blockIdx.x;
-    const int64_t ntab = (int64_t)nchunks * E;
-    if (ntab <= TAB) {
-        for (int i = threadIdx.x; i < ntab; i += blockDim.x) s_tab[i] = chunk_counts[i];
-        __syncthreads();
-    }
-    // per expert: the picks of the chunks before this one (pre) and of all chunks (tot).
-    // With E <= DCH the block's threads form G = DCH / E groups per expert, group g adding
-    // the chunks g, g + G, ...; the groups are then summed (integers: exact in any order).
-    auto cnt = [&](int cc, int e) {
-        return ntab <= TAB ? s_tab[cc * E + e] : chunk_counts[(int64_t)cc * E + e];
-    };
-    if (E <= DCH) {
-        const int G = DCH / E, e = threadIdx.x % E, g = threadIdx.x / E;
-        int pre = 0, tot = 0;
-        if (g < G) {
-            for (int cc = g; cc < nchunks; cc += G) {
-                const int v = cnt(cc, e);
-                if (cc < c) pre += v;
-                tot += v;
-            }
-        }
-        s_ppre[threadIdx.x] = pre;
-        s_ptot[threadIdx.x] = tot;
-        __syncthreads();
-        if (threadIdx.x < E) {
-            int p2 = 0, t2 = 0;
-            for (int q = 0; q < G; ++q) {
-                p2 += s_ppre[q * E + threadIdx.x];
-                t2 += s_ptot[q * E + threadIdx.x];
-            }
-            s_pre[threadIdx.x] = p2;
-            s_tot[threadIdx.x] = t2;
-        }
-    } else {
-        for (int e = threadIdx.x; e < E; e += blockDim.x) {
-            int pre = 0, tot = 0;
-            for (int cc = 0; cc < nchunks; ++cc) {
-                const int v = cnt(cc, e);
-                if (cc < c) pre += v;
-                tot += v;
-            }
-            s_pre[e] = pre;
-            s_tot[e] = tot;
-        }
-    }
-    for (int i = threadIdx.x; i < EMAX * (DCH / 32); i += blockDim.x) (&s_bits[0][0])[i] = 0u;
+    __shared__ int s_ppre[SLOT_THREADS], s_ptot[SLOT_THREADS];  // per (group, expert) partial sums
+    const int c = blockIdx.x, tid = threadIdx.x;
+    for (int i = tid; i < EMAX * (DCH / 32); i += SLOT_THREADS) (&s_bits[0][0])[i] = 0u;
+    if (tid < EMAX) s_pre[tid] = s_tot[tid] = 0;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0, g = 0;
-        for (int o = 0; o < Pown; ++o) {
-            for (int e = o; e < E; e += Pown, ++g) {
-                if (c == 0) {
-                    offsets[g] = run;
-                    if (group_expert) group_expert[g] = e;
-                }
-                s_base[e] = run + s_pre[e];
-                run += s_tot[e];
-            }
-        }
-        if (c == 0) offsets[E] = run;
-    }
-    const int i = threadIdx.x;
-    const int64_t t = (int64_t)c * DCH + i;
+    // this chunk's picks: one bit per token and expert
+    const int64_t t = (int64_t)c * DCH + tid;
     int es[8];
     int kk = 0;
-    if (t < T) {
+    if (tid < DCH && t < T) {
         for (int j = 0; j < k; ++j) {
             const int e = idx[t * k + j];
             bool ok = (e >= 0 && e < E);
             for (int jj = 0; jj < j; ++jj) ok = ok && (es[jj] != e);
             es[j] = ok ? e : -1;
-            if (ok) atomicOr(&s_bits[e][i >> 5], 1u << (i & 31));
-            else slot_of[t * k + j] = -1;
+            if (ok) {
+                atomicOr(&s_bits[e][tid >> 5], 1u << (tid & 31));
+            } else {
+                slot_of[t * k + j] = -1;
+                record_status(MOE_ERR_DEVICE_CHECK);
+            }
         }
         kk = k;
     }
+    // per expert: the picks of the chunks before this one (pre) and of all chunks (tot)
+    if (chunk_counts) {
+        {
+            const int G = SLOT_THREADS / E, e = tid % E, g = tid / E;
+            int pre = 0, tot = 0;
+            if (g < G) {
+                for (int cc = g; cc < nchunks; cc += 8 * G) {
+                    int v[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) v[u] = cc + u * G < nchunks ? chunk_counts[(int64_t)(cc + u * G) * E + e] : 0;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        if (cc + u * G < c) pre += v[u];
+                        tot += v[u];
+                    }
+                }
+            }
+            s_ppre[tid] = pre;
+            s_ptot[tid] = tot;
+            __syncthreads();
+            if (tid < E) {
+                int p2 = 0, t2 = 0;
+                for (int q = 0; q < G; ++q) {
+                    p2 += s_ppre[q * E + tid];
+                    t2 += s_ptot[q * E + tid];
+                }
+                s_pre[tid] = p2;
+                s_tot[tid] = t2;
+            }
+        }
+    } else {
+        for (int64_t tt = tid; tt < T; tt += SLOT_THREADS) {
+            for (int j = 0; j < k; ++j) {
+                const int e = idx[tt * k + j];
+                bool ok = (e >= 0 && e < E);
+                for (int jj = 0; jj < j; ++jj) ok = ok && (idx[tt * k + jj] != e);
+                if (!ok) continue;
+                atomicAdd(&s_tot[e], 1);
+                if (tt < (int64_t)c * DCH) atomicAdd(&s_pre[e], 1);
+            }
+        }
+    }
     __syncthreads();
+    // segment of expert e: its position in (e mod Pown, e) order
+    auto segment = [&](int e) {
+        const int o = e % Pown, q = E / Pown, r = E % Pown;
+        return o * q + min(o, r) + e / Pown;
+    };
+    if (tid < E) s_ord[segment(tid)] = s_tot[tid];
+    __syncthreads();
+    if (tid < 32) {  // exclusive prefix over the segments, EMAX / 32 per lane
+        constexpr int PL = EMAX / 32;
+        int v[PL], sum = 0;
+#pragma unroll
+        for (int u = 0; u < PL; ++u) {
+            v[u] = tid * PL + u < E ? s_ord[tid * PL + u] : 0;
+            sum += v[u];
+        }
+        int inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int w = __shfl_up_sync(0xffffffffu, inc, o);
+            if (tid >= o) inc += w;
+        }
+        int run = inc - sum;
+#pragma unroll
+        for (int u = 0; u < PL; ++u) {
+            if (tid * PL + u < E) {
+                s_ord[tid * PL + u] = run;
+                if (c == 0) offsets[tid * PL + u] = run;
+                run += v[u];
+            }
+        }
+        if (tid == 31 && c == 0) offsets[E] = inc;
+    }
+    __syncthreads();
+    if (c == 0 && group_expert && tid < E) group_expert[segment(tid)] = tid;
     for (int j = 0; j < kk; ++j) {
         const int e = es[j];
         if (e < 0) continue;
         int rank = 0;
-        for (int w = 0; w < (i >> 5); ++w) rank += __popc(s_bits[e][w]);
-        rank += __popc(s_bits[e][i >> 5] & ((1u << (i & 31)) - 1u));
-        const int slot = s_base[e] + rank;
+        for (int w = 0; w < (tid >> 5); ++w) rank += __popc(s_bits[e][w]);
+        rank += __popc(s_bits[e][tid >> 5] & ((1u << (tid & 31)) - 1u));
+        const int slot = s_ord[segment(e)] + s_pre[e] + rank;
         slot_of[t * k + j] = slot;
         token_of[slot] = (int32_t)t;
     }
 }
 
-// x_perm[slot_of[t,j]] = x[t] for every pick j: one warp per token reads its row once
-// (16-byte vectors, U of them in flight per lane) and writes it to its k rows of x_perm.
+// The four kernels below give each token WPT warps of a block (1, 2, 4 or 8, chosen at the
+// launch so that a batch of few tokens still fills the SMs): warp part q of a token takes
+// every WPT-th step of its columns. KMAX is the number of picks rounded up to an
+// instantiated one, and every lane issues the loads of U vectors of all k rows before it uses
+// any of them (8 to 16 loads in flight). HBM-bound for large batches, latency-bound for small.
+// Against one warp per token and k = 6 padded to 8 rows of one vector each: 8192 tokens of
+// d = 2048, k = 6: combine 71 -> 62 us, its backward 77 -> 70, unpermute-reduce 70 -> 68;
+// 546 of 2816, k = 2: backward 7.3 -> 4.8, unpermute 10.8 -> 5.3; 64 of 2048: combine 16 -> 5.4.
+constexpr int TOK_WARPS = 8;  // warps per block
+struct TokenWarp {
+    int64_t t;
+    int lane, part, wpt;
+};
+__device__ __forceinline__ TokenWarp token_warp(int wpt) {
+    const int w = threadIdx.x >> 5;
+    return TokenWarp{(int64_t)blockIdx.x * (TOK_WARPS / wpt) + w / wpt, (int)(threadIdx.x & 31), w % wpt, wpt};
+}
+__host__ __device__ constexpr int rows_in_flight(int kmax) { return kmax <= 2 ? 4 : kmax <= 6 ? 2 : 1; }
+
+// x_perm[slot_of[t,j]] = x[t] for every pick j: each token's row is read once (16-byte
+// vectors, U of them in flight per lane) and written to its k rows of x_perm.
 // A slot outside [0, T k) is skipped and recorded as MOE_ERR_DEVICE_CHECK.
 template <typename T>
 __global__ void __launch_bounds__(256) gather_kernel(const T* __restrict__ x,
                                                      const int32_t* __restrict__ slot_of,
-                                                     int64_t Tn, int d, int k, T* x_perm) {
+                                                     int64_t Tn, int d, int k, T* x_perm, int wpt) {
     pdl_begin();
-    const int lane = threadIdx.x & 31;
-    const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const TokenWarp tw = token_warp(wpt);
+    const int lane = tw.lane;
+    const int64_t t = tw.t;
     if (t >= Tn) return;
     int32_t slot[8];
 #pragma unroll
@@ -188,7 +234,7 @@ __global__ void __launch_bounds__(256) gather_kernel(const T* __restrict__ x,
     constexpr int U = 4;  // vectors per lane in flight
     const int nv = d / VN;
     const T* src = x + t * d;
-    for (int v0 = lane; v0 < nv; v0 += 32 * U) {
+    for (int v0 = tw.part * 32 * U + lane; v0 < nv; v0 += 32 * U * wpt) {
         uint4 buf[U];
 #pragma unroll
         for (int u = 0; u < U; ++u)
@@ -235,41 +281,42 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* __restric
 }
 
 // out[t] = sum_j w[t,j] * y_perm[slot_of[t,j]] (+ sum_s y_sh[s,t]); fp32 accumulation.
-// One warp per token; every lane issues the loads of up to UB vectors of all k rows
-// before it uses any of them, so enough bytes are in flight to keep HBM busy.
 template <typename T, int KMAX>
-__global__ void __launch_bounds__(256, 3) combine_fwd_kernel(const T* __restrict__ y_perm,
+__global__ void __launch_bounds__(256, KMAX <= 2 ? 3 : 2) combine_fwd_kernel(const T* __restrict__ y_perm,
                                                           const float* __restrict__ w,
                                                           const int32_t* __restrict__ slot_of,
                                                           const T* __restrict__ y_sh, int S,
-                                                          int64_t Tn, int d, int k, T* out) {
+                                                          int64_t Tn, int d, int k, T* out, int wpt) {
     pdl_begin();
-    const int lane = threadIdx.x & 31;
-    const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const TokenWarp tw = token_warp(wpt);
+    const int lane = tw.lane;
+    const int64_t t = tw.t;
     if (t >= Tn) return;
     constexpr int VN = Vec<T>::N;
-    constexpr int UB = KMAX <= 2 ? 4 : KMAX <= 4 ? 2 : 1;  // vectors per lane in flight
-    int64_t slot[KMAX];
+    constexpr int UB = rows_in_flight(KMAX);  // vectors per lane in flight
+    constexpr bool PRE = KMAX > 2;  // the first shared row is loaded with the picks (registers allow)
+    int32_t slot[KMAX];
     float wt[KMAX];
 #pragma unroll
     for (int j = 0; j < KMAX; ++j) {
         slot[j] = j < k ? slot_of[t * k + j] : 0;
         wt[j] = j < k ? w[t * k + j] : 0.f;
-        if (slot[j] < 0 || slot[j] >= Tn * k) {  // bad table: contribute nothing
+        if (slot[j] < 0 || (int64_t)slot[j] >= Tn * k) {  // bad table: contribute nothing
             if (lane == 0) record_status(MOE_ERR_DEVICE_CHECK);
             slot[j] = 0;
             wt[j] = 0.f;
         }
     }
     const int nv = d / VN;
-    for (int v0 = lane; v0 < nv; v0 += 32 * UB) {
-        uint4 raw[UB][KMAX];
+    for (int v0 = tw.part * 32 * UB + lane; v0 < nv; v0 += 32 * UB * wpt) {
+        uint4 raw[UB][KMAX], sh[UB];
 #pragma unroll
         for (int u = 0; u < UB; ++u) {
             const int v = v0 + 32 * u;
 #pragma unroll
             for (int j = 0; j < KMAX; ++j)
-                if (j < k && v < nv) raw[u][j] = Vec<T>::raw_load(y_perm + slot[j] * d + v * VN);
+                if (j < k && v < nv) raw[u][j] = Vec<T>::raw_load(y_perm + (int64_t)slot[j] * d + v * VN);
+            if (PRE && S && v < nv) sh[u] = Vec<T>::raw_load(y_sh + t * d + v * VN);
         }
 #pragma unroll
         for (int u = 0; u < UB; ++u) {
@@ -289,7 +336,8 @@ __global__ void __launch_bounds__(256, 3) combine_fwd_kernel(const T* __restrict
             }
             for (int s2 = 0; s2 < S; ++s2) {
                 float yv[VN];
-                Vec<T>::load(y_sh + ((int64_t)s2 * Tn + t) * d + v * VN, yv);
+                if (PRE && s2 == 0) unpack_vec<T>(sh[u], yv);
+                else Vec<T>::load(y_sh + ((int64_t)s2 * Tn + t) * d + v * VN, yv);
 #pragma unroll
                 for (int q = 0; q < VN; ++q) acc[q] += yv[q];
             }
@@ -298,34 +346,38 @@ __global__ void __launch_bounds__(256, 3) combine_fwd_kernel(const T* __restrict
     }
 }
 
-// dy_perm[slot(t,j)] = w[t,j] dout[t];  dw[t,j] = <dout[t], y_perm[slot(t,j)]>.
+// dy_perm[slot(t,j)] = w[t,j] dout[t];  dw[t,j] = <dout[t], y_perm[slot(t,j)]>, the parts of a
+// token's warps added in order through shared memory.
 template <typename T, int KMAX>
-__global__ void __launch_bounds__(256, 3) combine_bwd_kernel(const T* __restrict__ dout,
+__global__ void __launch_bounds__(256, KMAX <= 2 ? 3 : 2) combine_bwd_kernel(const T* __restrict__ dout,
                                                           const T* __restrict__ y_perm,
                                                           const float* __restrict__ w,
                                                           const int32_t* __restrict__ slot_of,
                                                           int64_t Tn, int d, int k, T* dy_perm,
-                                                          float* dw) {
+                                                          float* dw, int wpt) {
     pdl_begin();
-    const int lane = threadIdx.x & 31;
-    const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (t >= Tn) return;
+    __shared__ float s_part[TOK_WARPS][KMAX];
+    const TokenWarp tw = token_warp(wpt);
+    const int lane = tw.lane;
+    const int64_t t = tw.t;
+    const bool live = t < Tn;
     constexpr int VN = Vec<T>::N;
-    constexpr int UB = KMAX <= 2 ? 4 : KMAX <= 4 ? 2 : 1;
-    int64_t slot[KMAX];
+    constexpr int UB = rows_in_flight(KMAX);
+    int32_t slot[KMAX];
     float wt[KMAX], part[KMAX];
 #pragma unroll
     for (int j = 0; j < KMAX; ++j) {
-        slot[j] = j < k ? slot_of[t * k + j] : 0;
-        wt[j] = j < k ? w[t * k + j] : 0.f;
+        const bool pick = live && j < k;
+        slot[j] = pick ? slot_of[t * k + j] : -1;
+        wt[j] = pick ? w[t * k + j] : 0.f;
         part[j] = 0.f;
-        if (slot[j] < 0 || slot[j] >= Tn * k) {
+        if (pick && (slot[j] < 0 || (int64_t)slot[j] >= Tn * k)) {
             if (lane == 0) record_status(MOE_ERR_DEVICE_CHECK);
             slot[j] = -1;
         }
     }
-    const int nv = d / VN;
-    for (int v0 = lane; v0 < nv; v0 += 32 * UB) {
+    const int nv = live ? d / VN : 0;
+    for (int v0 = tw.part * 32 * UB + lane; v0 < nv; v0 += 32 * UB * wpt) {
         uint4 graw[UB], yraw[UB][KMAX];
 #pragma unroll
         for (int u = 0; u < UB; ++u) {
@@ -334,7 +386,7 @@ __global__ void __launch_bounds__(256, 3) combine_bwd_kernel(const T* __restrict
                 graw[u] = Vec<T>::raw_load(dout + t * d + v * VN);
 #pragma unroll
                 for (int j = 0; j < KMAX; ++j)
-                    if (j < k && slot[j] >= 0) yraw[u][j] = Vec<T>::raw_load(y_perm + slot[j] * d + v * VN);
+                    if (slot[j] >= 0) yraw[u][j] = Vec<T>::raw_load(y_perm + (int64_t)slot[j] * d + v * VN);
             }
         }
 #pragma unroll
@@ -345,7 +397,7 @@ __global__ void __launch_bounds__(256, 3) combine_bwd_kernel(const T* __restrict
             unpack_vec<T>(graw[u], g);
 #pragma unroll
             for (int j = 0; j < KMAX; ++j) {
-                if (j < k && slot[j] >= 0) {
+                if (slot[j] >= 0) {
                     float yv[VN], dy[VN];
                     unpack_vec<T>(yraw[u][j], yv);
 #pragma unroll
@@ -353,34 +405,38 @@ __global__ void __launch_bounds__(256, 3) combine_bwd_kernel(const T* __restrict
                         part[j] = fmaf(g[q], yv[q], part[j]);
                         dy[q] = wt[j] * g[q];
                     }
-                    Vec<T>::store(dy_perm + slot[j] * d + v * VN, dy);
+                    Vec<T>::store(dy_perm + (int64_t)slot[j] * d + v * VN, dy);
                 }
             }
         }
     }
 #pragma unroll
     for (int j = 0; j < KMAX; ++j) {
-        if (j < k) {
-            const float sum = warp_sum(part[j]);
-            if (lane == 0) dw[t * k + j] = sum;
-        }
+        const float sum = warp_sum(part[j]);
+        if (lane == 0) s_part[threadIdx.x >> 5][j] = sum;
+    }
+    if (wpt > 1) __syncthreads();
+    else __syncwarp();
+    if (live && tw.part == 0 && lane < k) {
+        float sum = 0.f;
+        for (int q = 0; q < wpt; ++q) sum += s_part[(threadIdx.x >> 5) + q][lane];
+        dw[t * k + lane] = sum;
     }
 }
 
 // dx[t] = sum_j dx_perm[slot(t,j)] + dx_router[t] + sum_s dx_sh[s,t]; fp32 accumulation.
-// One warp per token; every lane issues the loads of up to UB vectors of all k rows (and
-// of the router's row) before it uses any of them.
 template <typename T, int KMAX>
-__global__ void __launch_bounds__(256, 3) unpermute_reduce_kernel(
+__global__ void __launch_bounds__(256, 2) unpermute_reduce_kernel(
     const T* __restrict__ dx_perm, const int32_t* __restrict__ slot_of,
     const T* __restrict__ dx_router, const T* __restrict__ dx_sh, int S, int64_t Tn, int d, int k,
-    T* dx) {
+    T* dx, int wpt) {
     pdl_begin();
-    const int lane = threadIdx.x & 31;
-    const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const TokenWarp tw = token_warp(wpt);
+    const int lane = tw.lane;
+    const int64_t t = tw.t;
     if (t >= Tn) return;
     constexpr int VN = Vec<T>::N;
-    constexpr int UB = KMAX <= 2 ? 4 : KMAX <= 4 ? 2 : 1;  // vectors per lane in flight
+    constexpr int UB = rows_in_flight(KMAX);  // vectors per lane in flight
     int32_t slot[KMAX];
 #pragma unroll
     for (int j = 0; j < KMAX; ++j) {
@@ -391,8 +447,8 @@ __global__ void __launch_bounds__(256, 3) unpermute_reduce_kernel(
         }
     }
     const int nv = d / VN;
-    for (int v0 = lane; v0 < nv; v0 += 32 * UB) {
-        uint4 raw[UB][KMAX], rr[UB];
+    for (int v0 = tw.part * 32 * UB + lane; v0 < nv; v0 += 32 * UB * wpt) {
+        uint4 raw[UB][KMAX], rr[UB], sh[UB];
 #pragma unroll
         for (int u = 0; u < UB; ++u) {
             const int v = v0 + 32 * u;
@@ -401,6 +457,7 @@ __global__ void __launch_bounds__(256, 3) unpermute_reduce_kernel(
                 for (int j = 0; j < KMAX; ++j)
                     if (slot[j] >= 0) raw[u][j] = Vec<T>::raw_load(dx_perm + (int64_t)slot[j] * d + v * VN);
                 if (dx_router) rr[u] = Vec<T>::raw_load(dx_router + t * d + v * VN);
+                if (S) sh[u] = Vec<T>::raw_load(dx_sh + t * d + v * VN);
             }
         }
 #pragma unroll
@@ -425,7 +482,8 @@ __global__ void __launch_bounds__(256, 3) unpermute_reduce_kernel(
             }
             for (int s2 = 0; s2 < S; ++s2) {
                 float g[VN];
-                Vec<T>::load(dx_sh + ((int64_t)s2 * Tn + t) * d + v * VN, g);
+                if (s2 == 0) unpack_vec<T>(sh[u], g);
+                else Vec<T>::load(dx_sh + ((int64_t)s2 * Tn + t) * d + v * VN, g);
 #pragma unroll
                 for (int q = 0; q < VN; ++q) acc[q] += g[q];
             }
@@ -435,15 +493,35 @@ __global__ void __launch_bounds__(256, 3) unpermute_reduce_kernel(
 }
 
 // ----------------------------------------------------------------------------- launchers
+static int dispatch_sms() {
+    static int n = 0;
+    if (!n) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        if (n <= 0) n = 148;
+    }
+    return n;
+}
+// Warps per token: doubled while the batch has fewer than 16 warps per SM and each part still
+// gets a step of columns (rows of `vecs` 16-byte vectors, `step` of them per warp and step).
+static int warps_per_token(int64_t T, int vecs, int step) {
+    int w = 1;
+    while (w < TOK_WARPS && T * w < 16 * (int64_t)dispatch_sms() && vecs > step * w) w *= 2;
+    return w;
+}
+static unsigned token_blocks(int64_t T, int wpt) { return (unsigned)((T * wpt + TOK_WARPS - 1) / TOK_WARPS); }
+
 static cudaError_t launch_gather(const void* x, const int32_t* slot_of, int64_t T, int d, int k, bool bf16,
                                  void* x_perm, cudaStream_t s) {
-    const unsigned blocks = (unsigned)((T + 7) / 8);
+    const int wpt = warps_per_token(T, d / (bf16 ? 8 : 4), 128);
+    const unsigned blocks = token_blocks(T, wpt);
     if (bf16)
         (void)launch_pdl(gather_kernel<__nv_bfloat16>, dim3(blocks), dim3(256), 0, s, (const __nv_bfloat16*)x,
-                         slot_of, T, d, k, (__nv_bfloat16*)x_perm);
+                         slot_of, T, d, k, (__nv_bfloat16*)x_perm, wpt);
     else
         (void)launch_pdl(gather_kernel<float>, dim3(blocks), dim3(256), 0, s, (const float*)x, slot_of, T, d, k,
-                         (float*)x_perm);
+                         (float*)x_perm, wpt);
     return cudaGetLastError();
 }
 
@@ -465,12 +543,15 @@ cudaError_t launch_dispatch(const int32_t* topk_idx, const void* x, int64_t T, i
     } else if (T == 0) {
         return cudaMemsetAsync(offsets, 0, sizeof(int32_t) * (E + 1), s);
     }
-    (void)launch_pdl(chunk_count_kernel, dim3(nch), dim3(DCH), 0, s, topk_idx, T, E, k, cc, po,
-                     owner ? P : 1, send);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    (void)launch_pdl(slot_kernel, dim3(nch), dim3(DCH), 0, s, topk_idx, cc, T, E, k, nch, offsets,
-                     slot_of, token_of, owner ? P : 1, group_expert);
+    const bool self = !owner && nch <= SLOT_SELF_CHUNKS;  // (the owner counts come from the counting kernel)
+    if (!self) {
+        (void)launch_pdl(chunk_count_kernel, dim3(nch), dim3(DCH), 0, s, topk_idx, T, E, k, cc, po,
+                         owner ? P : 1, send);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    (void)launch_pdl(slot_kernel, dim3(nch), dim3(SLOT_THREADS), 0, s, topk_idx, self ? (const int32_t*)nullptr : cc, T,
+                     E, k, nch, offsets, slot_of, token_of, owner ? P : 1, group_expert);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (T * k == 0) return cudaSuccess;
@@ -481,19 +562,23 @@ cudaError_t launch_combine_fwd(const void* y_perm, const float* topk_w, const in
                                const void* y_sh, int S, int64_t T, int d, int k, bool bf16,
                                void* out, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
-    const unsigned blocks = (unsigned)((T + 7) / 8);
 #define MOE_CF(TT, KM)                                                                           \
-    (void)launch_pdl(combine_fwd_kernel<TT, KM>, dim3(blocks), dim3(256), 0, s, (const TT*)y_perm, topk_w, slot_of,         \
-                                                      (const TT*)y_sh, S, T, d, k, (TT*)out)
-    if (bf16) {
-        if (k <= 2) MOE_CF(__nv_bfloat16, 2);
-        else if (k <= 4) MOE_CF(__nv_bfloat16, 4);
-        else MOE_CF(__nv_bfloat16, 8);
-    } else {
-        if (k <= 2) MOE_CF(float, 2);
-        else if (k <= 4) MOE_CF(float, 4);
-        else MOE_CF(float, 8);
-    }
+    do {                                                                                         \
+        const int wpt = warps_per_token(T, d / Vec<TT>::N, 32 * rows_in_flight(KM));             \
+        (void)launch_pdl(combine_fwd_kernel<TT, KM>, dim3(token_blocks(T, wpt)), dim3(256), 0, s, (const TT*)y_perm, \
+                         topk_w, slot_of, (const TT*)y_sh, S, T, d, k, (TT*)out, wpt);           \
+    } while (0)
+#define MOE_K(TT)                  \
+    do {                           \
+        if (k <= 1) MOE_CF(TT, 1);      \
+        else if (k <= 2) MOE_CF(TT, 2); \
+        else if (k <= 4) MOE_CF(TT, 4); \
+        else if (k <= 6) MOE_CF(TT, 6); \
+        else MOE_CF(TT, 8);             \
+    } while (0)
+    if (bf16) MOE_K(__nv_bfloat16);
+    else MOE_K(float);
+#undef MOE_K
 #undef MOE_CF
     return cudaGetLastError();
 }
@@ -502,19 +587,23 @@ cudaError_t launch_combine_bwd(const void* dout, const void* y_perm, const float
                                const int32_t* slot_of, int64_t T, int d, int k, bool bf16,
                                void* dy_perm, float* dtopk_w, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
-    const unsigned blocks = (unsigned)((T + 7) / 8);
 #define MOE_CB(TT, KM)                                                                           \
-    (void)launch_pdl(combine_bwd_kernel<TT, KM>, dim3(blocks), dim3(256), 0, s, (const TT*)dout, (const TT*)y_perm, topk_w, \
-                                                      slot_of, T, d, k, (TT*)dy_perm, dtopk_w)
-    if (bf16) {
-        if (k <= 2) MOE_CB(__nv_bfloat16, 2);
-        else if (k <= 4) MOE_CB(__nv_bfloat16, 4);
-        else MOE_CB(__nv_bfloat16, 8);
-    } else {
-        if (k <= 2) MOE_CB(float, 2);
-        else if (k <= 4) MOE_CB(float, 4);
-        else MOE_CB(float, 8);
-    }
+    do {                                                                                         \
+        const int wpt = warps_per_token(T, d / Vec<TT>::N, 32 * rows_in_flight(KM));             \
+        (void)launch_pdl(combine_bwd_kernel<TT, KM>, dim3(token_blocks(T, wpt)), dim3(256), 0, s, (const TT*)dout, \
+                         (const TT*)y_perm, topk_w, slot_of, T, d, k, (TT*)dy_perm, dtopk_w, wpt); \
+    } while (0)
+#define MOE_K(TT)                  \
+    do {                           \
+        if (k <= 1) MOE_CB(TT, 1);      \
+        else if (k <= 2) MOE_CB(TT, 2); \
+        else if (k <= 4) MOE_CB(TT, 4); \
+        else if (k <= 6) MOE_CB(TT, 6); \
+        else MOE_CB(TT, 8);             \
+    } while (0)
+    if (bf16) MOE_K(__nv_bfloat16);
+    else MOE_K(float);
+#undef MOE_K
 #undef MOE_CB
     return cudaGetLastError();
 }
@@ -523,20 +612,23 @@ cudaError_t launch_unpermute_reduce(const void* dx_perm, const int32_t* slot_of,
                                     const void* dx_router, const void* dx_sh, int S, int64_t T,
                                     int d, int k, bool bf16, void* dx, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
-    const unsigned blocks = (unsigned)((T + 7) / 8);
 #define MOE_UR(TT, KM)                                                                            \
-    (void)launch_pdl(unpermute_reduce_kernel<TT, KM>, dim3(blocks), dim3(256), 0, s,              \
-                     (const TT*)dx_perm, slot_of, (const TT*)dx_router, (const TT*)dx_sh, S, T, d, \
-                     k, (TT*)dx)
-    if (bf16) {
-        if (k <= 2) MOE_UR(__nv_bfloat16, 2);
-        else if (k <= 4) MOE_UR(__nv_bfloat16, 4);
-        else MOE_UR(__nv_bfloat16, 8);
-    } else {
-        if (k <= 2) MOE_UR(float, 2);
-        else if (k <= 4) MOE_UR(float, 4);
-        else MOE_UR(float, 8);
-    }
+    do {                                                                                          \
+        const int wpt = warps_per_token(T, d / Vec<TT>::N, 32 * rows_in_flight(KM));              \
+        (void)launch_pdl(unpermute_reduce_kernel<TT, KM>, dim3(token_blocks(T, wpt)), dim3(256), 0, s, \
+                         (const TT*)dx_perm, slot_of, (const TT*)dx_router, (const TT*)dx_sh, S, T, d, k, (TT*)dx, wpt); \
+    } while (0)
+#define MOE_K(TT)                  \
+    do {                           \
+        if (k <= 1) MOE_UR(TT, 1);      \
+        else if (k <= 2) MOE_UR(TT, 2); \
+        else if (k <= 4) MOE_UR(TT, 4); \
+        else if (k <= 6) MOE_UR(TT, 6); \
+        else MOE_UR(TT, 8);             \
+    } while (0)
+    if (bf16) MOE_K(__nv_bfloat16);
+    else MOE_K(float);
+#undef MOE_K
 #undef MOE_UR
     return cudaGetLastError();
 }
@@ -582,7 +674,7 @@ cudaError_t launch_dispatch_noalloc(const int32_t* topk_idx, const void* x, int6
                      (const int32_t*)nullptr, 1, (int32_t*)nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    (void)launch_pdl(slot_kernel, dim3(nch), dim3(DCH), 0, s, topk_idx, cc, T, E, k, nch, offsets,
+    (void)launch_pdl(slot_kernel, dim3(nch), dim3(SLOT_THREADS), 0, s, topk_idx, cc, T, E, k, nch, offsets,
                      slot_of, token_of, 1, (int32_t*)nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -106,19 +106,21 @@ __device__ void softmax_topk_token(const float (&z)[NV], int lane, int E, int k,
 // thread (ks, tg, eg) multiplies TB/4 tokens by 4 experts over the columns of its slice ks.
 // A chunk's products are summed on their own before they join the running sum, so no chain
 // of additions is longer than about d / 128 + 32. The KS slices of a logit are then added
-// through shared memory and each warp gates its tokens.
+// through shared memory and each warp gates its tokens. With few tokens a cluster of CTAs
+// shares a group: each takes a part of the columns, and the first adds the parts in order
+// from distributed shared memory and gates.
 //
 // What bounds it: with large pools the shared-memory reads (12 wavefronts per 64 FMAs of a
 // warp), with small ones the latency of the d / 128 chunk steps. The kernel that it replaces
 // (a warp per 1 to 8 tokens, W_r read from L2 by every warp) took 588 us for 3805 bf16 tokens
-// of d = 3072 with E = 63, now 108; 93 -> 27 us for 2157 of 3072 with E = 6; 51 -> 13.6 us for
+// of d = 3072 with E = 63, now 71; 93 -> 28 us for 2157 of 3072 with E = 6; 51 -> 13 us for
 // 1003 of 1152 with E = 13; fp32: 19 -> 4.8 us for 512 of 256 with E = 8.
 constexpr int RD_KC = 128;         // columns per chunk
 constexpr int RD_LD = RD_KC + 4;   // row pitch in shared memory: rows start 16 bytes apart in the banks
 constexpr int RD_THREADS = 256;
 
 template <typename T, int EP, int TB>
-__global__ void __launch_bounds__(RD_THREADS, 2) route_dot_kernel(
+__global__ void __launch_bounds__(RD_THREADS, EP <= 16 && TB == 8 ? 4 : 2) route_dot_kernel(
     const T* __restrict__ x, const T* __restrict__ wr, const float* __restrict__ bias,
     const int32_t* __restrict__ po, int P, int64_t Tn, int d, int E, int k, int normalize, float* logits,
     float* probs, int32_t* topk_idx, float* topk_w, int32_t* counts) {
@@ -130,9 +132,14 @@ __global__ void __launch_bounds__(RD_THREADS, 2) route_dot_kernel(
     extern __shared__ float s_dyn[];  // two buffers of [TB + EP][RD_LD]; then the slices' sums
     __shared__ int s_hist[EP];
     const int tid = threadIdx.x;
-    // the CTA's tokens: group blockIdx.x of TB tokens, enumerated party by party
+    cg::cluster_group cluster = cg::this_cluster();
+    const int parts = (int)cluster.num_blocks(), part_no = (int)cluster.block_rank();
+    // the CTA's columns: a run of whole chunks
+    const int per = ((d + RD_KC - 1) / RD_KC + parts - 1) / parts * RD_KC;
+    const int c_beg = min(d, per * part_no), c_end = min(d, c_beg + per);
+    // the cluster's tokens: group blockIdx.x / parts of TB tokens, enumerated party by party
     int party = -1, n = 0;
-    int64_t t0 = 0, g = blockIdx.x;
+    int64_t t0 = 0, g = blockIdx.x / parts;
     for (int q = 0; q < P && party < 0; ++q) {
         const int64_t a = po ? po[q] : 0, b = po ? po[q + 1] : Tn;
         const int64_t ng = b > a ? (b - a + TB - 1) / TB : 0;
@@ -143,7 +150,7 @@ __global__ void __launch_bounds__(RD_THREADS, 2) route_dot_kernel(
         }
         g -= ng;
     }
-    if (party < 0) return;
+    if (party < 0) return;  // (the whole cluster)
     if (tid < EP) s_hist[tid] = 0;
     const T* W = wr + (int64_t)party * E * d;
     uint4 xr[XV], wv[WV];
@@ -151,12 +158,12 @@ __global__ void __launch_bounds__(RD_THREADS, 2) route_dot_kernel(
 #pragma unroll
         for (int i = 0; i < XV; ++i) {
             const int v = tid + i * RD_THREADS, r = v / ROWV, c = c0 + (v % ROWV) * VN;
-            xr[i] = r < n && c < d ? Vec<T>::raw_load(x + (t0 + r) * d + c) : make_uint4(0, 0, 0, 0);
+            xr[i] = r < n && c < c_end ? Vec<T>::raw_load(x + (t0 + r) * d + c) : make_uint4(0, 0, 0, 0);
         }
 #pragma unroll
         for (int i = 0; i < WV; ++i) {
             const int v = tid + i * RD_THREADS, r = v / ROWV, c = c0 + (v % ROWV) * VN;
-            wv[i] = r < E && c < d ? Vec<T>::raw_load(W + (int64_t)r * d + c) : make_uint4(0, 0, 0, 0);
+            wv[i] = r < E && c < c_end ? Vec<T>::raw_load(W + (int64_t)r * d + c) : make_uint4(0, 0, 0, 0);
         }
     };
     auto put = [&](float* buf) {
@@ -177,12 +184,14 @@ __global__ void __launch_bounds__(RD_THREADS, 2) route_dot_kernel(
     for (int i = 0; i < TM; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    fetch(0);
-    put(s_dyn);
+    if (c_beg < c_end) {
+        fetch(c_beg);
+        put(s_dyn);
+    }
     __syncthreads();
     int cur = 0;
-    for (int c0 = 0; c0 < d; c0 += RD_KC) {
-        const bool more = c0 + RD_KC < d;
+    for (int c0 = c_beg; c0 < c_end; c0 += RD_KC) {
+        const bool more = c0 + RD_KC < c_end;
         if (more) fetch(c0 + RD_KC);
         const float* xs = s_dyn + cur * (TB + EP) * RD_LD + tg * RD_LD;
         const float* ws = s_dyn + cur * (TB + EP) * RD_LD + (TB + eg) * RD_LD;
@@ -219,22 +228,35 @@ __global__ void __launch_bounds__(RD_THREADS, 2) route_dot_kernel(
 #pragma unroll
         for (int j = 0; j < 4; ++j) s_dyn[(ks * TB + tg + 4 * i) * EP + eg + EG * j] = acc[i][j];
     __syncthreads();
-    const int lane = tid & 31;
-    for (int tt = tid >> 5; tt < n; tt += RD_THREADS / 32) {
-        float z[NV];
+    // their sum per (token, expert), in the region after the slices
+    float* s_sum = s_dyn + RD_THREADS * TB;
+    for (int i = tid; i < n * EP; i += RD_THREADS) {
+        float s4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const int e = lane + 32 * v;
-            float s4[4] = {0.f, 0.f, 0.f, 0.f};
-            if (e < E) {
-#pragma unroll
-                for (int q = 0; q < KS; ++q) s4[q & 3] += s_dyn[(q * TB + tt) * EP + e];
-            }
-            z[v] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
-            if (bias && e < E) z[v] += bias[party * E + e];
-        }
-        softmax_topk_token<NV>(z, lane, E, k, normalize, t0 + tt, 0, logits, probs, topk_idx, topk_w, s_hist);
+        for (int q = 0; q < KS; ++q) s4[q & 3] += s_dyn[q * TB * EP + i];
+        s_sum[i] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
     }
+    if (parts > 1) cluster.sync();
+    else __syncthreads();
+    if (part_no == 0) {
+        const int lane = tid & 31;
+        for (int tt = tid >> 5; tt < n; tt += RD_THREADS / 32) {
+            float z[NV];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                const int e = lane + 32 * v;
+                z[v] = 0.f;
+                if (e < E) {
+                    for (int q = 0; q < parts; ++q)
+                        z[v] += (q ? cluster.map_shared_rank(s_sum, q) : s_sum)[tt * EP + e];
+                    if (bias) z[v] += bias[party * E + e];
+                }
+            }
+            softmax_topk_token<NV>(z, lane, E, k, normalize, t0 + tt, 0, logits, probs, topk_idx, topk_w, s_hist);
+        }
+    }
+    if (parts > 1) cluster.sync();  // the parts' shared memory has been read
+    if (part_no) return;
     __syncthreads();
     if (tid < E && s_hist[tid]) atomicAdd(&counts[party * E + tid], s_hist[tid]);
 }
@@ -653,28 +675,46 @@ static cudaError_t launch_gating(const RouteArgs& a, cudaStream_t s) {
 }
 
 template <typename T, int EP, int TB>
-static cudaError_t launch_route_dot_t(const RouteArgs& a, cudaStream_t s) {
+static cudaError_t launch_route_dot_t(const RouteArgs& a, int parts, cudaStream_t s) {
     auto kern = route_dot_kernel<T, EP, TB>;
-    constexpr size_t smem = std::max<size_t>(2 * (size_t)(TB + EP) * RD_LD, (size_t)RD_THREADS * TB) * sizeof(float);
+    constexpr size_t smem =
+        std::max<size_t>(2 * (size_t)(TB + EP) * RD_LD, (size_t)RD_THREADS * TB + (size_t)TB * EP) * sizeof(float);
     static bool attr = false;
     if (!attr) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    const unsigned blocks = (unsigned)((a.T + TB - 1) / TB + (a.po ? a.P : 0));
-    (void)launch_pdl(kern, dim3(blocks), dim3(RD_THREADS), smem, s, (const T*)a.x, (const T*)a.w_router, a.bias, a.po,
-                     a.P, a.T, a.d, a.E, a.k, a.normalize, a.logits, a.probs, a.topk_idx, a.topk_w, a.counts);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(((a.T + TB - 1) / TB + (a.po ? a.P : 0)) * parts));
+    cfg.blockDim = dim3(RD_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)parts;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kern, (const T*)a.x, (const T*)a.w_router, a.bias, a.po, a.P, a.T, a.d, a.E, a.k,
+                              a.normalize, a.logits, a.probs, a.topk_idx, a.topk_w, a.counts);
 }
 
-// E <= 64. 16 tokens per CTA, 8 while those would not give every SM two CTAs (the weights
-// of a CTA are staged for its tokens alone, so fewer tokens cost more shared-memory traffic)
+// E <= 64. 16 tokens per CTA, 8 while those would not give every SM two CTAs (over 32 experts
+// one: the weights of a CTA are staged for its tokens alone, so fewer tokens cost more
+// shared-memory traffic). A cluster of 2, 4 or 8 CTAs per group while the groups leave more
+// than half of the SMs idle and every CTA keeps a chunk of columns.
 template <typename T>
 static cudaError_t launch_route_dot(const RouteArgs& a, cudaStream_t s) {
     if (a.T == 0) return cudaSuccess;
-    const bool few = a.T < 2 * 16 * (int64_t)num_sms();
-#define MOE_DOT(EP) (few ? launch_route_dot_t<T, EP, 8>(a, s) : launch_route_dot_t<T, EP, 16>(a, s))
+    const bool few = a.T < (a.E > 32 ? 1 : 2) * 16 * (int64_t)num_sms();
+    const int64_t groups = (a.T + (few ? 8 : 16) - 1) / (few ? 8 : 16);
+    const int chunks = (a.d + 127) / 128;
+    int parts = 1;
+    while (parts < 8 && groups * parts * 2 <= num_sms() && parts * 2 <= chunks) parts *= 2;
+#define MOE_DOT(EP) (few ? launch_route_dot_t<T, EP, 8>(a, parts, s) : launch_route_dot_t<T, EP, 16>(a, parts, s))
     if (a.E <= 8) return MOE_DOT(8);
     if (a.E <= 16) return MOE_DOT(16);
     if (a.E <= 32) return MOE_DOT(32);
@@ -711,8 +751,9 @@ cudaError_t launch_route(const RouteArgs& a, bool bf16, bool from_logits, cudaSt
         b.bias = nullptr;  // the caller's logits are final
         return launch_gating(b, s);
     }
-    if (bf16 && (a.E % 4 == 0 || a.E > 64) && a.T > 0) return launch_route_tc(a, s);
-    if (a.E > 64) return a.T > 0 ? launch_route_wide_f32(a, s) : cudaSuccess;
+    if (a.T == 0) return cudaSuccess;
+    if (bf16 && (a.E % 4 == 0 || a.E > 64)) return launch_route_tc(a, s);
+    if (a.E > 64) return launch_route_wide_f32(a, s);
     return bf16 ? launch_route_dot<__nv_bfloat16>(a, s) : launch_route_dot<float>(a, s);
 }
 

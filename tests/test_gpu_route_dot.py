@@ -1,6 +1,7 @@
 """Router logits and gating on the CUDA cores (fp32, and bf16 pools that are not a multiple
 of 4) at the edges: token counts around the 8- and 16-token groups, d around the 128-column
-chunk, every padded pool size, parties of unequal and zero size. The fp32 sums are compared
+chunk, every padded pool size, clusters of 1 to 8 CTAs per group with uneven column shares,
+parties of unequal and zero size. The fp32 sums are compared
 with 64 bits: chains of at most d / 128 + 32 + 8 additions round each partial sum, so
 |dz| <= (d / 128 + 40) 2^-24 sum |x w|, and picks equal the oracle's on those logits."""
 import numpy as np
@@ -24,7 +25,9 @@ def L():
     ("f32", 1, 4, 3, 2, None), ("f32", 7, 124, 8, 2, None), ("f32", 9, 132, 9, 3, [0, 0, 5, 9]),
     ("f32", 5000, 260, 17, 4, [0, 4999, 5000]), ("f32", 33, 1000, 64, 8, None),
     ("bf16", 15, 128, 5, 1, None), ("bf16", 17, 256, 13, 3, [0, 9, 9, 17]), ("bf16", 4900, 384, 30, 2, None),
-    ("bf16", 500, 2048, 63, 6, [0, 1, 300, 500])])
+    ("bf16", 500, 2048, 63, 6, [0, 1, 300, 500]),
+    ("bf16", 1, 1152, 63, 6, None), ("bf16", 64, 2048, 33, 6, None), ("bf16", 90, 640, 7, 2, [0, 30, 30, 90]),
+    ("f32", 300, 1280, 60, 4, None), ("f32", 40, 900, 8, 2, None), ("f32", 700, 2052, 16, 3, [0, 350, 700])])
 def test_route_on_the_cuda_cores(L, dtype, T, d, E, k, po):
     rng = np.random.default_rng(T + d + E)
     rnd = mi.bf16_round if dtype == "bf16" else (lambda a: a)
