@@ -10,12 +10,12 @@
 // loses more than an FFMA chain does, so an accumulator holds only 32 contraction terms
 // (the smallest products first) and is then added to fp32 registers with round-to-nearest.
 // Measured against 64 bits, the worst tensor of a whole fp32 step is 2.4e-7 (512 tokens,
-// d = 256, F = 512) and 5.7e-7 (1501 tokens, d = 1000, F = 1366) off; the FFMA kernels that
+// d = 256, F = 512) and 5e-7 (1501 tokens, d = 1000, F = 1366) off; the FFMA kernels that
 // this replaces were 7.1e-7 and 1.5e-6 off, and accumulators of 64 terms (1.5% faster)
 // 8.3e-7 and 1.1e-6.
 //
 // Roles (one persistent CTA per SM, 128 x BN tiles): 16 producer warps copy fp32 into
-// shared memory up to three stages ahead (cp.async), split it and write three swizzled bf16
+// shared memory up to two stages ahead (cp.async), split it and write three swizzled bf16
 // planes per operand into a ring of two 32-deep stages; one warp issues the 12 MMAs of a
 // stage into one of four TMEM accumulators; 8 warps add the accumulators into registers and
 // run the epilogue. cp.async and not TMA because lines need only 4-byte alignment (any d_ff).
@@ -24,8 +24,8 @@
 // fp32 written and read, 48 KB of planes written, and 96 KB of operand reads by the MMAs;
 // the counters show the LSU pipe at 41% and the tensor pipe's reads at 47% (accumulating an
 // eighth as often, or issuing one MMA of six, changed the time by 10% and 4%). Whole fp32 steps:
-// 1501 tokens, d = 1000, F = 1366, E = 6, k = 3: 5.44 -> 1.35 ms (20 -> 82 TFLOP/s);
-// 512 tokens, d = 256, F = 512, E = 8, k = 2: 494 -> 177 us.
+// 1501 tokens, d = 1000, F = 1366, E = 6, k = 3: 5.39 -> 1.13 ms (21 -> 98 TFLOP/s);
+// 512 tokens, d = 256, F = 512, E = 8, k = 2: 493 -> 133 us.
 //
 // An infinite or NaN operand makes 0 * inf terms in the split, so an output element that is
 // not finite is computed again by a plain fp32 FMA chain, which gives IEEE results.
@@ -74,7 +74,7 @@ constexpr uint32_t plane_a() { return BM * FK * 2; }
 constexpr uint32_t plane_b(int bn) { return (uint32_t)bn * FK * 2; }
 constexpr uint32_t stage_bytes(int bn) { return 3 * (plane_a() + plane_b(bn)); }
 constexpr int NST = 2;                // bf16 stages (the MMAs of one, the split into the other)
-constexpr int NRAW = 3;               // fp32 stages: copies in flight ahead of the split
+constexpr int NRAW = 2;               // fp32 stages: copies in flight ahead of the split (three: no faster)
 constexpr uint32_t raw_bytes() { return PROD_WARPS * 2048; }  // a block of each operand per warp
 constexpr uint32_t smem_bytes(int bn) {
     return 1024 + NST * stage_bytes(bn) + NRAW * raw_bytes() + EPI_W * ST_FLOATS * 4;
@@ -266,6 +266,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
         const int oa = lane / per_a, ia = (lane % per_a) * p.vec_a, ob = lane / per_b, ib = (lane % per_b) * p.vec_b;
         int t = (int)blockIdx.x - (int)gridDim.x, left = 0;
         const float *src_a = nullptr, *src_b = nullptr;  // this lane's first element of the block
+        bool has_rows = false, has_cols = false;  // whether this warp's blocks of the tile hold anything
         int lim_a = 0, lim_b = 0;  // outer lines with data past the lane's (K-contiguous), or whether the column has any
         auto seek = [&]() -> bool {  // the next stage: of this tile, or of the next one with work
             if ((left -= FK) > 0) {
@@ -277,6 +278,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
                 const Tile ti = tile_at(t);
                 left = ti.klen;
                 if (left <= 0) continue;
+                has_rows = ti.m0 + arow < ti.mrows;
                 const int ra = ti.m0 + arow + (A_MN ? ia : oa);
                 lim_a = A_MN ? (ra < ti.mrows ? 1 : 0) : ti.mrows - ra;
                 src_a = a_base(ti) + (A_MN ? (ak + oa) * lda + ra : ra * lda + ia);
@@ -285,6 +287,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
                     const int rb = b_row(ti, c), end = EPI == EPI_SWIGLU_FWD ? (c < BN / 2 ? F : 2 * F) : p.N;
                     lim_b = B_MN ? (rb < end ? 1 : 0) : end - rb;
                     src_b = b_base(ti) + (B_MN ? (bk + ob) * ldb + rb : rb * ldb + ib);
+                    has_cols = b_row(ti, brow) < end;
                 }
                 return true;
             }
@@ -311,8 +314,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
         };
         auto issue = [&](int slot) {
             const uint32_t dst = raw + slot * raw_bytes();
-            copy_op(std::integral_constant<bool, A_MN>{}, p.vec_a, src_a, lda, oa, ia, ak, lim_a, dst);
-            if (has_b) copy_op(std::integral_constant<bool, B_MN>{}, p.vec_b, src_b, ldb, ob, ib, bk, lim_b, dst + 1024);
+            if (has_rows) copy_op(std::integral_constant<bool, A_MN>{}, p.vec_a, src_a, lda, oa, ia, ak, lim_a, dst);
+            if (has_cols) copy_op(std::integral_constant<bool, B_MN>{}, p.vec_b, src_b, ldb, ob, ib, bk, lim_b, dst + 1024);
         };
         // split one landed block into the three planes at d
         auto split_block = [&](auto mnc, const uint8_t* q, uint8_t* d, uint32_t plane) {
@@ -338,11 +341,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
         bool more = seek();
         int slot_in = 0, slot = 0, ahead = 0;  // stages copied and not yet split
         uint32_t phase = 0;
+        uint32_t held = 0;  // two bits per slot: has_rows, has_cols of the stage in it
         int stage = 0;
         for (;;) {
             while (more && ahead < NRAW) {
                 issue(slot_in);
                 cp_commit();
+                held = (held & ~(3u << (2 * slot_in))) | ((uint32_t)has_rows | ((uint32_t)has_cols << 1)) << (2 * slot_in);
                 slot_in = slot_in + 1 == NRAW ? 0 : slot_in + 1;
                 ++ahead;
                 more = seek();
@@ -354,8 +359,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
             if (!wait(empty_bar(stage), phase ^ 1u)) break;
             uint8_t* sa = ring_ptr + (size_t)stage * STAGE;
             const uint8_t* rp = raw_ptr + slot * raw_bytes();
-            split_block(std::integral_constant<bool, A_MN>{}, rp, sa + da, plane_a());
-            if (has_b) split_block(std::integral_constant<bool, B_MN>{}, rp + 1024, sa + db, plane_b(BN));
+            // (blocks past the operand's rows stay as they are: their accumulators are not stored)
+            if ((held >> (2 * slot)) & 1u) split_block(std::integral_constant<bool, A_MN>{}, rp, sa + da, plane_a());
+            if ((held >> (2 * slot)) & 2u) split_block(std::integral_constant<bool, B_MN>{}, rp + 1024, sa + db, plane_b(BN));
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(full_bar(stage));
@@ -453,12 +459,18 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
             // along the columns, so that loads and stores are coalesced
             auto put = [&](int at, float v) { st[lane * 32 + (at ^ lane)] = v; };
             auto get = [&](int r, int at) { return st[r * 32 + (at ^ r)]; };
-            auto redo = [&](float v, int m, int n) -> float {
-                if (fabsf(v) <= 3.402823466e38f) return v;
+            auto finite = [](float v) { return fabsf(v) <= 3.402823466e38f; };
+            auto redo = [&](int m, int n) -> float {
                 const float* A = a_base(ti) + (A_MN ? (int64_t)m : (int64_t)m * p.K);
                 const float* B = b_base(ti) + (B_MN ? (int64_t)n : (int64_t)n * p.K);
                 return dot_plain(A, A_MN ? p.M : 1, B, B_MN ? p.N : 1, ti.klen);
             };
+            // Eight rows at a time, so that their loads and stores overlap and one vote covers
+            // the check for non-finite values. (Row by row, with the check's branch at every
+            // element, a tile's epilogue took 8 us: the weight gradients of experts with few
+            // rows are all epilogue, dW2 of 78 experts of d = 1928, F = 591 at 10 rows took
+            // 362 us, now 173; dA waited for G and U row by row, 4503 rows of d = 1000,
+            // F = 1366 258 -> 163 us.)
             const int mrow = ti.m0 + q * 32;
             if constexpr (EPI == EPI_SWIGLU_FWD) {
                 // 16 gate columns beside the 16 up columns of the same features; a half-warp per row
@@ -472,15 +484,39 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
                     }
                     __syncwarp();
                     const int c = lane & 15, f = ti.n0 + hc * CW + c0 + c;
-#pragma unroll 4
-                    for (int i = 0; i < 16; ++i) {
-                        const int r = 2 * i + (lane >> 4), m = mrow + r;
-                        if (f >= F || m >= ti.mrows) continue;
-                        const float G = redo(get(r, c), m, f), U = redo(get(r, 16 + c), m, F + f);
-                        const int64_t row = ti.o0 + m;
-                        p.out0[row * 2 * F + f] = G;
-                        p.out0[row * 2 * F + F + f] = U;
-                        p.out1[row * F + f] = G * sigmoidf_(G) * U;
+#pragma unroll 1
+                    for (int i0 = 0; i0 < 16; i0 += 8) {
+                        const int m0 = mrow + 2 * i0 + (lane >> 4);  // rows m0, m0 + 2, ...
+                        float G[8], U[8];
+                        bool ok8 = true;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int r = 2 * (i0 + i) + (lane >> 4);
+                            G[i] = get(r, c);
+                            U[i] = get(r, 16 + c);
+                            ok8 = ok8 && finite(G[i]) && finite(U[i]);
+                        }
+                        if (!__all_sync(0xffffffffu, ok8)) {
+                            for (int i = 0; i < 8; ++i) {
+                                const int m = m0 + 2 * i;
+                                if (f >= F || m >= ti.mrows) continue;
+#pragma unroll
+                                for (int u = 0; u < 8; ++u) {
+                                    if (u == i && !finite(G[u])) G[u] = redo(m, f);
+                                    if (u == i && !finite(U[u])) U[u] = redo(m, F + f);
+                                }
+                            }
+                        }
+                        if (f >= F) continue;
+                        float* h = p.out0 + (ti.o0 + m0) * 2 * F + f;
+                        float* o = p.out1 + (ti.o0 + m0) * F + f;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            if (m0 + 2 * i >= ti.mrows) break;
+                            h[(int64_t)i * 4 * F] = G[i];
+                            h[(int64_t)i * 4 * F + F] = U[i];
+                            o[(int64_t)i * 2 * F] = G[i] * sigmoidf_(G[i]) * U[i];
+                        }
                     }
                 }
             } else {
@@ -492,20 +528,48 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
                     for (int i = 0; i < 32; ++i) put(i, CW == 32 ? acc[u][i % CW] : acc[i / CW][i % CW]);
                     __syncwarp();
                     const int n = ti.n0 + hc * CW + (CW == 32 ? u * (BN / 2) + lane : (lane >> 4) * (BN / 2) + (lane & 15));
-#pragma unroll 4
-                    for (int r = 0; r < 32; ++r) {
-                        const int m = mrow + r;
-                        if (n >= p.N || m >= ti.mrows) continue;
-                        const float v = redo(get(r, lane), m, n);
+                    const int64_t row0 = (VAR_K ? (int64_t)ti.we * p.M : ti.o0) + mrow;
+#pragma unroll 1
+                    for (int r0 = 0; r0 < 32 && mrow + r0 < ti.mrows; r0 += 8) {
+                        const int rows = n < p.N ? min(8, ti.mrows - mrow - r0) : 0;
+                        float v[8], G[8], U[8];
                         if constexpr (EPI == EPI_SWIGLU_BWD) {  // v = dA[row, n], N = F
-                            const int64_t row = (ti.o0 + m) * 2 * F;
-                            const float G = p.aux[row + n], U = p.aux[row + F + n];
-                            const float s = sigmoidf_(G);
-                            p.out0[row + F + n] = v * G * s;
-                            p.out0[row + n] = v * U * s * (1.f + G * (1.f - s));
+                            const float* gu = p.aux + (row0 + r0) * 2 * F + n;
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                G[i] = i < rows ? __ldg(gu + (int64_t)i * 2 * F) : 0.f;
+                                U[i] = i < rows ? __ldg(gu + (int64_t)i * 2 * F + F) : 0.f;
+                            }
+                        }
+                        bool ok8 = true;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            v[i] = get(r0 + i, lane);
+                            ok8 = ok8 && finite(v[i]);
+                        }
+                        if (!__all_sync(0xffffffffu, ok8)) {
+                            for (int i = 0; i < rows; ++i) {
+#pragma unroll
+                                for (int w = 0; w < 8; ++w)
+                                    if (w == i && !finite(v[w])) v[w] = redo(mrow + r0 + i, n);
+                            }
+                        }
+                        if constexpr (EPI == EPI_SWIGLU_BWD) {
+                            float* o = p.out0 + (row0 + r0) * 2 * F + n;
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                if (i >= rows) break;
+                                const float s = sigmoidf_(G[i]);
+                                o[(int64_t)i * 2 * F + F] = v[i] * G[i] * s;
+                                o[(int64_t)i * 2 * F] = v[i] * U[i] * s * (1.f + G[i] * (1.f - s));
+                            }
                         } else {
-                            const int64_t row = VAR_K ? (int64_t)ti.we * p.M + m : ti.o0 + m;
-                            p.out0[row * p.N + n] = v;
+                            float* o = p.out0 + (row0 + r0) * p.N + n;
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                if (i >= rows) break;
+                                o[(int64_t)i * p.N] = v[i];
+                            }
                         }
                     }
                 }
@@ -565,9 +629,11 @@ static cudaError_t launch(const Params& p, int64_t mt, cudaStream_t s) {
     const int cols = EPI == EPI_SWIGLU_FWD ? p.N / 2 : p.N, per = EPI == EPI_SWIGLU_FWD ? 2 : 1;
     const int64_t wide = mt * ((cols + 128 / per - 1) / (128 / per));
     if (wide <= 0) return cudaSuccess;
-    // 128-wide tiles once they fill the SMs; under that, twice as many 64-wide ones
-    if (wide >= sm_count()) return launch_bn<A_MN, B_MN, VAR_K, EPI, 128>(p, wide, s);
-    return launch_bn<A_MN, B_MN, VAR_K, EPI, 64>(p, mt * ((cols + 64 / per - 1) / (64 / per)), s);
+    // by rounds of tiles: a 32-deep stage of a 64-wide tile takes 1.1 us, of a 128-wide one 1.45
+    const int64_t narrow = mt * ((cols + 64 / per - 1) / (64 / per)), sms = sm_count();
+    if ((wide + sms - 1) / sms * 145 <= (narrow + sms - 1) / sms * 110)
+        return launch_bn<A_MN, B_MN, VAR_K, EPI, 128>(p, wide, s);
+    return launch_bn<A_MN, B_MN, VAR_K, EPI, 64>(p, narrow, s);
 }
 
 }  // namespace f32
