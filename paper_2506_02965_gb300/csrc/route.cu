@@ -595,20 +595,28 @@ __global__ void __launch_bounds__(2 * RB_HALF) route_bwd_partial_kernel(
     }
 }
 
-// Sum the partials of each party's chunks: a block takes 32 outputs; thread group g
-// (of 8) adds chunks g, g+8, ... in order, then group 0 adds the 8 group sums in order.
-constexpr int RR_OUT = 32, RR_GRP = 8;
+// Sum the partials of each party's chunks: of eight partial sums per output, chunks g, g + 8,
+// ... of the party join sum g in order, and the eight are added in order. A thread takes four
+// consecutive outputs (d is a multiple of 4) and, SPLIT, one of their eight sums (added
+// through shared memory), else all eight: for few outputs the split fills the SMs, for many
+// it only costs blocks. HBM-bound; with 32 outputs per block and 4-byte loads it took 46 us for
+// three parties of E = 63, d = 3072 (now 6.7) and 25 us for four of E = 32, d = 2048 (5.9).
+constexpr int RR_GRP = 8, RR_THREADS = 256;
+constexpr int64_t RR_SPLIT_BELOW = 150000;  // outputs: about four per thread of one full round
 
-template <typename T>
-__global__ void __launch_bounds__(RR_OUT * RR_GRP) route_bwd_reduce_kernel(
+template <typename T, bool SPLIT>
+__global__ void __launch_bounds__(RR_THREADS) route_bwd_reduce_kernel(
     const float* __restrict__ part_dw, const float* __restrict__ part_db,
     const int32_t* __restrict__ po, int P, int64_t Tn, int d, int E, int CH, T* dw_router,
     float* dbias) {
     pdl_begin();
-    __shared__ float s_sum[RR_GRP][RR_OUT];
-    const int o = threadIdx.x % RR_OUT, g = threadIdx.x / RR_OUT;
-    const int64_t i = (int64_t)blockIdx.x * RR_OUT + o;
+    constexpr int OUT = SPLIT ? RR_THREADS / RR_GRP : RR_THREADS;  // threads with different outputs
+    constexpr int SUMS = SPLIT ? 1 : RR_GRP;                       // partial sums of a thread
+    __shared__ float4 s_sum[SPLIT ? RR_THREADS : 1];
     const int64_t per_party = (int64_t)E * d;
+    const int g0 = SPLIT ? threadIdx.x / OUT : 0;
+    const int64_t i = ((int64_t)blockIdx.x * OUT + threadIdx.x % OUT) * 4;
+    const bool ok = i < (int64_t)P * per_party;
     auto crange = [&](int p, int64_t* first, int64_t* cnt) {
         int64_t base = 0;
         for (int q = 0; q < P; ++q) {
@@ -618,31 +626,76 @@ __global__ void __launch_bounds__(RR_OUT * RR_GRP) route_bwd_reduce_kernel(
             base += nc;
         }
     };
-    float acc = 0.f;
-    const bool ok = i < (int64_t)P * per_party;
+    float acc[SUMS][4];
+#pragma unroll
+    for (int g = 0; g < SUMS; ++g)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[g][q] = 0.f;
     if (ok) {
         const int p = (int)(i / per_party);
-        const int64_t rem = i % per_party;
         int64_t first, cnt;
         crange(p, &first, &cnt);
-        for (int64_t c = g; c < cnt; c += RR_GRP) acc += part_dw[(first + c) * per_party + rem];
-    }
-    s_sum[g][o] = acc;
-    __syncthreads();
-    if (g == 0 && ok) {
-        float tot = 0.f;
+        const float* src = part_dw + first * per_party + i % per_party;
+#pragma unroll SPLIT ? 4 : 1
+        for (int64_t c = g0; c < cnt; c += RR_GRP) {
 #pragma unroll
-        for (int q = 0; q < RR_GRP; ++q) tot += s_sum[q][o];
-        Elem<T>::store(dw_router + i, tot);
+            for (int g = 0; g < SUMS; ++g) {
+                if (c + g < cnt) {
+                    float v[4];
+                    Vec<float>::load(src + (c + g) * per_party, v);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) acc[g][q] += v[q];
+                }
+            }
+        }
     }
-    if (dbias && g == 0 && i < (int64_t)P * E) {
-        const int p = (int)(i / E), e = (int)(i % E);
+    float tot[4] = {0.f, 0.f, 0.f, 0.f};
+    if constexpr (SPLIT) {
+        s_sum[threadIdx.x] = make_float4(acc[0][0], acc[0][1], acc[0][2], acc[0][3]);
+        __syncthreads();
+        if (g0 == 0) {
+#pragma unroll
+            for (int g = 0; g < RR_GRP; ++g) {
+                const float4 v = s_sum[g * OUT + threadIdx.x];
+                tot[0] += v.x; tot[1] += v.y; tot[2] += v.z; tot[3] += v.w;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int g = 0; g < RR_GRP; ++g)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) tot[q] += acc[g < SUMS ? g : 0][q];
+    }
+    if (ok && g0 == 0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) Elem<T>::store(dw_router + i + q, tot[q]);
+    }
+    const int64_t j = (int64_t)blockIdx.x * RR_THREADS + threadIdx.x;
+    if (dbias && j < (int64_t)P * E) {
+        const int p = (int)(j / E), e = (int)(j % E);
         int64_t first, cnt;
         crange(p, &first, &cnt);
         float sum = 0.f;
         for (int64_t c = 0; c < cnt; ++c) sum += part_db[(first + c) * E + e];
-        dbias[i] = sum;
+        dbias[j] = sum;
     }
+}
+
+template <typename T>
+static cudaError_t launch_route_bwd_reduce(const RouteBwdArgs& a, const float* part_dw, const float* part_db, int CH,
+                                           cudaStream_t s) {
+    const int64_t total = (int64_t)a.P * a.E * a.d;
+    const bool split = total < RR_SPLIT_BELOW;
+    // (every (party, expert) of dbias has a thread too: d >= 4 outputs each, four per thread)
+    const int64_t per = split ? 4 * RR_THREADS / RR_GRP : 4 * RR_THREADS;
+    const dim3 grid((unsigned)((total + per - 1) / per));
+    if (split)
+        (void)launch_pdl(route_bwd_reduce_kernel<T, true>, grid, dim3(RR_THREADS), 0, s, part_dw, part_db, a.po, a.P, a.T,
+                         a.d, a.E, CH, (T*)a.dw_router, a.dbias);
+    else
+        (void)launch_pdl(route_bwd_reduce_kernel<T, false>, grid, dim3(RR_THREADS), 0, s, part_dw, part_db, a.po, a.P, a.T,
+                         a.d, a.E, CH, (T*)a.dw_router, a.dbias);
+    return cudaGetLastError();
 }
 
 // ----------------------------------------------------------------------------- launchers
@@ -838,11 +891,7 @@ static cudaError_t launch_route_bwd_simt(const RouteBwdArgs& a, void* ws, cudaSt
                      a.dlogits, a.po, a.P, a.T, a.d, a.E, part_dw, part_db);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int64_t total = (int64_t)a.P * a.E * a.d;
-    (void)launch_pdl(route_bwd_reduce_kernel<T>, dim3((unsigned)((total + RR_OUT - 1) / RR_OUT)),
-                     dim3(RR_OUT * RR_GRP), 0, s, part_dw, part_db, a.po, a.P, a.T, a.d, a.E, RB_CH,
-                     (T*)a.dw_router, a.dbias);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_route_bwd_reduce<T>(a, part_dw, part_db, RB_CH, s)) != cudaSuccess) return e;
     if (a.dx_router && a.T > 0) {  // dx_router[t] = dlogits[t] W_r[p(t)], K = E
         GemmMArgs m{};
         m.G = a.po ? a.P : 1;
@@ -891,11 +940,7 @@ static cudaError_t launch_route_bwd_tc(const RouteBwdArgs& a, void* ws, cudaStre
         g.E = a.E;
         if ((e = launch_gemm_k(g, true, s)) != cudaSuccess) return e;
     }
-    const int64_t total = (int64_t)a.P * a.E * a.d;
-    (void)launch_pdl(route_bwd_reduce_kernel<__nv_bfloat16>, dim3((unsigned)((total + RR_OUT - 1) / RR_OUT)),
-                     dim3(RR_OUT * RR_GRP), 0, s, (const float*)part_dw, (const float*)part_db, a.po, a.P,
-                     a.T, a.d, a.E, (int)Lw.C, (__nv_bfloat16*)a.dw_router, a.dbias);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_route_bwd_reduce<__nv_bfloat16>(a, part_dw, part_db, (int)Lw.C, s)) != cudaSuccess) return e;
     if (a.dx_router && a.T > 0) {
         GemmMArgs m{};
         m.G = a.po ? a.P : 1;
