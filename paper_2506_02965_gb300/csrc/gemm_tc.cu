@@ -41,17 +41,22 @@ __host__ __device__ constexpr int kblocks_per_stage(int epi, int bn, bool pair, 
     if (pair) return epi != EPI_SWIGLU_BWD ? 2 : 1;
     return bn == 128 ? 2 : 1;
 }
-constexpr int EPI_WARPS = 4;
-constexpr int THREADS = 64 + 32 * EPI_WARPS;  // TMA warp, MMA warp, epilogue warps
+// EW epilogue warps: four (one per TMEM lane quarter), or eight that halve the tile's columns,
+// for contractions so short that the epilogue and not the mainloop sets a tile's time:
+// weight gradients with under 384 rows a group on average (60 rows of d = 3072, F = 384, 63
+// experts: dW1 89 -> 70 us, dW2 61 -> 49; 231 rows 42 -> 35; at 512 rows 80.6 -> 82), GEMM1
+// and GEMM2 with contractions under 1024 (d = 384: GEMM1 50 -> 42 us; d = 1024 84 -> 86).
+constexpr int kWideEpiRows = 384, kWideEpiK = 1024;
+// TMA warp, MMA warp, epilogue warps
+__host__ __device__ constexpr int gemm_threads(int ew) { return 64 + 32 * ew; }
 constexpr int EPI_BOX = 32;                     // TMA-store box: 32 columns x 32 rows (bf16)
 constexpr int EPI_BUF_BYTES = EPI_BOX * EPI_BOX * 2;
-// per epilogue warp: a ring of 4 output boxes (each box leaves by its own TMA store, so
-// up to 3 stores are in flight while the next box is written), or for the SwiGLU
-// backward 2 x (G, U) boxes
-constexpr int EPI_NBUF = 4;
-constexpr int EPI_STAGE_BYTES = EPI_NBUF * EPI_BUF_BYTES;
-// per epilogue warp (the router-gradient partials are stored straight from registers)
-__host__ __device__ constexpr int epi_stage_bytes(int epi) { return epi == EPI_DWR ? 0 : EPI_STAGE_BYTES; }
+// Staging of the epilogue warps together: each has a ring of 4 output boxes (2 of eight warps;
+// each box leaves by its own TMA store, so up to 3 stores are in flight while the next box is
+// written), or for the SwiGLU backward 2 x (G, U) boxes. (The router-gradient partials are
+// stored straight from registers.)
+constexpr int EPI_BOXES = 16;
+__host__ __device__ constexpr int epi_stage_bytes(int epi) { return epi == EPI_DWR ? 0 : EPI_BOXES * EPI_BUF_BYTES; }
 constexpr int MAX_GROUPS = 256;
 
 struct Params {
@@ -89,7 +94,7 @@ struct Params {
 // about half of the SM's 228 KiB each, for launches bound by their epilogue, whose
 // stores then come from twice as many warps per SM).
 __host__ __device__ constexpr int epi_extra_bytes(int epi) {
-    return epi == EPI_ROUTE ? 64 * 64 * 4 : EPI_WARPS * epi_stage_bytes(epi);
+    return epi == EPI_ROUTE ? 64 * 64 * 4 : epi_stage_bytes(epi);
 }
 __host__ __device__ constexpr int num_stages(uint32_t stage_bytes, int epi, int occ = 1) {
     const int per_cta = occ == 1 ? 227 * 1024 : 112 * 1024;
@@ -325,14 +330,15 @@ __device__ __forceinline__ void pair_down(uint32_t u, int lane, float* a, float*
 }
 
 template <int EPI>
-__device__ __forceinline__ void swapped_epilogue(const Params& p, const Tile& ti, int rank, int q, int lane, uint32_t tbase) {
+__device__ __forceinline__ void swapped_epilogue(const Params& p, const Tile& ti, int rank, int q, int lane, uint32_t tbase,
+                                                  int c_beg, int c_step) {
     const int v = ti.mvalid - ti.m0;       // rows of the tile
     const int64_t row0 = ti.out_row + ti.m0;
     const int F = p.F;
     const int n = ti.n0 + rank * 128 + q * 32 + (lane & ~1);  // this lane's pair of features
     if (n >= p.N) return;                                      // (a ragged last tile: whole CTAs)
 #pragma unroll 1
-    for (int c = 0; c < v; c += 32) {
+    for (int c = c_beg; c < v; c += c_step) {
         if constexpr (EPI == EPI_STORE) {
             float y[32];
             tmem_ld32(tbase + c, y);
@@ -393,8 +399,8 @@ __device__ __forceinline__ void swapped_epilogue(const Params& p, const Tile& ti
 // for a weight gradient and the M-variable GEMM of the same backward step. (Interleaving
 // the two problems' tiles group by group measured slower: a tile with a long epilogue
 // followed by one with a short mainloop leaves the MMA waiting for an accumulator.)
-template <int BN, bool B_MN, bool VAR_K, int EPI, bool PAIR = false, bool DW2 = false, int OCC = 1>
-__global__ void __launch_bounds__(THREADS, OCC)
+template <int BN, bool B_MN, bool VAR_K, int EPI, bool PAIR = false, bool DW2 = false, int OCC = 1, int EW = 4>
+__global__ void __launch_bounds__(gemm_threads(EW), OCC)
     grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                         const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmO0,
@@ -406,6 +412,8 @@ __global__ void __launch_bounds__(THREADS, OCC)
     pdl_begin();
     static_assert(!DW2 || (B_MN && !VAR_K && !PAIR && BN == 256), "fused: M-variable, MN-major B");
     static_assert(OCC == 1 || (!PAIR && !DW2 && 2 * BN * OCC <= 512), "shared SMs: single-CTA tiles, TMEM for all");
+    static_assert(EW == 4 || (EW == 8 && !DW2 && (EPI == EPI_STORE || EPI == EPI_SWIGLU_FWD)), "epilogue warps");
+    constexpr int NBUF = EPI_BOXES / EW;  // output boxes of one epilogue warp
     constexpr bool A_MN = VAR_K;
     constexpr bool SWAP = PAIR && !VAR_K && EPI != EPI_SWIGLU_FWD;  // swapped tiles possible
     constexpr int NPAIR = PAIR ? 2 : 1;
@@ -428,7 +436,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
     extern __shared__ uint8_t smem_raw[];
     // K-variable pairs: the peer's own barriers for the partial last k-block of a tile
     constexpr int NPART = (PAIR && VAR_K) ? NST : 0;
-    __shared__ uint64_t bars[2 * NST + 5 + 2 * EPI_WARPS + NPART];
+    __shared__ uint64_t bars[2 * NST + 5 + 2 * EW + NPART];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     __shared__ int s_tile_start[MAX_GROUPS + 1];
@@ -445,24 +453,35 @@ __global__ void __launch_bounds__(THREADS, OCC)
     // 256-wide tiles: its columns past N are computed from zero-filled or unused operand
     // columns and never stored)
     const int tiles_n = (EPI == EPI_SWIGLU_FWD) ? p.N / 256 : (EPI == EPI_ROUTE) ? 1 : (p.N + BN - 1) / BN;
-    if (threadIdx.x == 0) {
-        int acc = 0;
-        for (int g = 0; g < p.G; ++g) {
-            s_tile_start[g] = acc;
-            int mt;
-            if (VAR_K) {
-                mt = p.Mout / BMP;
-            } else {
-                const int rows = p.offsets ? (p.offsets[g + 1] - p.offsets[g]) : p.rows;
-                const int rpt = (EPI == EPI_ROUTE) ? p.tile_rows : BMP;  // rows per tile
-                mt = rows > 0 ? (rows + rpt - 1) / rpt : 0;
+    if (warp == 0) {  // a warp scan: one thread reading 64 groups' offsets in turn took over a microsecond
+        int run = 0;
+        for (int g0 = 0; g0 < p.G; g0 += 32) {
+            const int g = g0 + lane;
+            int n = 0;
+            if (g < p.G) {
+                if (VAR_K) {
+                    n = p.Mout / BMP;
+                } else {
+                    const int rows = p.offsets ? (p.offsets[g + 1] - p.offsets[g]) : p.rows;
+                    const int rpt = (EPI == EPI_ROUTE) ? p.tile_rows : BMP;  // rows per tile
+                    n = rows > 0 ? (rows + rpt - 1) / rpt : 0;
+                }
+                n *= tiles_n;
             }
-            acc += mt * tiles_n;
+            int inc = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += u;
+            }
+            if (g < p.G) s_tile_start[g] = run + inc - n;
+            run += __shfl_sync(0xffffffffu, inc, 31);
         }
-        s_tile_start[p.G] = acc;
-        s_total1 = acc;
-        if constexpr (DW2) s_tile_start[p.G] = acc + p.G * (p2.Mout / BM) * (p2.N / BN);
-        s_abort = 0;
+        if (lane == 0) {
+            s_total1 = run;
+            s_tile_start[p.G] = DW2 ? run + p.G * (p2.Mout / BM) * (p2.N / BN) : run;
+            s_abort = 0;
+        }
     }
     __syncthreads();
     if constexpr (DW2) {
@@ -596,7 +615,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
     const uint32_t raw_u32 = smem_u32(smem_raw);
     const uint32_t ring = raw_u32 + ((1024u - (raw_u32 & 1023u)) & 1023u);
     uint8_t* ring_ptr = smem_raw + (ring - raw_u32);
-    uint8_t* stage_out = ring_ptr + (size_t)NST * STAGE_BYTES;  // EPI_WARPS x EPI_STAGE_BYTES
+    uint8_t* stage_out = ring_ptr + (size_t)NST * STAGE_BYTES;  // the epilogue warps' staging boxes
     int* route_hist = reinterpret_cast<int*>(stage_out);             // EPI_ROUTE has no staging
     if constexpr (EPI == EPI_ROUTE) {
         for (int i = threadIdx.x; i < p.hist_n; i += blockDim.x) route_hist[i] = 0;
@@ -607,7 +626,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
     auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * NST + a); };
     auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * NST + 2 + a); };
     const uint32_t drain_bar = bar0 + 8u * (2 * NST + 4);
-    auto pfull_bar = [&](int s) { return bar0 + 8u * (2 * NST + 5 + 2 * EPI_WARPS + s); };
+    auto pfull_bar = [&](int s) { return bar0 + 8u * (2 * NST + 5 + 2 * EW + s); };
     // waits: cluster-scope acquire when the barrier also collects the peer's arrivals
     auto wait_bar = [&](uint32_t bar, uint32_t parity) -> bool {
         if constexpr (PAIR) {
@@ -634,10 +653,10 @@ __global__ void __launch_bounds__(THREADS, OCC)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(tfull_bar(a), 1);
-            mbar_init(tempty_bar(a), EPI_WARPS * NPAIR);  // one arrival per epilogue warp
+            mbar_init(tempty_bar(a), EW * NPAIR);  // one arrival per epilogue warp
         }
         mbar_init(drain_bar, 1);
-        for (int i = 0; i < 2 * EPI_WARPS; ++i) mbar_init(bar0 + 8u * (2 * NST + 5 + i), 1);
+        for (int i = 0; i < 2 * EW; ++i) mbar_init(bar0 + 8u * (2 * NST + 5 + i), 1);
         for (int s = 0; s < NPART; ++s) mbar_init(pfull_bar(s), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -941,8 +960,10 @@ __global__ void __launch_bounds__(THREADS, OCC)
         // staged in shared memory and written by TMA stores; a box that reaches past the
         // group's last row (the last M tile of an expert) is written row by row instead.
         const int q = warp & 3;
+        const int half = EW == 8 ? (warp - 2) >> 2 : 0;  // of the tile's columns, with eight warps
+        constexpr int SPLIT = EW / 4;
         const int row_local = q * 32 + lane;
-        uint8_t* stg = stage_out + (size_t)(warp - 2) * epi_stage_bytes(EPI);
+        uint8_t* stg = stage_out + (size_t)(warp - 2) * (epi_stage_bytes(EPI) / EW);
         const uint32_t stg_u32 = smem_u32(stg);
         int acc = 0;
         uint32_t acc_phase = 0;
@@ -990,9 +1011,9 @@ __global__ void __launch_bounds__(THREADS, OCC)
                 if (full_box) {
 #pragma unroll
                     for (int o = 0; o < nout; ++o) {
-                        const uint32_t b = box_seq & (EPI_NBUF - 1);
-                        // the store that last used box b (EPI_NBUF boxes ago) has read it
-                        if (lane == 0) bulk_wait_read<EPI_NBUF - 1>();
+                        const uint32_t b = box_seq & (NBUF - 1);
+                        // the store that last used box b (NBUF boxes ago) has read it
+                        if (lane == 0) bulk_wait_read<NBUF - 1>();
                         __syncwarp();
                         store_row32_sw64(stg + b * EPI_BUF_BYTES + lane * 64, lane, vals[o]);
                         fence_proxy_async();
@@ -1013,7 +1034,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
                 fence_after();
                 __nv_bfloat16* out = (__nv_bfloat16*)p2.out0 + (int64_t)ti.we * p2.Mout * p2.N + (int64_t)m * p2.N;
 #pragma unroll 1
-                for (int c = 0; c < BN; c += 32) {
+                for (int c = half * (BN / SPLIT); c < (half + 1) * (BN / SPLIT); c += 32) {
                     float y[32];
                     if (ti.k_iters > 0) {
                         tmem_ld32(tbase + c, y);
@@ -1030,7 +1051,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
             } else if (SWAP && ti.ntok) {
                 if (!wait_bar(tfull_bar(acc), acc_phase)) break;
                 fence_after();
-                swapped_epilogue<EPI>(p, ti, (int)rank, q, lane, tbase);
+                swapped_epilogue<EPI>(p, ti, (int)rank, q, lane, tbase, half * 32, SPLIT * 32);
             } else if constexpr (EPI == EPI_SWIGLU_BWD) {
                 // dA in TMEM. G and U of each 32-column chunk arrive by TMA in one of two
                 // staging buffers (the next chunk's load is in flight while this one is
@@ -1099,7 +1120,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
                     __nv_bfloat16* hgu = (__nv_bfloat16*)p.out0 + (ti.out_row + m) * (int64_t)(2 * F);
                     __nv_bfloat16* actp = (__nv_bfloat16*)p.out1 + (ti.out_row + m) * (int64_t)F;
 #pragma unroll 1
-                    for (int c = 0; c < 128; c += 32) {
+                    for (int c = half * (128 / SPLIT); c < (half + 1) * (128 / SPLIT); c += 32) {
                         float g[32], u[32], a[32];
                         tmem_ld32(tbase + c, g);
                         tmem_ld32(tbase + 128 + c, u);
@@ -1145,7 +1166,7 @@ __global__ void __launch_bounds__(THREADS, OCC)
                     else
                         out = (__nv_bfloat16*)p.out0 + (ti.out_row + m) * (int64_t)p.N;
 #pragma unroll 1
-                    for (int c = 0; c < BN && ti.n0 + c < p.N; c += 32) {
+                    for (int c = half * (BN / SPLIT); c < (half + 1) * (BN / SPLIT) && ti.n0 + c < p.N; c += 32) {
                         float y[32];
                         if (ti.k_iters > 0) {
                             tmem_ld32(tbase + c, y);
@@ -1266,13 +1287,13 @@ static int band_for(int c) {
     return b;
 }
 
-template <int BN, bool B_MN, bool VAR_K, int EPI, bool PAIR = false, bool DW2 = false, int OCC = 1>
+template <int BN, bool B_MN, bool VAR_K, int EPI, bool PAIR = false, bool DW2 = false, int OCC = 1, int EW = 4>
 static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mo0,
                           const CUtensorMap& mo1, const Params& p, int64_t tiles_ub,
                           cudaStream_t s, const CUtensorMap* ma2 = nullptr,
                           const CUtensorMap* mb2 = nullptr, const CUtensorMap* mo2 = nullptr,
                           const Params* p2 = nullptr, const CUtensorMap* mas = nullptr) {
-    auto kern = grouped_gemm_kernel<BN, B_MN, VAR_K, EPI, PAIR, DW2, OCC>;
+    auto kern = grouped_gemm_kernel<BN, B_MN, VAR_K, EPI, PAIR, DW2, OCC, EW>;
     const CUtensorMap& A2 = ma2 ? *ma2 : ma;
     const CUtensorMap& B2 = mb2 ? *mb2 : mb;
     const CUtensorMap& O2 = mo2 ? *mo2 : mo0;
@@ -1283,8 +1304,8 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
     constexpr int KB = kblock_rows(VAR_K, PAIR, EPI, BN);
     constexpr int STB = (BM * KB * 2 + BN / NPAIR * KB * 2) * kblocks_per_stage(EPI, BN, PAIR, VAR_K, DW2, OCC);  // bytes of one operand stage
     constexpr int NST = num_stages((uint32_t)STB, EPI, OCC);
-    const int extra_max = EPI == EPI_ROUTE ? 64 * 64 * 4 : EPI_WARPS * epi_stage_bytes(EPI);
-    const int extra = EPI == EPI_ROUTE ? p.hist_n * 4 : EPI_WARPS * epi_stage_bytes(EPI);
+    const int extra_max = EPI == EPI_ROUTE ? 64 * 64 * 4 : epi_stage_bytes(EPI);
+    const int extra = EPI == EPI_ROUTE ? p.hist_n * 4 : epi_stage_bytes(EPI);
     const int smem_max = NST * STB + 1024 + extra_max;
     const int smem = NST * STB + 1024 + extra;
     static bool attr_set = false;
@@ -1301,7 +1322,7 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
         if (!max_clusters) {
             cudaLaunchConfig_t q = {};
             q.gridDim = dim3(2 * (sm_count() / 2));
-            q.blockDim = dim3(THREADS);
+            q.blockDim = dim3(gemm_threads(EW));
             q.dynamicSmemBytes = smem_max;
             cudaLaunchAttribute qa[1];
             qa[0].id = cudaLaunchAttributeClusterDimension;
@@ -1321,7 +1342,7 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
         P1.band = P2.band = band_for(clusters);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(2 * clusters);
-        cfg.blockDim = dim3(THREADS);
+        cfg.blockDim = dim3(gemm_threads(EW));
         cfg.dynamicSmemBytes = smem;
         cfg.stream = s;
         cudaLaunchAttribute attr[2];
@@ -1337,7 +1358,7 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
     } else {
         const int grid = (int)std::min<int64_t>(tiles_ub, (int64_t)OCC * sm_count());
         P1.band = P2.band = band_for(grid);
-        (void)launch_pdl(kern, dim3(grid), dim3(THREADS), smem, s, ma, mb, mo0, mo1, AS, P1, A2, B2, O2, P2);
+        (void)launch_pdl(kern, dim3(grid), dim3(gemm_threads(EW)), smem, s, ma, mb, mo0, mo1, AS, P1, A2, B2, O2, P2);
         return cudaGetLastError();
     }
 }
@@ -1423,6 +1444,7 @@ cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s) {
     CUtensorMap ma, mb, mo0, mo1, mas;  // mas: A in boxes of 32 rows (swapped tiles)
     if (!make_map(&ma, g.a, g.K, a_rows, BM)) return cudaErrorInvalidValue;
     if (pair && !make_map(&mas, g.a, g.K, a_rows, 32)) return cudaErrorInvalidValue;
+    const bool wide_epi = g.K < kWideEpiK;
     if (g.epi == EPI_SWIGLU_FWD) {
         const int F = g.N / 2;
         p.F = F;
@@ -1430,7 +1452,9 @@ cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s) {
         if (!make_map(&mb, g.b, g.K, (int64_t)g.G * 2 * F, 128)) return cudaErrorInvalidValue;
         if (!make_map(&mo0, g.out0, 2 * (int64_t)F, o_rows, 0, true)) return cudaErrorInvalidValue;
         if (!make_map(&mo1, g.out1, F, o_rows, 0, true)) return cudaErrorInvalidValue;
+        if (pair && wide_epi) return launch<256, false, false, EPI_SWIGLU_FWD, true, false, 1, 8>(ma, mb, mo0, mo1, p, pt_ub * (F / 128), s);
         if (pair) return launch<256, false, false, EPI_SWIGLU_FWD, true>(ma, mb, mo0, mo1, p, pt_ub * (F / 128), s);
+        if (wide_epi) return launch<256, false, false, EPI_SWIGLU_FWD, false, false, 1, 8>(ma, mb, mo0, mo1, p, mt_ub * (F / 128), s);
         return launch<256, false, false, EPI_SWIGLU_FWD>(ma, mb, mo0, mo1, p, mt_ub * (F / 128), s);
     }
     if (g.epi == EPI_STORE && g.b_kmajor) {  // Y = A W2^T: B = W2[e] as [N=d, K=F]
@@ -1438,14 +1462,19 @@ cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s) {
         if (!make_map(&mo0, g.out0, g.N, o_rows, 0, true)) return cudaErrorInvalidValue;
         if (pair) {
             if (!make_map(&mb, g.b, g.K, (int64_t)g.G * g.N, 128)) return cudaErrorInvalidValue;
+            if (wide_epi)
+                return launch<256, false, false, EPI_STORE, true, false, 1, 8>(ma, mb, mo0, mo0, p, pt_ub * ((g.N + 255) / 256),
+                                                                               s, nullptr, nullptr, nullptr, nullptr, &mas);
             return launch<256, false, false, EPI_STORE, true>(ma, mb, mo0, mo0, p, pt_ub * ((g.N + 255) / 256), s, nullptr,
                                                               nullptr, nullptr, nullptr, &mas);
         }
         if (g.N % 256 == 0) {
             if (!make_map(&mb, g.b, g.K, (int64_t)g.G * g.N, 256)) return cudaErrorInvalidValue;
+            if (wide_epi) return launch<256, false, false, EPI_STORE, false, false, 1, 8>(ma, mb, mo0, mo0, p, mt_ub * (g.N / 256), s);
             return launch<256, false, false, EPI_STORE>(ma, mb, mo0, mo0, p, mt_ub * (g.N / 256), s);
         }
         if (!make_map(&mb, g.b, g.K, (int64_t)g.G * g.N, 128)) return cudaErrorInvalidValue;
+        if (wide_epi) return launch<128, false, false, EPI_STORE, false, false, 1, 8>(ma, mb, mo0, mo0, p, mt_ub * (g.N / 128), s);
         return launch<128, false, false, EPI_STORE>(ma, mb, mo0, mo0, p, mt_ub * (g.N / 128), s);
     }
     // MN-major B: weights stored [G*K, N] (or [G*b_rows, N])
@@ -1511,8 +1540,13 @@ cudaError_t launch_gemm_k(const GemmKArgs& g, bool bf16, cudaStream_t s) {
         return launch<256, true, true, EPI_DWR>(ma, mb, ma, ma, p, tiles, s);
     }
     if (!make_map(&mo, g.out, g.N, (int64_t)g.G * g.M, 0, true)) return cudaErrorInvalidValue;
-    if (pair)
-        return launch<256, true, true, EPI_STORE, true>(ma, mb, mo, mo, p, (int64_t)g.G * (g.M / 256) * ((g.N + 255) / 256), s);
+    const int64_t pair_tiles = (int64_t)g.G * (g.M / 256) * ((g.N + 255) / 256);
+    if ((g.rows.offsets ? (int64_t)g.rows.rows / g.G : (int64_t)g.rows.rows) < kWideEpiRows) {
+        if (pair) return launch<256, true, true, EPI_STORE, true, false, 1, 8>(ma, mb, mo, mo, p, pair_tiles, s);
+        if (g.N % 256 == 0) return launch<256, true, true, EPI_STORE, false, false, 1, 8>(ma, mb, mo, mo, p, tiles * (g.N / 256), s);
+        return launch<128, true, true, EPI_STORE, false, false, 1, 8>(ma, mb, mo, mo, p, tiles * (g.N / 128), s);
+    }
+    if (pair) return launch<256, true, true, EPI_STORE, true>(ma, mb, mo, mo, p, pair_tiles, s);
     if (g.N % 256 == 0) return launch<256, true, true, EPI_STORE>(ma, mb, mo, mo, p, tiles * (g.N / 256), s);
     return launch<128, true, true, EPI_STORE>(ma, mb, mo, mo, p, tiles * (g.N / 128), s);
 }
