@@ -335,13 +335,13 @@ moe_status moe_set_wait_limit_ns(uint64_t ns);
  * as few tiles share the SMs, so a launch with few tiles loses to its last round.
  *   MOE_PAIRS_OFF  (0): single-CTA tiles everywhere;
  *   MOE_PAIRS_ALL  (1): pair tiles for every such GEMM;
- *   MOE_PAIRS_AUTO (2, default): pair tiles for the input-gradient GEMM dX = dH W1
- *                   (contraction 2F) and wherever a launch has at least four rounds
- *                   of them, except under the SwiGLU backward epilogue when d < 2048
- *                   (there the epilogue, not the operand feed, bounds the dA GEMM).
+ *   MOE_PAIRS_AUTO (2, default): pair tiles where a launch takes less time by them,
+ *                   counted in rounds of tiles over the SMs; under the SwiGLU backward
+ *                   epilogue when d >= 2048 and there are at least four rounds (below,
+ *                   the epilogue, not the operand feed, bounds the dA GEMM).
  * The weight-gradient GEMMs launched on their own (dW1; dW2 when dA runs as pairs; the
- * shared experts') follow the same mode with 256 x 256 output tiles where both output
- * dimensions are multiples of 256.
+ * shared experts') follow the same mode with 256 x 256 output tiles where M is a multiple
+ * of 256.
  * Results agree up to fp32 summation order. Any other mode: MOE_ERR_INVALID_ARG. */
 enum { MOE_PAIRS_OFF = 0, MOE_PAIRS_ALL = 1, MOE_PAIRS_AUTO = 2 };
 moe_status moe_set_gemm_pairs(int mode);

@@ -12,6 +12,7 @@
 // records MOE_ERR_TIMEOUT, drains its in-flight copies and MMAs, frees TMEM and
 // returns.
 #include <algorithm>
+#include <cmath>
 
 #include "moe_internal.h"
 #include "tc_ptx.cuh"
@@ -1369,26 +1370,47 @@ void set_wait_limit_ns(uint64_t ns) { tc::g_wait_ns = ns ? ns : 1; }
 uint64_t wait_limit_ns() { return tc::g_wait_ns; }
 void set_gemm_pairs(int mode) { tc::g_pairs = mode; }
 
-// Pair tiles where they fill at least four rounds of the SMs (the last, partly empty
-// round then costs little) and the operand feed, not the epilogue, bounds the tile.
-// The input-gradient GEMM (plain store, MN-major weights, a long contraction) takes
-// pairs with fewer tiles too: an SM ingests at most ~145 GB/s from L2 with TMA, which
-// caps a single-CTA 128 x 256 tile near 80% of the MMA rate and a pair's 256 x 256 tile
-// (half the B bytes per SM) does not, and its weight-gradient partner then runs beside
-// it on the second stream. The SwiGLU-backward GEMM (dA) moves G, U, dG and dU in its
-// epilogue: with a short contraction (d < 2048) the epilogue bounds it and single-CTA
-// tiles fused with dW2 in one launch are faster; from d = 2048 the mainloop dominates
-// and pairs win (d = 4096: the expert backward 17.8 -> 17.2 ms; d = 1024: +4%).
+// Tiles of `tile` rows that `rows` rows in G groups make, if the router spreads them evenly:
+// each group has r = rows / G of them give or take sqrt(r), so the mean of the tiles at half
+// a deviation below and above. (The counts are on the device; a rule that waited for them
+// would synchronise.)
+static int64_t expected_tiles(const GroupRows& gr, int G, int tile) {
+    if (!gr.offsets) return (int64_t)G * ((gr.rows + tile - 1) / tile);
+    const double r = (double)gr.rows / G, dev = 0.5 * std::sqrt(r);
+    const double lo = std::ceil(std::max(r - dev, 1.0) / tile), hi = std::ceil((r + dev) / tile);
+    return (int64_t)(G * (lo + hi) / 2);
+}
+
+// Pair tiles or single-CTA tiles, by rounds: a pair's 256 x 256 tile takes half of the B bytes
+// per SM and flop of a 128 x 256 tile, so a round of pairs (two rows of single tiles) takes
+// 1 where a round of single tiles takes 1.3 (128 x 128: 1.05), but has half as many tiles and
+// loses more in a last round. Measured, pairs against single: dX of 8192 rows, 16 experts,
+// d = 1024 (3 rounds, 2) 97, 84 us; of 49152 rows, 64 experts, d = 2048 (24, 22) 351, 409;
+// GEMM1 of 4314 rows, 6 experts (2, 2) 41, 47 and of 1092, 4 experts (2, 1) 40, 31; GEMM2 of
+// 3009 rows, 13 experts, d = 1152 (1, 2 of 128 x 128) 22, 25; 6 rows an expert, 64 experts,
+// d = 2048: GEMM1 (10, 5) 135, 118. With a contraction under 512 the epilogue weighs more:
+// pairs only with fewer rounds, or as many from four on (GEMM2 of F = 256 in two: 12.6, 11.4). The
+// SwiGLU-backward GEMM (dA) moves G, U, dG and dU in its epilogue: with a short contraction
+// (d < 2048) the epilogue bounds it and single-CTA tiles (fused with dW2 in one launch) are
+// faster; from d = 2048 the mainloop dominates and pairs win (d = 4096: the expert backward
+// 17.8 -> 17.2 ms; d = 1024: +4%).
 bool gemm_m_uses_pairs(const GemmMArgs& g) {
     using namespace tc;
     if (g.N % 128 != 0) return false;  // 256-wide pair tiles, the last one possibly ragged
     if (g_pairs == MOE_PAIRS_ALL) return true;
-    if (g_pairs != MOE_PAIRS_AUTO) return false;
-    if (g.epi == EPI_SWIGLU_BWD && g.K < 2048) return false;
-    if (g.epi == EPI_STORE && !g.b_kmajor && g.K >= 512) return true;
-    const int64_t pt_ub = g.rows.offsets ? ((int64_t)g.rows.rows + 2 * BM - 1) / (2 * BM) + g.G
-                                         : (int64_t)g.G * ((g.rows.rows + 2 * BM - 1) / (2 * BM));
-    return pt_ub * ((g.N + 255) / 256) >= 4 * (int64_t)(sm_count() / 2);
+    if (g_pairs != MOE_PAIRS_AUTO || g.slim) return false;
+    if (g.epi == EPI_SWIGLU_BWD) {
+        if (g.K < 2048) return false;
+        const int64_t pt_ub = g.rows.offsets ? ((int64_t)g.rows.rows + 2 * BM - 1) / (2 * BM) + g.G
+                                             : (int64_t)g.G * ((g.rows.rows + 2 * BM - 1) / (2 * BM));
+        return pt_ub * ((g.N + 255) / 256) >= 4 * (int64_t)(sm_count() / 2);
+    }
+    const bool wide = g.N % 256 == 0;  // (a GEMM1 tile's 256 columns are 128 features, gate and up)
+    const int64_t sms = sm_count(), pairs = sms / 2;
+    const int64_t tp = expected_tiles(g.rows, g.G, 2 * BM) * ((g.N + 255) / 256);
+    const int64_t ts = expected_tiles(g.rows, g.G, BM) * (wide ? g.N / 256 : g.N / 128);
+    const int64_t rp = (tp + pairs - 1) / pairs, rs = (ts + sms - 1) / sms;
+    return g.K < 512 ? rp < rs || (rp == rs && rp >= 4) : rp * 100 <= rs * (wide ? 130 : 105);
 }
 
 // K-variable weight gradients (dW = A^T B over each group's rows) as 256 x 256 CTA-pair

@@ -541,10 +541,10 @@ moe_status moe_expert_ffn_bwd(const moe_config* cfg, const void* x_perm, const i
     // Each M-variable GEMM runs with its weight gradient in one persistent launch (one
     // tail instead of two, and no two persistent grids contending for SMs): dA then dW2
     // (which needs only dY and A), dX then dW1 (which needs dH). A GEMM that runs as
-    // CTA-pair tiles, and the fp32 path, instead put the weight gradient on a side
-    // stream: dW2 alongside dA, dW1 alongside dX once dH exists.
-    const bool fuse_a = bf16 && !gemm_m_uses_pairs(a);
-    const bool fuse_b = bf16 && !gemm_m_uses_pairs(b);  // the same rule as moe_expert_ffn_bwd_kernels
+    // CTA-pair tiles, a dX whose dW1 does, and the fp32 path, instead put the weight gradient
+    // on a side stream: dW2 alongside dA, dW1 alongside dX once dH exists.
+    const bool fuse_a = bf16 && !gemm_m_uses_pairs(a);  // the same rules as moe_expert_ffn_bwd_kernels
+    const bool fuse_b = bf16 && !gemm_m_uses_pairs(b) && !gemm_k_uses_pairs(w1g);
     SideStream* ss = nullptr;
     std::unique_lock<std::mutex> side_lock(g_side_mu, std::defer_lock);
     if (!fuse_a || !fuse_b) {
@@ -719,7 +719,11 @@ moe_status moe_expert_ffn_bwd_kernels(const moe_config* cfg, int32_t* count) {
     int n = 0;
     if (TK > 0) {
         n += (bf16 && !gemm_m_uses_pairs(a)) ? 1 : 2;
-        n += (bf16 && !gemm_m_uses_pairs(b)) ? 1 : 2;
+        GemmKArgs w1g{};
+        w1g.G = cfg->n_experts;
+        w1g.M = 2 * cfg->d_ff;
+        w1g.N = cfg->d_model;
+        n += (bf16 && !gemm_m_uses_pairs(b) && !gemm_k_uses_pairs(w1g)) ? 1 : 2;
     }
     if (cfg->n_shared && cfg->T > 0) n += 4;
     *count = n;
