@@ -115,6 +115,7 @@ struct Tile {
     int k_iters;
     int last_rows;      // K-var: valid contraction rows in the last k-block (1..64)
     bool dw;            // a tile of the second (K-variable) problem of a fused launch
+    bool sec;           // a tile of the second M-variable problem (the shared experts')
     int we;             // expert whose weights (M-variable) or weight gradient (K-variable)
                         // the tile uses: group_expert[g], or g
     int ntok;           // swapped tile (below): its rows rounded up to 16, else 0
@@ -331,28 +332,27 @@ __device__ __forceinline__ void pair_down(uint32_t u, int lane, float* a, float*
 }
 
 template <int EPI>
-__device__ __forceinline__ void swapped_epilogue(const Params& p, const Tile& ti, int rank, int q, int lane, uint32_t tbase,
-                                                  int c_beg, int c_step) {
+__device__ __forceinline__ void swapped_epilogue(int N, int F, void* out0, const void* aux, const Tile& ti, int rank, int q,
+                                                  int lane, uint32_t tbase, int c_beg, int c_step) {
     const int v = ti.mvalid - ti.m0;       // rows of the tile
     const int64_t row0 = ti.out_row + ti.m0;
-    const int F = p.F;
     const int n = ti.n0 + rank * 128 + q * 32 + (lane & ~1);  // this lane's pair of features
-    if (n >= p.N) return;                                      // (a ragged last tile: whole CTAs)
+    if (n >= N) return;                                        // (a ragged last tile: whole CTAs)
 #pragma unroll 1
     for (int c = c_beg; c < v; c += c_step) {
         if constexpr (EPI == EPI_STORE) {
             float y[32];
             tmem_ld32(tbase + c, y);
-            __nv_bfloat16* out = (__nv_bfloat16*)p.out0 + (row0 + c) * (int64_t)p.N + n;
+            __nv_bfloat16* out = (__nv_bfloat16*)out0 + (row0 + c) * (int64_t)N + n;
 #pragma unroll
             for (int i = 0; i < 32; i += 2) {
                 const uint32_t u = pair_up(y[i], y[i + 1], lane);
                 const int j = i + (lane & 1);
-                if (c + j < v) *reinterpret_cast<uint32_t*>(out + j * (int64_t)p.N) = u;
+                if (c + j < v) *reinterpret_cast<uint32_t*>(out + j * (int64_t)N) = u;
             }
         } else {  // SwiGLU backward: y = dA
-            const __nv_bfloat16* gu = (const __nv_bfloat16*)p.aux + (row0 + c) * (int64_t)(2 * F) + n;
-            __nv_bfloat16* dh = (__nv_bfloat16*)p.out0 + (row0 + c) * (int64_t)(2 * F) + n;
+            const __nv_bfloat16* gu = (const __nv_bfloat16*)aux + (row0 + c) * (int64_t)(2 * F) + n;
+            __nv_bfloat16* dh = (__nv_bfloat16*)out0 + (row0 + c) * (int64_t)(2 * F) + n;
 #pragma unroll 1
             for (int h = 0; h < 32 && c + h < v; h += 16) {
                 uint32_t gr[8], ur[8];
@@ -400,6 +400,12 @@ __device__ __forceinline__ void swapped_epilogue(const Params& p, const Tile& ti
 // for a weight gradient and the M-variable GEMM of the same backward step. (Interleaving
 // the two problems' tiles group by group measured slower: a tile with a long epilogue
 // followed by one with a short mainloop leaves the MMA waiting for an accumulator.)
+// The forward GEMMs (K-major B) take a second problem of their own kind with uniform groups
+// (p2.G > 0; tmA2, tmB2, tmO2, tmX2 = its out1 or its boxes of swapped tiles): the shared
+// experts' tiles after the routed ones, in the SMs that the last round leaves free. On
+// their own they are short and latency-bound (64 tokens, two of d = 2048, Fs = 1408: 18.7 and
+// 12.5 us for 35 MB of weights): the forward of 64 tokens with 64 such routed experts
+// 264 -> 233 us (of 2999 tokens, where they had rounds of their own, 0.5% less).
 template <int BN, bool B_MN, bool VAR_K, int EPI, bool PAIR = false, bool DW2 = false, int OCC = 1, int EW = 4>
 __global__ void __launch_bounds__(gemm_threads(EW), OCC)
     grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
@@ -409,8 +415,10 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                         const __grid_constant__ CUtensorMap tmAs, const Params p,
                         const __grid_constant__ CUtensorMap tmA2,
                         const __grid_constant__ CUtensorMap tmB2,
-                        const __grid_constant__ CUtensorMap tmO2, const Params p2) {
+                        const __grid_constant__ CUtensorMap tmO2,
+                        const __grid_constant__ CUtensorMap tmX2, const Params p2) {
     pdl_begin();
+    constexpr bool SH = !VAR_K && !B_MN && (EPI == EPI_STORE || EPI == EPI_SWIGLU_FWD);
     static_assert(!DW2 || (B_MN && !VAR_K && !PAIR && BN == 256), "fused: M-variable, MN-major B");
     static_assert(OCC == 1 || (!PAIR && !DW2 && 2 * BN * OCC <= 512), "shared SMs: single-CTA tiles, TMEM for all");
     static_assert(EW == 4 || (EW == 8 && !DW2 && (EPI == EPI_STORE || EPI == EPI_SWIGLU_FWD)), "epilogue warps");
@@ -454,6 +462,8 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
     // 256-wide tiles: its columns past N are computed from zero-filled or unused operand
     // columns and never stored)
     const int tiles_n = (EPI == EPI_SWIGLU_FWD) ? p.N / 256 : (EPI == EPI_ROUTE) ? 1 : (p.N + BN - 1) / BN;
+    const int tiles_n2 = (EPI == EPI_SWIGLU_FWD) ? p2.N / 256 : (p2.N + BN - 1) / BN;  // (SH)
+    const int tiles_m2 = (p2.rows + BMP - 1) / BMP;
     if (warp == 0) {  // a warp scan: one thread reading 64 groups' offsets in turn took over a microsecond
         int run = 0;
         for (int g0 = 0; g0 < p.G; g0 += 32) {
@@ -480,7 +490,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
         }
         if (lane == 0) {
             s_total1 = run;
-            s_tile_start[p.G] = DW2 ? run + p.G * (p2.Mout / BM) * (p2.N / BN) : run;
+            s_tile_start[p.G] = run + (DW2 ? p.G * (p2.Mout / BM) * (p2.N / BN) : SH ? p2.G * tiles_m2 * tiles_n2 : 0);
             s_abort = 0;
         }
     }
@@ -532,7 +542,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
     };
     auto tile_at = [&](int t) -> Tile {
         Tile ti;
-        ti.dw = false;
+        ti.dw = ti.sec = false;
         ti.ntok = 0;
         if constexpr (DW2) {
             if (t >= s_total1) {  // second problem: K-variable, rows of group g
@@ -556,27 +566,38 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                 return ti;
             }
         }
-        // the group whose tile range holds t: last g with s_tile_start[g] <= t (binary
-        // search; empty groups share their start with the next one)
-        int lo = 0, hi = p.G - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (s_tile_start[mid] <= t) lo = mid;
-            else hi = mid - 1;
+        int g, mt, nt;
+        if (SH && t >= s_total1) {  // second problem: uniform groups
+            ti.sec = true;
+            g = (t - s_total1) / (tiles_m2 * tiles_n2);
+            band_split((t - s_total1) % (tiles_m2 * tiles_n2), tiles_m2, tiles_n2, group_band(p2, p2.rows, tiles_m2), &mt, &nt);
+        } else {
+            // the group whose tile range holds t: last g with s_tile_start[g] <= t (binary
+            // search; empty groups share their start with the next one)
+            int lo = 0, hi = p.G - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (s_tile_start[mid] <= t) lo = mid;
+                else hi = mid - 1;
+            }
+            g = lo;
+            const int local = t - s_tile_start[g];
+            const int g_end = (g + 1 < p.G) ? s_tile_start[g + 1] : s_total1;
+            const int mt_g = (g_end - s_tile_start[g]) / tiles_n;
+            const int64_t rows_g = p.offsets ? (int64_t)(p.offsets[g + 1] - p.offsets[g]) : (int64_t)p.rows;
+            band_split(local, mt_g, tiles_n, group_band(p, rows_g, mt_g), &mt, &nt);
         }
-        const int g = lo;
-        const int local = t - s_tile_start[g];
-        const int g_end = (g + 1 < p.G) ? s_tile_start[g + 1] : s_total1;
-        const int mt_g = (g_end - s_tile_start[g]) / tiles_n;
-        const int64_t rows_g = p.offsets ? (int64_t)(p.offsets[g + 1] - p.offsets[g]) : (int64_t)p.rows;
-        int mt, nt;
-        band_split(local, mt_g, tiles_n, group_band(p, rows_g, mt_g), &mt, &nt);
         ti.g = g;
-        ti.we = p.gexp ? p.gexp[g] : g;
+        ti.we = !ti.sec && p.gexp ? p.gexp[g] : g;
         ti.m0 = (EPI == EPI_ROUTE) ? mt * p.tile_rows : mt * BMP + (int)rank * BM;
         ti.n0 = nt * ((EPI == EPI_SWIGLU_FWD) ? 128 : BN);
         int64_t r0, nrows, a0, b0, o0;
-        if (p.offsets) {
+        if (SH && ti.sec) {
+            nrows = p2.rows;
+            a0 = (int64_t)g * p2.a_stride;
+            b0 = 0;
+            o0 = (int64_t)g * p2.out_stride;
+        } else if (p.offsets) {
             r0 = p.offsets[g];
             nrows = p.offsets[g + 1] - r0;
             a0 = b0 = o0 = r0;
@@ -599,7 +620,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
             ti.a_row = a0;
             ti.b_row = 0;
             ti.out_row = o0;
-            ti.k_iters = p.K / (BK * KPS);
+            ti.k_iters = (SH && ti.sec ? p2.K : p.K) / (BK * KPS);
             ti.last_rows = BK;
             if constexpr (SWAP) {
                 const int v = (int)nrows - mt * BMP;
@@ -705,7 +726,11 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
             };
             for (int t = tile0; t < total_tiles && ok; t += tile_step) {
                 const Tile ti = tile_at(t);
-                const bool dw = DW2 && ti.dw;
+                const bool dw = DW2 && ti.dw, sec = SH && ti.sec;
+                const CUtensorMap* mA = dw || sec ? &tmA2 : &tmA;
+                const CUtensorMap* mAs = sec ? &tmX2 : &tmAs;
+                const CUtensorMap* mB = dw || sec ? &tmB2 : &tmB;
+                const int F = sec ? p2.F : p.F;
                 // a swapped tile's rows: half in each CTA, in boxes of 32
                 const int trows = SWAP ? ti.ntok / 2 : 0;
                 uint32_t tile_bytes = NPAIR * STAGE_BYTES;  // per stage, both CTAs of a pair
@@ -716,8 +741,8 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                 int brow;
                 if (VAR_K || dw) brow = (int)ti.b_row;
                 else if (B_MN) brow = (int)((int64_t)ti.we * p.b_group_rows);
-                else brow = (int)((int64_t)ti.we * p.b_group_rows + ti.n0) +
-                            (EPI == EPI_SWIGLU_FWD ? (PAIR && rank ? p.F : 0) : (int)rank * BNL);
+                else brow = (int)((int64_t)ti.we * (sec ? p2.b_group_rows : p.b_group_rows) + ti.n0) +
+                            (EPI == EPI_SWIGLU_FWD ? (PAIR && rank ? F : 0) : (int)rank * BNL);
                 for (int kb = 0; kb < ti.k_iters; ++kb) {
                     if (!wait_bar(empty_bar(stage), phase ^ 1u)) {
                         ok = false;
@@ -749,26 +774,24 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                         if (SWAP && trows) {
                             for (int r = 0; r < trows; r += 32)
 #pragma unroll
-                                for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX + r * 128, &tmAs, fb, k0 + KB * i, arow + r);
+                                for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX + r * 128, mAs, fb, k0 + KB * i, arow + r);
                         } else {
 #pragma unroll
-                            for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX, &tmA, fb, k0 + KB * i, arow);
+                            for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX, mA, fb, k0 + KB * i, arow);
                         }
                     } else {
-                        const CUtensorMap* mA = dw ? &tmA2 : &tmA;
 #pragma unroll
                         for (int i = 0; i < BM / 64; ++i) load(sa + i * ATOM, mA, fb, ti.m0 + 64 * i, arow + k0);
                     }
                     if (!B_MN) {
 #pragma unroll
                         for (int i = 0; i < KPS; ++i) {
-                            load(sb + i * B_BOX, &tmB, fb, k0 + KB * i, brow);
+                            load(sb + i * B_BOX, mB, fb, k0 + KB * i, brow);
                             // SwiGLU forward: 128 gate rows, then 128 up rows of the same features
                             // (in a pair the leader holds the gate half and the peer the up half)
-                            if (EPI == EPI_SWIGLU_FWD && !PAIR) load(sb + i * B_BOX + 128 * 128, &tmB, fb, k0 + KB * i, brow + p.F);
+                            if (EPI == EPI_SWIGLU_FWD && !PAIR) load(sb + i * B_BOX + 128 * 128, mB, fb, k0 + KB * i, brow + F);
                         }
                     } else {
-                        const CUtensorMap* mB = dw ? &tmB2 : &tmB;
 #pragma unroll
                         for (int i = 0; i < BNL / 64; ++i)
                             load(sb + i * ATOM_B, mB, fb, ti.n0 + (int)rank * BNL + 64 * i, brow + k0);
@@ -1002,7 +1025,9 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
             const bool valid = m < ti.mvalid;
             const int wrow0 = ti.m0 + q * 32;
             const bool full_box = wrow0 + 32 <= ti.mvalid;
-            const bool dwt = DW2 && ti.dw;
+            const bool dwt = DW2 && ti.dw, sec = SH && ti.sec;
+            const int N = sec ? p2.N : p.N;
+            void* const out0 = sec ? p2.out0 : p.out0;
             const int64_t grow0 = (VAR_K || dwt) ? (int64_t)ti.we * (dwt ? p2.Mout : p.Mout) + wrow0
                                                  : ti.out_row + wrow0;
             const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
@@ -1052,7 +1077,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
             } else if (SWAP && ti.ntok) {
                 if (!wait_bar(tfull_bar(acc), acc_phase)) break;
                 fence_after();
-                swapped_epilogue<EPI>(p, ti, (int)rank, q, lane, tbase, half * 32, SPLIT * 32);
+                swapped_epilogue<EPI>(N, p.F, out0, p.aux, ti, (int)rank, q, lane, tbase, half * 32, SPLIT * 32);
             } else if constexpr (EPI == EPI_SWIGLU_BWD) {
                 // dA in TMEM. G and U of each 32-column chunk arrive by TMA in one of two
                 // staging buffers (the next chunk's load is in flight while this one is
@@ -1117,9 +1142,10 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                 fence_after();
                 if constexpr (EPI == EPI_SWIGLU_FWD) {
                     // accumulator columns [0,128) = G, [128,256) = U of features n0 .. n0+127
-                    const int F = p.F;
-                    __nv_bfloat16* hgu = (__nv_bfloat16*)p.out0 + (ti.out_row + m) * (int64_t)(2 * F);
-                    __nv_bfloat16* actp = (__nv_bfloat16*)p.out1 + (ti.out_row + m) * (int64_t)F;
+                    const int F = sec ? p2.F : p.F;
+                    const CUtensorMap *mO0 = sec ? &tmO2 : &tmO0, *mO1 = sec ? &tmX2 : &tmO1;
+                    __nv_bfloat16* hgu = (__nv_bfloat16*)out0 + (ti.out_row + m) * (int64_t)(2 * F);
+                    __nv_bfloat16* actp = (__nv_bfloat16*)(sec ? p2.out1 : p.out1) + (ti.out_row + m) * (int64_t)F;
 #pragma unroll 1
                     for (int c = half * (128 / SPLIT); c < (half + 1) * (128 / SPLIT); c += 32) {
                         float g[32], u[32], a[32];
@@ -1129,7 +1155,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                         for (int i = 0; i < 32; ++i) a[i] = __fdividef(g[i], 1.0f + __expf(-g[i])) * u[i];
                         const int f = ti.n0 + c;
                         const float* vals[3] = {g, u, a};
-                        const CUtensorMap* maps[3] = {&tmO0, &tmO0, &tmO1};
+                        const CUtensorMap* maps[3] = {mO0, mO0, mO1};
                         const int cols[3] = {f, F + f, f};
                         __nv_bfloat16* direct[3] = {hgu + f, hgu + F + f, actp + f};
                         emit(3, vals, maps, cols, direct);
@@ -1165,9 +1191,9 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                     if (VAR_K)
                         out = (__nv_bfloat16*)p.out0 + (int64_t)ti.we * p.Mout * p.N + (int64_t)m * p.N;
                     else
-                        out = (__nv_bfloat16*)p.out0 + (ti.out_row + m) * (int64_t)p.N;
+                        out = (__nv_bfloat16*)out0 + (ti.out_row + m) * (int64_t)N;
 #pragma unroll 1
-                    for (int c = half * (BN / SPLIT); c < (half + 1) * (BN / SPLIT) && ti.n0 + c < p.N; c += 32) {
+                    for (int c = half * (BN / SPLIT); c < (half + 1) * (BN / SPLIT) && ti.n0 + c < N; c += 32) {
                         float y[32];
                         if (ti.k_iters > 0) {
                             tmem_ld32(tbase + c, y);
@@ -1176,7 +1202,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                             for (int i = 0; i < 32; ++i) y[i] = 0.f;
                         }
                         const float* vals[1] = {y};
-                        const CUtensorMap* maps[1] = {&tmO0};
+                        const CUtensorMap* maps[1] = {sec ? &tmO2 : &tmO0};
                         const int cols[1] = {ti.n0 + c};
                         __nv_bfloat16* direct[1] = {out + ti.n0 + c};
                         emit(1, vals, maps, cols, direct);
@@ -1293,14 +1319,16 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
                           const CUtensorMap& mo1, const Params& p, int64_t tiles_ub,
                           cudaStream_t s, const CUtensorMap* ma2 = nullptr,
                           const CUtensorMap* mb2 = nullptr, const CUtensorMap* mo2 = nullptr,
-                          const Params* p2 = nullptr, const CUtensorMap* mas = nullptr) {
+                          const Params* p2 = nullptr, const CUtensorMap* mas = nullptr, const CUtensorMap* mx2 = nullptr) {
     auto kern = grouped_gemm_kernel<BN, B_MN, VAR_K, EPI, PAIR, DW2, OCC, EW>;
     const CUtensorMap& A2 = ma2 ? *ma2 : ma;
     const CUtensorMap& B2 = mb2 ? *mb2 : mb;
     const CUtensorMap& O2 = mo2 ? *mo2 : mo0;
     const CUtensorMap& AS = mas ? *mas : ma;  // boxes of swapped tiles (M-variable pairs)
+    const CUtensorMap& X2 = mx2 ? *mx2 : mo0;
     Params P1 = p;
     Params P2 = p2 ? *p2 : p;
+    if (!p2) P2.G = 0;  // no second problem
     constexpr int NPAIR = PAIR ? 2 : 1;
     constexpr int KB = kblock_rows(VAR_K, PAIR, EPI, BN);
     constexpr int STB = (BM * KB * 2 + BN / NPAIR * KB * 2) * kblocks_per_stage(EPI, BN, PAIR, VAR_K, DW2, OCC);  // bytes of one operand stage
@@ -1355,11 +1383,11 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 2;
-        return cudaLaunchKernelEx(&cfg, kern, ma, mb, mo0, mo1, AS, P1, A2, B2, O2, P2);
+        return cudaLaunchKernelEx(&cfg, kern, ma, mb, mo0, mo1, AS, P1, A2, B2, O2, X2, P2);
     } else {
         const int grid = (int)std::min<int64_t>(tiles_ub, (int64_t)OCC * sm_count());
         P1.band = P2.band = band_for(grid);
-        (void)launch_pdl(kern, dim3(grid), dim3(gemm_threads(EW)), smem, s, ma, mb, mo0, mo1, AS, P1, A2, B2, O2, P2);
+        (void)launch_pdl(kern, dim3(grid), dim3(gemm_threads(EW)), smem, s, ma, mb, mo0, mo1, AS, P1, A2, B2, O2, X2, P2);
         return cudaGetLastError();
     }
 }
@@ -1394,7 +1422,7 @@ static int64_t expected_tiles(const GroupRows& gr, int G, int tile) {
 // (d < 2048) the epilogue bounds it and single-CTA tiles (fused with dW2 in one launch) are
 // faster; from d = 2048 the mainloop dominates and pairs win (d = 4096: the expert backward
 // 17.8 -> 17.2 ms; d = 1024: +4%).
-bool gemm_m_uses_pairs(const GemmMArgs& g) {
+bool gemm_m_uses_pairs(const GemmMArgs& g, const GemmMArgs* second) {
     using namespace tc;
     if (g.N % 128 != 0) return false;  // 256-wide pair tiles, the last one possibly ragged
     if (g_pairs == MOE_PAIRS_ALL) return true;
@@ -1407,8 +1435,12 @@ bool gemm_m_uses_pairs(const GemmMArgs& g) {
     }
     const bool wide = g.N % 256 == 0;  // (a GEMM1 tile's 256 columns are 128 features, gate and up)
     const int64_t sms = sm_count(), pairs = sms / 2;
-    const int64_t tp = expected_tiles(g.rows, g.G, 2 * BM) * ((g.N + 255) / 256);
-    const int64_t ts = expected_tiles(g.rows, g.G, BM) * (wide ? g.N / 256 : g.N / 128);
+    int64_t tp = 0, ts = 0;
+    for (const GemmMArgs* q : {&g, second}) {
+        if (!q) continue;
+        tp += expected_tiles(q->rows, q->G, 2 * BM) * ((q->N + 255) / 256);
+        ts += expected_tiles(q->rows, q->G, BM) * (wide ? q->N / 256 : q->N / 128);
+    }
     const int64_t rp = (tp + pairs - 1) / pairs, rs = (ts + sms - 1) / sms;
     return g.K < 512 ? rp < rs || (rp == rs && rp >= 4) : rp * 100 <= rs * (wide ? 130 : 105);
 }
@@ -1430,12 +1462,10 @@ bool gemm_k_uses_pairs(const GemmKArgs& g) {
     return (tp + pairs - 1) / pairs * 49 <= (ts + sms - 1) / sms * (wide ? 67 : 45);
 }
 
-// M-variable grouped GEMM (forward, dA, dX).
-cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s) {
-    if (!bf16) return launch_gemm_m_f32(g, s);
-    using namespace tc;
-    if (g.G > MAX_GROUPS) return cudaErrorInvalidValue;
-    Params p{};
+// What launch_gemm_m and its second problem share: the kernel's parameters, and the rows of
+// A's and the outputs' 2D views (OFFSETS: all routed rows; UNIFORM: groups * stride, or rows).
+static tc::Params m_params(const GemmMArgs& g) {
+    tc::Params p{};
     p.offsets = g.rows.offsets;
     p.rows = g.rows.offsets ? 0 : g.rows.rows;
     p.a_stride = g.rows.a_stride;
@@ -1447,60 +1477,82 @@ cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s) {
     p.out0 = g.out0;
     p.out1 = g.out1;
     p.aux = g.aux;
-    p.wait_ns = g_wait_ns;
+    p.wait_ns = tc::g_wait_ns;
     p.gexp = g.group_expert;
     p.a_row_bytes = (int64_t)g.K * 2;
     p.b_all_bytes = (int64_t)g.N * (g.b_kmajor ? g.K : (g.b_rows ? g.b_rows : g.K)) * 2;
-    // A rows in the 2D view: OFFSETS -> all routed rows; UNIFORM -> groups * stride (or rows)
-    const int64_t a_rows = g.rows.offsets ? (int64_t)g.rows.rows
-                                          : std::max<int64_t>(g.rows.rows, (int64_t)(g.G - 1) * g.rows.a_stride + g.rows.rows);
-    const int64_t mt_ub = g.rows.offsets ? ((int64_t)g.rows.rows + BM - 1) / BM + g.G
-                                         : (int64_t)g.G * ((g.rows.rows + BM - 1) / BM);
-    // pair tiles (256 rows)
-    const int64_t pt_ub = g.rows.offsets ? ((int64_t)g.rows.rows + 2 * BM - 1) / (2 * BM) + g.G
-                                         : (int64_t)g.G * ((g.rows.rows + 2 * BM - 1) / (2 * BM));
-    const bool pair = gemm_m_uses_pairs(g);
-    // output rows in the 2D view of the outputs
-    const int64_t o_rows = g.rows.offsets ? (int64_t)g.rows.rows
-                                          : std::max<int64_t>(g.rows.rows, (int64_t)(g.G - 1) * g.rows.out_stride + g.rows.rows);
+    if (g.epi == EPI_SWIGLU_FWD) p.F = g.N / 2;
+    p.b_group_rows = g.b_kmajor ? g.N : (g.b_rows ? g.b_rows : g.K);
+    return p;
+}
+static int64_t view_rows(const GemmMArgs& g, int64_t stride) {
+    return g.rows.offsets ? (int64_t)g.rows.rows : std::max<int64_t>(g.rows.rows, (int64_t)(g.G - 1) * stride + g.rows.rows);
+}
+// most tiles of `tile` rows that the groups can make
+static int64_t max_tiles(const GemmMArgs& g, int tile) {
+    return g.rows.offsets ? ((int64_t)g.rows.rows + tile - 1) / tile + g.G : (int64_t)g.G * ((g.rows.rows + tile - 1) / tile);
+}
+
+// M-variable grouped GEMM (forward, dA, dX). `second`: another one of the same kind (forward
+// GEMMs; uniform groups; for a plain store of the same N) whose tiles follow in the launch.
+cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s, const GemmMArgs* second) {
+    if (!bf16) {
+        const cudaError_t e = launch_gemm_m_f32(g, s);
+        return e == cudaSuccess && second ? launch_gemm_m_f32(*second, s) : e;
+    }
+    using namespace tc;
+    if (g.G > MAX_GROUPS || (second && second->G > MAX_GROUPS)) return cudaErrorInvalidValue;
+    Params p = m_params(g);
+    const int64_t a_rows = view_rows(g, g.rows.a_stride), o_rows = view_rows(g, g.rows.out_stride);
+    const int64_t mt_ub = max_tiles(g, BM), pt_ub = max_tiles(g, 2 * BM);
+    const bool pair = gemm_m_uses_pairs(g, second);
     CUtensorMap ma, mb, mo0, mo1, mas;  // mas: A in boxes of 32 rows (swapped tiles)
     if (!make_map(&ma, g.a, g.K, a_rows, BM)) return cudaErrorInvalidValue;
     if (pair && !make_map(&mas, g.a, g.K, a_rows, 32)) return cudaErrorInvalidValue;
     const bool wide_epi = g.K < kWideEpiK;
-    if (g.epi == EPI_SWIGLU_FWD) {
-        const int F = g.N / 2;
-        p.F = F;
-        p.b_group_rows = 2 * (int64_t)F;
-        if (!make_map(&mb, g.b, g.K, (int64_t)g.G * 2 * F, 128)) return cudaErrorInvalidValue;
-        if (!make_map(&mo0, g.out0, 2 * (int64_t)F, o_rows, 0, true)) return cudaErrorInvalidValue;
-        if (!make_map(&mo1, g.out1, F, o_rows, 0, true)) return cudaErrorInvalidValue;
-        if (pair && wide_epi) return launch<256, false, false, EPI_SWIGLU_FWD, true, false, 1, 8>(ma, mb, mo0, mo1, p, pt_ub * (F / 128), s);
-        if (pair) return launch<256, false, false, EPI_SWIGLU_FWD, true>(ma, mb, mo0, mo1, p, pt_ub * (F / 128), s);
-        if (wide_epi) return launch<256, false, false, EPI_SWIGLU_FWD, false, false, 1, 8>(ma, mb, mo0, mo1, p, mt_ub * (F / 128), s);
-        return launch<256, false, false, EPI_SWIGLU_FWD>(ma, mb, mo0, mo1, p, mt_ub * (F / 128), s);
-    }
-    if (g.epi == EPI_STORE && g.b_kmajor) {  // Y = A W2^T: B = W2[e] as [N=d, K=F]
-        p.b_group_rows = g.N;
-        if (!make_map(&mo0, g.out0, g.N, o_rows, 0, true)) return cudaErrorInvalidValue;
-        if (pair) {
-            if (!make_map(&mb, g.b, g.K, (int64_t)g.G * g.N, 128)) return cudaErrorInvalidValue;
-            if (wide_epi)
-                return launch<256, false, false, EPI_STORE, true, false, 1, 8>(ma, mb, mo0, mo0, p, pt_ub * ((g.N + 255) / 256),
-                                                                               s, nullptr, nullptr, nullptr, nullptr, &mas);
-            return launch<256, false, false, EPI_STORE, true>(ma, mb, mo0, mo0, p, pt_ub * ((g.N + 255) / 256), s, nullptr,
-                                                              nullptr, nullptr, nullptr, &mas);
+    if (g.b_kmajor) {  // forward: SwiGLU (B = gate rows then up rows), or Y = A W2^T (B = W2[e] as [N=d, K=F])
+        const bool fwd = g.epi == EPI_SWIGLU_FWD;
+        // tile columns, and rows of one B box
+        const int bn = fwd || pair || g.N % 256 == 0 ? 256 : 128, brows = fwd || pair ? 128 : bn;
+        auto maps = [&](const GemmMArgs& q, CUtensorMap* b, CUtensorMap* o0, CUtensorMap* o1) {
+            const int64_t rows = view_rows(q, q.rows.out_stride);
+            return make_map(b, q.b, q.K, (int64_t)q.G * q.N, brows) && make_map(o0, q.out0, q.N, rows, 0, true) &&
+                   (!fwd || make_map(o1, q.out1, q.N / 2, rows, 0, true));
+        };
+        auto tiles = [&](const GemmMArgs& q) { return max_tiles(q, pair ? 2 * BM : BM) * ((q.N + bn - 1) / bn); };
+        if (!maps(g, &mb, &mo0, &mo1)) return cudaErrorInvalidValue;
+        if (!fwd) mo1 = mo0;
+        int64_t n = tiles(g);
+        CUtensorMap a2, b2, o2, x2;
+        Params p2;
+        const Params* pp2 = nullptr;
+        if (second) {
+            const int64_t rows2 = view_rows(*second, second->rows.a_stride);
+            if (!make_map(&a2, second->a, second->K, rows2, BM) || !maps(*second, &b2, &o2, &x2)) return cudaErrorInvalidValue;
+            if (!fwd && !make_map(&x2, second->a, second->K, rows2, 32)) return cudaErrorInvalidValue;
+            p2 = m_params(*second);
+            pp2 = &p2;
+            n += tiles(*second);
         }
-        if (g.N % 256 == 0) {
-            if (!make_map(&mb, g.b, g.K, (int64_t)g.G * g.N, 256)) return cudaErrorInvalidValue;
-            if (wide_epi) return launch<256, false, false, EPI_STORE, false, false, 1, 8>(ma, mb, mo0, mo0, p, mt_ub * (g.N / 256), s);
-            return launch<256, false, false, EPI_STORE>(ma, mb, mo0, mo0, p, mt_ub * (g.N / 256), s);
+        const CUtensorMap *A2 = pp2 ? &a2 : nullptr, *B2 = pp2 ? &b2 : nullptr, *O2 = pp2 ? &o2 : nullptr,
+                          *X2 = pp2 ? &x2 : nullptr, *as = pair ? &mas : nullptr;
+#define MOE_FWD(BN, EPI, PAIR, EW) \
+    return launch<BN, false, false, EPI, PAIR, false, 1, EW>(ma, mb, mo0, mo1, p, n, s, A2, B2, O2, pp2, as, X2)
+        if (fwd) {
+            if (pair && wide_epi) MOE_FWD(256, EPI_SWIGLU_FWD, true, 8);
+            if (pair) MOE_FWD(256, EPI_SWIGLU_FWD, true, 4);
+            if (wide_epi) MOE_FWD(256, EPI_SWIGLU_FWD, false, 8);
+            MOE_FWD(256, EPI_SWIGLU_FWD, false, 4);
         }
-        if (!make_map(&mb, g.b, g.K, (int64_t)g.G * g.N, 128)) return cudaErrorInvalidValue;
-        if (wide_epi) return launch<128, false, false, EPI_STORE, false, false, 1, 8>(ma, mb, mo0, mo0, p, mt_ub * (g.N / 128), s);
-        return launch<128, false, false, EPI_STORE>(ma, mb, mo0, mo0, p, mt_ub * (g.N / 128), s);
+        if (pair && wide_epi) MOE_FWD(256, EPI_STORE, true, 8);
+        if (pair) MOE_FWD(256, EPI_STORE, true, 4);
+        if (bn == 256 && wide_epi) MOE_FWD(256, EPI_STORE, false, 8);
+        if (bn == 256) MOE_FWD(256, EPI_STORE, false, 4);
+        if (wide_epi) MOE_FWD(128, EPI_STORE, false, 8);
+        MOE_FWD(128, EPI_STORE, false, 4);
+#undef MOE_FWD
     }
     // MN-major B: weights stored [G*K, N] (or [G*b_rows, N])
-    p.b_group_rows = g.b_rows ? g.b_rows : g.K;
     const bool slim = g.slim && g.epi == EPI_STORE && g.N % 128 == 0;
     const int kps = kblocks_per_stage(g.epi, pair || g.N % 256 == 0 ? 256 : 128, pair, false, false, slim ? 2 : 1);
     if (!make_map(&mb, g.b, g.N, (int64_t)g.G * p.b_group_rows, BK * kps)) return cudaErrorInvalidValue;

@@ -367,7 +367,6 @@ moe_status moe_expert_ffn_fwd(const moe_config* cfg, const void* x_perm, const i
     g1.epi = EPI_SWIGLU_FWD;
     g1.out0 = h_gu;
     g1.out1 = act;
-    if ((st = cuda_status(launch_gemm_m(g1, bf16, s), "expert gemm1"))) return st;
     GemmMArgs g2{};
     g2.group_expert = group_expert;
     g2.G = E;
@@ -380,10 +379,10 @@ moe_status moe_expert_ffn_fwd(const moe_config* cfg, const void* x_perm, const i
     g2.K = F;
     g2.epi = EPI_STORE;
     g2.out0 = y_perm;
-    if ((st = cuda_status(launch_gemm_m(g2, bf16, s), "expert gemm2"))) return st;
+    // the shared experts' GEMMs run in the routed experts' launches (bf16)
+    GemmMArgs h1 = g1, h2 = g2;
     if (S) {
         const int Fs = cfg->d_ff_shared;
-        GemmMArgs h1 = g1;
         h1.group_expert = nullptr;  // shared experts: one group per expert
         h1.G = S;
         h1.rows = GroupRows{nullptr, (int)T, 0, 0, T};
@@ -393,9 +392,7 @@ moe_status moe_expert_ffn_fwd(const moe_config* cfg, const void* x_perm, const i
         h1.N = 2 * Fs;
         h1.out0 = h_gu_sh;
         h1.out1 = act_sh;
-        if ((st = cuda_status(launch_gemm_m(h1, bf16, s), "shared gemm1"))) return st;
-        GemmMArgs h2 = g2;
-        h2.group_expert = nullptr;  // shared experts: one group per expert
+        h2.group_expert = nullptr;
         h2.G = S;
         h2.rows = GroupRows{nullptr, (int)T, T, 0, T};
         h2.a = act_sh;
@@ -403,9 +400,9 @@ moe_status moe_expert_ffn_fwd(const moe_config* cfg, const void* x_perm, const i
         h2.b_group_elems = (int64_t)d * Fs;
         h2.K = Fs;
         h2.out0 = y_sh;
-        if ((st = cuda_status(launch_gemm_m(h2, bf16, s), "shared gemm2"))) return st;
     }
-    return MOE_OK;
+    if ((st = cuda_status(launch_gemm_m(g1, bf16, s, S ? &h1 : nullptr), "expert gemm1"))) return st;
+    return cuda_status(launch_gemm_m(g2, bf16, s, S ? &h2 : nullptr), "expert gemm2");
 }
 
 moe_status moe_combine_fwd(const moe_config* cfg, const void* y_perm, const float* topk_w,

@@ -139,13 +139,14 @@ struct GemmKArgs {
     const int32_t* group_expert = nullptr;  // device [G]: group g's output is group_expert[g]'s
 };
 
-cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s);
+// second: a further GEMM of the same forward kind with uniform groups, in the same launch (bf16)
+cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s, const GemmMArgs* second = nullptr);
 cudaError_t launch_gemm_k(const GemmKArgs& g, bool bf16, cudaStream_t s);
 // bf16: an M-variable GEMM (MN-major B) and a K-variable GEMM over the same groups in
 // one persistent launch (the second problem's tiles after the first's)
 cudaError_t launch_gemm_mk(const GemmMArgs& m, const GemmKArgs& k, cudaStream_t s);
 // whether launch_gemm_m runs this GEMM as CTA-pair tiles (bf16)
-bool gemm_m_uses_pairs(const GemmMArgs& g);
+bool gemm_m_uses_pairs(const GemmMArgs& g, const GemmMArgs* second = nullptr);
 bool gemm_k_uses_pairs(const GemmKArgs& g);
 void set_wait_limit_ns(uint64_t ns);
 void set_gemm_pairs(int mode);  // MOE_PAIRS_*

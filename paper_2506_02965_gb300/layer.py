@@ -338,11 +338,12 @@ class MoELayer:
         unpermute-reduce 1; the expert backward as moe_expert_ffn_bwd_kernels reports it
         (its shared experts included); router backward: bf16 5 (dlogits, chunk dbias,
         dW_r partial GEMM, reduce, dx_router GEMM), fp32 4 (dlogits, partials, reduce,
-        dx_router GEMM); shared experts add 2 to the forward."""
+        dx_router GEMM); shared experts add 2 to an fp32 forward (bf16: they run in the
+        routed experts' launches)."""
         bf16 = self.shape.dtype == "bf16"
         few = not self.owner_grouped and self.shape.T <= 1024
         return ((9 if few else 10) + L.moe_expert_ffn_bwd_kernels(self.cfg) + (5 if bf16 else 4)
-                + (2 if self.shape.n_shared else 0))
+                + (2 if self.shape.n_shared and not bf16 else 0))
 
     def check_status(self, stream=None):
         code = L.moe_device_status(stream)
