@@ -36,7 +36,8 @@ __host__ __device__ constexpr int kblock_rows(bool var_k, bool pair, int epi, in
 // dA at d = 3072, F = 640 46 -> 37 us, GEMM2 at d = 384 35 -> 28 us); else 1: the
 // SwiGLU-backward pairs measured faster with six stages, and 256-wide single-CTA tiles lose
 // with two stages of 96 KiB (GEMM1 47 -> 53 us)
-__host__ __device__ constexpr int kblocks_per_stage(int epi, int bn, bool pair, bool var_k, bool dw2, int occ) {
+__host__ __device__ constexpr int kblocks_per_stage(int epi, int bn, bool pair, bool var_k, bool dw2, int occ, int ar) {
+    if (epi == EPI_ROUTE && ar < BM) return bn <= 32 ? 8 : 4;  // one copy each of A and B (below)
     if (epi == EPI_ROUTE) return bn <= 64 ? 2 : 1;
     if (var_k || dw2 || occ > 1) return 1;
     if (pair) return epi != EPI_SWIGLU_BWD ? 2 : 1;
@@ -97,9 +98,18 @@ struct Params {
 __host__ __device__ constexpr int epi_extra_bytes(int epi) {
     return epi == EPI_ROUTE ? 64 * 64 * 4 : epi_stage_bytes(epi);
 }
-__host__ __device__ constexpr int num_stages(uint32_t stage_bytes, int epi, int occ = 1) {
+// Router tiles of at most AR < BM token rows keep only AR rows per A box in shared memory and
+// fetch four or eight k-blocks of an operand in one 3D copy: a short batch, streamed by few CTAs, is
+// bound by the fixed cost of its copies (90 ns each) and stages, not by bytes in flight (deeper
+// rings alone changed nothing). With the epilogue below: 64 tokens, d = 2048, E = 64 24.7 -> 13.9
+// us; 33, 4096, 8 22.0 -> 16.3; 4, 1024, 16 10.2 -> 7.7; 2999, 2048, 64 24.9 -> 18.7. At 4096
+// tokens, d = 1024 equal (11.5), so not above 32 rows a tile, where bytes bound it.
+// The MMA still reads BM rows per box: what follows the box (bytes that only reach accumulator
+// rows that nobody reads), after the last box up to this many bytes past the ring.
+__host__ __device__ constexpr int mma_overread(int ar) { return ar < BM ? BM * 128 : 0; }
+__host__ __device__ constexpr int num_stages(uint32_t stage_bytes, int epi, int occ, int ar) {
     const int per_cta = occ == 1 ? 227 * 1024 : 112 * 1024;
-    const int budget = per_cta - 1024 - 1024 - epi_extra_bytes(epi);  // dyn. smem, align, static
+    const int budget = per_cta - 1024 - 1024 - epi_extra_bytes(epi) - mma_overread(ar);  // dyn. smem, align, static
     const int n = budget / (int)stage_bytes;
     return n > 12 ? 12 : n;
 }
@@ -207,6 +217,116 @@ __device__ __forceinline__ void route_epilogue(const Params& p, const Tile& ti, 
     if (p.normalize) {
 #pragma unroll 1
         for (int j = 0; j < k; ++j) tw_out[j] = tw_out[j] / wsum;
+    }
+}
+
+// Whether any thread of the four epilogue warps passes true: the same answer to all of them.
+__device__ __forceinline__ bool epilogue_any(bool x) {
+    uint32_t r;
+    __syncwarp();
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.red.or.pred q, 1, 128, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+        : "=r"(r)
+        : "r"((uint32_t)x)
+        : "memory");
+    return r != 0;
+}
+
+// The same gating for a tile of at most 32 tokens, whose accumulator rows are all in one
+// warp's TMEM quarter: that warp lays the raw logits out in shared memory (s_z, rows of
+// BN + 1) and all four take eight lanes a token (one thread a token took over 10 us at
+// E = 64, k = 6). The picks are those of route_epilogue, NaN logits included: of the experts
+// not taken the first if its logit is NaN, else the largest that is not, lower ids first.
+template <int BN, int AR>
+__device__ __forceinline__ void route_epilogue_short(const Params& p, const Tile& ti, int q, int wid, int lane,
+                                                     uint32_t tbase, float* s_z, int* hist) {
+    constexpr int V = BN / 8;
+    if (q == 0) {
+        float z[BN];
+        if constexpr (BN == 16) {
+            tmem_ld16(tbase, z);
+        } else {
+#pragma unroll
+            for (int c = 0; c < BN / 32; ++c) tmem_ld32(tbase + 32 * c, z + 32 * c);
+        }
+        if (lane < AR) {
+#pragma unroll
+            for (int e = 0; e < BN; ++e) s_z[lane * (BN + 1) + e] = z[e];
+        }
+    }
+    (void)epilogue_any(false);  // the logits are there
+    const int E = p.E, k = p.k, l8 = lane & 7;
+    const float* bias = (const float*)p.aux;
+#pragma unroll 1
+    for (int r0 = 0; r0 < AR; r0 += 16) {
+        const int row = r0 + wid * 4 + (lane >> 3);
+        const bool valid = ti.m0 + row < ti.mvalid;
+        const int64_t t = ti.out_row + ti.m0 + row;
+        float* zr = s_z + row * (BN + 1);
+        float z[V], ez[V], mx = -3.402823466e38f, sum = 0.f;
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            const int e = l8 + 8 * j;
+            z[j] = zr[e];
+            if (e < E) {
+                if (bias) z[j] += bias[ti.g * E + e];
+                mx = fmaxf(mx, z[j]);
+            }
+            zr[e] = z[j];
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            ez[j] = l8 + 8 * j < E ? expf(z[j] - mx) : 0.f;
+            sum += ez[j];
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            const int e = l8 + 8 * j;
+            if (valid && e < E) {
+                ((float*)p.out0)[t * E + e] = z[j];
+                ((float*)p.out1)[t * E + e] = ez[j] / sum;
+            }
+        }
+        __syncwarp();
+        uint64_t taken = 0;
+        float wsum = 0.f;
+#pragma unroll 1
+        for (int i = 0; i < k; ++i) {
+            const int first = __ffsll((long long)~taken) - 1;
+            // (logit in an order-preserving unsigned code, BN - e): the largest is the pick
+            uint64_t best = 0;
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                const int e = l8 + 8 * j;
+                const uint32_t u = __float_as_uint(z[j] + 0.f);  // -0 counts as 0
+                uint32_t key = (u & 0x80000000u) ? ~u : u | 0x80000000u;
+                if (z[j] != z[j]) key = e == first ? 0xffffffffu : 0u;
+                const uint64_t c = ((uint64_t)key << 32) | (uint32_t)(BN - e);
+                if (e < E && !((taken >> e) & 1ull) && c > best) best = c;
+            }
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                const uint64_t other = __shfl_xor_sync(0xffffffffu, best, o);
+                best = other > best ? other : best;
+            }
+            const int bi = BN - (int)(uint32_t)best;
+            taken |= 1ull << bi;
+            const float w = expf(zr[bi] - mx) / sum;
+            wsum += w;
+            if (valid && l8 == 0) {
+                p.topk_idx[t * k + i] = bi;
+                p.topk_w[t * k + i] = w;
+                atomicAdd(&hist[ti.g * E + bi], 1);
+            }
+        }
+        if (p.normalize && valid && l8 == 0) {
+#pragma unroll 1
+            for (int i = 0; i < k; ++i) p.topk_w[t * k + i] = p.topk_w[t * k + i] / wsum;
+        }
     }
 }
 
@@ -406,7 +526,7 @@ __device__ __forceinline__ void swapped_epilogue(int N, int F, void* out0, const
 // their own they are short and latency-bound (64 tokens, two of d = 2048, Fs = 1408: 18.7 and
 // 12.5 us for 35 MB of weights): the forward of 64 tokens with 64 such routed experts
 // 264 -> 233 us (of 2999 tokens, where they had rounds of their own, 0.5% less).
-template <int BN, bool B_MN, bool VAR_K, int EPI, bool PAIR = false, bool DW2 = false, int OCC = 1, int EW = 4>
+template <int BN, bool B_MN, bool VAR_K, int EPI, bool PAIR = false, bool DW2 = false, int OCC = 1, int EW = 4, int AR = BM>
 __global__ void __launch_bounds__(gemm_threads(EW), OCC)
     grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                         const __grid_constant__ CUtensorMap tmB,
@@ -422,6 +542,8 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
     static_assert(!DW2 || (B_MN && !VAR_K && !PAIR && BN == 256), "fused: M-variable, MN-major B");
     static_assert(OCC == 1 || (!PAIR && !DW2 && 2 * BN * OCC <= 512), "shared SMs: single-CTA tiles, TMEM for all");
     static_assert(EW == 4 || (EW == 8 && !DW2 && (EPI == EPI_STORE || EPI == EPI_SWIGLU_FWD)), "epilogue warps");
+    constexpr bool SHORT = AR < BM;
+    static_assert(AR == BM || (EPI == EPI_ROUTE && (AR == 16 || AR == 32) && BN <= 64), "short A boxes: the router");
     constexpr int NBUF = EPI_BOXES / EW;  // output boxes of one epilogue warp
     constexpr bool A_MN = VAR_K;
     constexpr bool SWAP = PAIR && !VAR_K && EPI != EPI_SWIGLU_FWD;  // swapped tiles possible
@@ -429,15 +551,15 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
     constexpr int BNL = BN / NPAIR;  // B rows held by this CTA
     constexpr int BMP = BM * NPAIR;  // rows of one (pair) tile
     constexpr int KB = kblock_rows(VAR_K, PAIR, EPI, BN);  // contraction rows per k-block
-    constexpr int KPS = kblocks_per_stage(EPI, BN, PAIR, VAR_K, DW2, OCC);
+    constexpr int KPS = kblocks_per_stage(EPI, BN, PAIR, VAR_K, DW2, OCC, AR);
     constexpr uint32_t ATOM = KB * 128;         // bytes of one 64-wide MN-major box
     constexpr uint32_t ATOM_B = ATOM * KPS;     // of B's: one box holds all of a stage's k-blocks
-    constexpr uint32_t A_BOX = BM * KB * 2;   // one k-block of A
+    constexpr uint32_t A_BOX = AR * KB * 2;   // one k-block of A
     constexpr uint32_t B_BOX = BNL * KB * 2;  // one k-block of B
     constexpr uint32_t A_BYTES = A_BOX * KPS;
     constexpr uint32_t B_BYTES = B_BOX * KPS;
     constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
-    constexpr int NST = num_stages(STAGE_BYTES, EPI, OCC);
+    constexpr int NST = num_stages(STAGE_BYTES, EPI, OCC, AR);
     constexpr uint32_t IDESC = instr_desc<BN, A_MN, B_MN, BMP>();
     constexpr uint32_t IDESC_DW = instr_desc<BN, true, true, BM>();
     constexpr int TMEM_COLS = (2 * BN <= 32) ? 32 : (2 * BN <= 64) ? 64 : (2 * BN <= 128) ? 128 : (2 * BN <= 256) ? 256 : 512;
@@ -620,7 +742,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
             ti.a_row = a0;
             ti.b_row = 0;
             ti.out_row = o0;
-            ti.k_iters = (SH && ti.sec ? p2.K : p.K) / (BK * KPS);
+            ti.k_iters = ((SH && ti.sec ? p2.K : p.K) + (SHORT ? BK * KPS - 1 : 0)) / (BK * KPS);  // (zero-filled)
             ti.last_rows = BK;
             if constexpr (SWAP) {
                 const int v = (int)nrows - mt * BMP;
@@ -734,7 +856,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                 // a swapped tile's rows: half in each CTA, in boxes of 32
                 const int trows = SWAP ? ti.ntok / 2 : 0;
                 uint32_t tile_bytes = NPAIR * STAGE_BYTES;  // per stage, both CTAs of a pair
-                if (EPI == EPI_ROUTE) tile_bytes = (uint32_t)p.tile_rows * 128u * KPS + B_BYTES;  // A boxes of tile_rows rows
+                if (EPI == EPI_ROUTE && !SHORT) tile_bytes = (uint32_t)p.tile_rows * 128u * KPS + B_BYTES;  // A boxes of tile_rows rows
                 if (SWAP && trows) tile_bytes = NPAIR * (B_BYTES + (uint32_t)((trows + 31) / 32) * (32u * 128u * KPS));
                 // the tile's coordinates: A (first row, or contraction row), B (row, or contraction row)
                 const int arow = (int)ti.a_row + ((A_MN || dw) ? 0 : ti.m0 + (int)rank * trows);
@@ -770,6 +892,10 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                         }
                     }
                     const int k0 = kb * KB * KPS;
+                    if constexpr (SHORT) {
+                        tma_load_3d(sa, &tmA, fb, 0, arow, kb * KPS);
+                        tma_load_3d(sb, &tmB, fb, 0, brow, kb * KPS);
+                    } else {
                     if (!A_MN && !dw) {
                         if (SWAP && trows) {
                             for (int r = 0; r < trows; r += 32)
@@ -795,6 +921,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
 #pragma unroll
                         for (int i = 0; i < BNL / 64; ++i)
                             load(sb + i * ATOM_B, mB, fb, ti.n0 + (int)rank * BNL + 64 * i, brow + k0);
+                    }
                     }
                     issued |= 1u << stage;
                     issued_par = (issued_par & ~(1u << stage)) | (phase << stage);
@@ -1138,7 +1265,9 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                 }
                 if (stop) break;
             } else {
-                if (!wait_bar(tfull_bar(acc), acc_phase)) break;
+                const bool got = wait_bar(tfull_bar(acc), acc_phase);
+                // (short router tiles: the epilogue warps meet per tile, and give up together)
+                if (SHORT ? epilogue_any(!got) : !got) break;
                 fence_after();
                 if constexpr (EPI == EPI_SWIGLU_FWD) {
                     // accumulator columns [0,128) = G, [128,256) = U of features n0 .. n0+127
@@ -1164,7 +1293,9 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                     // the per-(party, expert) counts: a shared-memory histogram when P E fits
                     // (hist_n > 0), else straight to the global counts
                     int* hist = p.hist_n ? route_hist : p.counts;
-                    if constexpr (BN <= 64) route_epilogue<BN>(p, ti, m, valid, tbase, hist);
+                    if constexpr (SHORT)
+                        route_epilogue_short<BN, AR>(p, ti, q, warp - 2, lane, tbase, (float*)(stage_out + 4 * p.hist_n), hist);
+                    else if constexpr (BN <= 64) route_epilogue<BN>(p, ti, m, valid, tbase, hist);
                     else route_epilogue_wide<BN>(p, ti, m, valid, tbase, hist);
                 } else if constexpr (EPI == EPI_DWR) {
                     // one token chunk's partial router gradient: accumulator row m is model
@@ -1292,6 +1423,20 @@ static bool make_map(CUtensorMap* m, const void* base, int64_t inner, int64_t ou
     return r == CUDA_SUCCESS;
 }
 
+// The same operand seen as [inner / 64][outer][64], box {64, box_rows, kblocks}: several
+// k-blocks in one copy, each in its own swizzled box (the last one zero-filled past inner).
+static bool make_map_kblocks(CUtensorMap* m, const void* base, int64_t inner, int64_t outer, int box_rows, int kblocks) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {64u, (cuuint64_t)outer, (cuuint64_t)(inner / 64)};
+    cuuint64_t strides[2] = {(cuuint64_t)inner * 2, 128u};
+    cuuint32_t box[3] = {64u, (cuuint32_t)box_rows, (cuuint32_t)kblocks};
+    cuuint32_t estr[3] = {1u, 1u, 1u};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 static uint64_t g_wait_ns = 2000000000ull;
 static int g_pairs = MOE_PAIRS_AUTO;  // CTA-pair tiles for the 256-wide M-variable expert GEMMs
 
@@ -1314,13 +1459,13 @@ static int band_for(int c) {
     return b;
 }
 
-template <int BN, bool B_MN, bool VAR_K, int EPI, bool PAIR = false, bool DW2 = false, int OCC = 1, int EW = 4>
+template <int BN, bool B_MN, bool VAR_K, int EPI, bool PAIR = false, bool DW2 = false, int OCC = 1, int EW = 4, int AR = BM>
 static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mo0,
                           const CUtensorMap& mo1, const Params& p, int64_t tiles_ub,
                           cudaStream_t s, const CUtensorMap* ma2 = nullptr,
                           const CUtensorMap* mb2 = nullptr, const CUtensorMap* mo2 = nullptr,
                           const Params* p2 = nullptr, const CUtensorMap* mas = nullptr, const CUtensorMap* mx2 = nullptr) {
-    auto kern = grouped_gemm_kernel<BN, B_MN, VAR_K, EPI, PAIR, DW2, OCC, EW>;
+    auto kern = grouped_gemm_kernel<BN, B_MN, VAR_K, EPI, PAIR, DW2, OCC, EW, AR>;
     const CUtensorMap& A2 = ma2 ? *ma2 : ma;
     const CUtensorMap& B2 = mb2 ? *mb2 : mb;
     const CUtensorMap& O2 = mo2 ? *mo2 : mo0;
@@ -1331,12 +1476,12 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
     if (!p2) P2.G = 0;  // no second problem
     constexpr int NPAIR = PAIR ? 2 : 1;
     constexpr int KB = kblock_rows(VAR_K, PAIR, EPI, BN);
-    constexpr int STB = (BM * KB * 2 + BN / NPAIR * KB * 2) * kblocks_per_stage(EPI, BN, PAIR, VAR_K, DW2, OCC);  // bytes of one operand stage
-    constexpr int NST = num_stages((uint32_t)STB, EPI, OCC);
+    constexpr int STB = (AR * KB * 2 + BN / NPAIR * KB * 2) * kblocks_per_stage(EPI, BN, PAIR, VAR_K, DW2, OCC, AR);  // bytes of one operand stage
+    constexpr int NST = num_stages((uint32_t)STB, EPI, OCC, AR);
     const int extra_max = EPI == EPI_ROUTE ? 64 * 64 * 4 : epi_stage_bytes(EPI);
     const int extra = EPI == EPI_ROUTE ? p.hist_n * 4 : epi_stage_bytes(EPI);
-    const int smem_max = NST * STB + 1024 + extra_max;
-    const int smem = NST * STB + 1024 + extra;
+    const int smem_max = NST * STB + 1024 + extra_max + mma_overread(AR);
+    const int smem = NST * STB + 1024 + extra + mma_overread(AR);
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
@@ -1554,7 +1699,7 @@ cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s, const G
     }
     // MN-major B: weights stored [G*K, N] (or [G*b_rows, N])
     const bool slim = g.slim && g.epi == EPI_STORE && g.N % 128 == 0;
-    const int kps = kblocks_per_stage(g.epi, pair || g.N % 256 == 0 ? 256 : 128, pair, false, false, slim ? 2 : 1);
+    const int kps = kblocks_per_stage(g.epi, pair || g.N % 256 == 0 ? 256 : 128, pair, false, false, slim ? 2 : 1, BM);
     if (!make_map(&mb, g.b, g.N, (int64_t)g.G * p.b_group_rows, BK * kps)) return cudaErrorInvalidValue;
     if (g.epi == EPI_SWIGLU_BWD) {
         p.F = g.N;
@@ -1721,13 +1866,32 @@ cudaError_t launch_route_tc(const RouteArgs& a, cudaStream_t s) {
     // under 128 rows, at least 16
     const int64_t share = (a.T + sm_count() - 1) / sm_count();
     p.tile_rows = (int)std::max<int64_t>(16, std::min<int64_t>(BM, share));
-    CUtensorMap ma, mb;
-    if (!make_map(&ma, a.x, a.d, a.T, p.tile_rows)) return cudaErrorInvalidValue;
-    if (!make_map(&mb, a.w_router, a.d, (int64_t)a.P * a.E, BNr)) return cudaErrorInvalidValue;
     const int64_t tiles = (a.T + p.tile_rows - 1) / p.tile_rows + a.P;
-    if (BNr == 16) return launch<16, false, false, EPI_ROUTE>(ma, mb, ma, ma, p, tiles, s);
-    if (BNr == 32) return launch<32, false, false, EPI_ROUTE>(ma, mb, ma, ma, p, tiles, s);
-    if (BNr == 64) return launch<64, false, false, EPI_ROUTE>(ma, mb, ma, ma, p, tiles, s);
+    const int ar = BNr > 64 || p.tile_rows > 32 ? BM : p.tile_rows > 16 ? 32 : 16;
+    const int kps = kblocks_per_stage(EPI_ROUTE, BNr, false, false, false, 1, ar);
+    CUtensorMap ma, mb;
+    if (ar < BM) {
+        if (!make_map_kblocks(&ma, a.x, a.d, a.T, ar, kps)) return cudaErrorInvalidValue;
+        if (!make_map_kblocks(&mb, a.w_router, a.d, (int64_t)a.P * a.E, BNr, kps)) return cudaErrorInvalidValue;
+    } else {
+        if (!make_map(&ma, a.x, a.d, a.T, p.tile_rows)) return cudaErrorInvalidValue;
+        if (!make_map(&mb, a.w_router, a.d, (int64_t)a.P * a.E, BNr)) return cudaErrorInvalidValue;
+    }
+#define MOE_ROUTE(BN, AR) return launch<BN, false, false, EPI_ROUTE, false, false, 1, 4, AR>(ma, mb, ma, ma, p, tiles, s)
+    if (ar == 16) {
+        if (BNr == 16) MOE_ROUTE(16, 16);
+        if (BNr == 32) MOE_ROUTE(32, 16);
+        MOE_ROUTE(64, 16);
+    }
+    if (ar == 32) {
+        if (BNr == 16) MOE_ROUTE(16, 32);
+        if (BNr == 32) MOE_ROUTE(32, 32);
+        MOE_ROUTE(64, 32);
+    }
+    if (BNr == 16) MOE_ROUTE(16, BM);
+    if (BNr == 32) MOE_ROUTE(32, BM);
+    if (BNr == 64) MOE_ROUTE(64, BM);
+#undef MOE_ROUTE
     if (BNr == 128) return launch<128, false, false, EPI_ROUTE>(ma, mb, ma, ma, p, tiles, s);
     return launch<256, false, false, EPI_ROUTE>(ma, mb, ma, ma, p, tiles, s);
 }
