@@ -521,11 +521,11 @@ def main():
     pk = peaks()
     gemm_flops = sh.gemm_flops()
     achieved = gemm_flops / (gms / 1e3) / 1e12
-    # expert-GEMM launches: GEMM1, GEMM2 (+2 for shared experts), then the backward's as
-    # the library reports them (dA with dW2 in one launch, dX as CTA pairs beside dW1 on
-    # the tensor cores by default; four on the CUDA cores; shared experts' four)
+    # expert-GEMM launches: GEMM1 and GEMM2 (with the shared experts' in bf16, +2 in fp32),
+    # then the backward's as the library reports them (dA with dW2 in one launch or beside
+    # it as CTA pairs, dX with dW1 likewise; four in fp32; shared experts' four)
     from paper_2506_02965_gb300 import _lib as L
-    n_gemm = 2 + L.moe_expert_ffn_bwd_kernels(lay.cfg) + (2 if sh.n_shared else 0)
+    n_gemm = 2 + L.moe_expert_ffn_bwd_kernels(lay.cfg) + (2 if sh.n_shared and sh.dtype != "bf16" else 0)
     traffic = gemm_traffic_record(sh)
     fwd_flops, bwd_flops = gemm_flops / 3.0, 2.0 * gemm_flops / 3.0
     roofline = {"bound": "tensor", "kernel": "grouped_gemm_kernel (tcgen05, all expert GEMM launches)",
