@@ -293,8 +293,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
             }
             return false;
         };
-        // copy one block, W floats a copy: outer lines o0, o0 + 32 / PER, ...
-        auto copy_block = [&](auto mnc, auto wc, const float* src, int64_t ld, int o, int in, int k0, int lim, uint32_t dst) {
+        // copy one block, W floats a copy: outer lines o0, o0 + 32 / PER, ... (a copy that reads
+        // nothing names the operand's base, which is aligned to W: addresses are checked all the same)
+        auto copy_block = [&](auto mnc, auto wc, const float* base, const float* src, int64_t ld, int o, int in, int k0,
+                              int lim, uint32_t dst) {
             constexpr bool MN = decltype(mnc)::value;
             constexpr int W = decltype(wc)::value, STEP = W;  // 32 / (32 / W) lines per copy
             // K-contiguous lines are swizzled so that the 32-byte reads below spread over the banks
@@ -304,18 +306,19 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
             for (int o0 = 0; o0 < 8; o0 += STEP) {
                 const int n = MN ? (lim && o0 < nk ? 4 * W : 0) : (o0 < lim ? nk : 0);
                 const uint32_t at = dst + o0 * 128;
-                cp_async<W>(MN ? at : at ^ (((o + o0) & 1) << 4), n ? src + o0 * ld : p.a, n);
+                cp_async<W>(MN ? at : at ^ (((o + o0) & 1) << 4), n ? src + o0 * ld : base, n);
             }
         };
-        auto copy_op = [&](auto mnc, int vec, const float* src, int64_t ld, int o, int in, int k0, int lim, uint32_t dst) {
-            if (vec == 4) copy_block(mnc, std::integral_constant<int, 4>{}, src, ld, o, in, k0, lim, dst);
-            else if (vec == 2) copy_block(mnc, std::integral_constant<int, 2>{}, src, ld, o, in, k0, lim, dst);
-            else copy_block(mnc, std::integral_constant<int, 1>{}, src, ld, o, in, k0, lim, dst);
+        auto copy_op = [&](auto mnc, int vec, const float* base, const float* src, int64_t ld, int o, int in, int k0, int lim,
+                           uint32_t dst) {
+            if (vec == 4) copy_block(mnc, std::integral_constant<int, 4>{}, base, src, ld, o, in, k0, lim, dst);
+            else if (vec == 2) copy_block(mnc, std::integral_constant<int, 2>{}, base, src, ld, o, in, k0, lim, dst);
+            else copy_block(mnc, std::integral_constant<int, 1>{}, base, src, ld, o, in, k0, lim, dst);
         };
         auto issue = [&](int slot) {
             const uint32_t dst = raw + slot * raw_bytes();
-            if (has_rows) copy_op(std::integral_constant<bool, A_MN>{}, p.vec_a, src_a, lda, oa, ia, ak, lim_a, dst);
-            if (has_cols) copy_op(std::integral_constant<bool, B_MN>{}, p.vec_b, src_b, ldb, ob, ib, bk, lim_b, dst + 1024);
+            if (has_rows) copy_op(std::integral_constant<bool, A_MN>{}, p.vec_a, p.a, src_a, lda, oa, ia, ak, lim_a, dst);
+            if (has_cols) copy_op(std::integral_constant<bool, B_MN>{}, p.vec_b, p.b, src_b, ldb, ob, ib, bk, lim_b, dst + 1024);
         };
         // split one landed block into the three planes at d
         auto split_block = [&](auto mnc, const uint8_t* q, uint8_t* d, uint32_t plane) {

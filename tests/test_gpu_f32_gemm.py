@@ -92,3 +92,30 @@ def test_non_finite_values_follow_ieee(L):
     assert np.allclose(h[129].double().numpy(), want, rtol=1e-6, atol=0)
     rest = [i for i in range(130) if i not in (3, 50, 51, 129)]
     assert torch.equal(h[rest], clean[rest])
+
+
+@pytest.mark.parametrize("E", [7, 8, 40])
+def test_operand_with_element_alignment(L, E):
+    """The router's input gradient with dlogits (the A operand) aligned to one element only,
+    beside weights that are copied 16 bytes at a time: pools that leave a contraction tail, so
+    that copies of nothing occur in both operands. The same bits as with an aligned dlogits."""
+    T, d, k = 150, 132, 2
+    rng = np.random.default_rng(E)
+    f = lambda *s: dev(rng.standard_normal(s).astype(np.float32), torch.float32)  # noqa: E731
+    x, wr, dtw = f(T, d), f(1, E, d), f(T, k)
+    pr = torch.softmax(f(T, E), 1)
+    w, idx = pr.topk(k, 1)
+    cfg = cfg_of(L, mi.MoEShape("r", T, d, E, 128, k, "f32"))
+    n = L.moe_workspace_size(cfg)
+    ws = torch.empty(n, dtype=torch.uint8, device="cuda")
+    got = []
+    for shift in (0, 1):
+        dl, dx = empty((T * E + 1,), torch.float32)[shift:shift + T * E].view(T, E), empty((T, d), torch.float32)
+        assert dl.data_ptr() % 16 == 4 * shift
+        L.moe_route_bwd(cfg, x, wr, pr, idx.int(), w.contiguous(), dtw, None, None, dl, empty((1, E, d), torch.float32),
+                        empty((1, E), torch.float32), dx, ws, n)
+        assert status(L) == 0
+        got.append(dx)
+        z, wd = dl.double().cpu().numpy(), wr[0].double().cpu().numpy()
+        close("dx_router", dx, z @ wd, np.abs(z) @ np.abs(wd), E)
+    assert torch.equal(got[0], got[1])
