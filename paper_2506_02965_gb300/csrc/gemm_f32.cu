@@ -413,8 +413,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
                     }
                 }
             }
-            if ((!ok || *abort_flag) && lane == 0 && issued) {
-                // every MMA issued has completed before TMEM is released
+            if (lane == 0 && issued) {
+                // every MMA issued has completed before TMEM is released, also when another role
+                // gives up only after this one is through
                 mma_commit(drain_bar);
                 const uint64_t limit = p.wait_ns > 200000000ull ? p.wait_ns : 200000000ull, t0 = gtimer();
                 while (!mbar_try(drain_bar, 0) && gtimer() - t0 < limit) {

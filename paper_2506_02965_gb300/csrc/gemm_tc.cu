@@ -931,8 +931,11 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                     }
                 }
             }
+            // Every copy started into this pair lands before the CTAs exit (after a whole launch at
+            // once: the MMAs have read them), also when another role gives up only after this one
+            // is through.
             if constexpr (PAIR && VAR_K) {
-                if ((!ok || *abort_flag) && rank == 1) {
+                if (rank == 1) {
                     // partial copies on this CTA's own barriers: the last phase armed
                     for (int s2 = 0; s2 < NST; ++s2) {
                         if (!((parmed >> s2) & 1u)) continue;
@@ -943,9 +946,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                     }
                 }
             }
-            if ((!ok || *abort_flag) && rank == 0) {
-                // let every copy started into this pair land before the CTAs exit (the
-                // leader's full barriers count the peer's bytes too)
+            if (rank == 0) {  // (the leader's full barriers count the peer's bytes too)
                 for (int s = 0; s < NST; ++s) {
                     if (!((issued >> s) & 1u)) continue;
                     const uint64_t t0 = gtimer();
@@ -1052,8 +1053,8 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                 acc_phase ^= 1u;
             }
         }
-        if ((!ok || *abort_flag) && lane == 0 && issued_any) {
-            // wait for every MMA this CTA issued before TMEM is released
+        if (lane == 0 && issued_any) {
+            // wait for every MMA this CTA issued before TMEM is released (always, as above)
             if constexpr (PAIR) mma_commit_pair(drain_bar, 1);
             else mma_commit(drain_bar);
             const uint64_t t0 = gtimer();
