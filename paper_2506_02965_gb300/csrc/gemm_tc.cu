@@ -789,6 +789,10 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
             return mbar_wait(bar, parity, abort_flag, p.wait_ns);
         }
     };
+    // the same for a whole warp: one answer to all lanes, of which some may have given up where
+    // others saw the barrier complete (they must not part before warp-wide tcgen05.ld, nor at
+    // the block's barrier)
+    auto warp_wait = [&](uint32_t bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, wait_bar(bar, parity)); };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < NST; ++s) {
@@ -970,14 +974,14 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
             const Tile ti = tile_at(t);
             // kind::f16 descriptor of a swapped tile: A = weights (M = 256), B = rows (K-major)
             const uint32_t idesc_s = instr_desc<16, B_MN, false, BMP>() - (2u << 17) + ((uint32_t)(ti.ntok >> 3) << 17);
-            if (!wait_bar(tempty_bar(acc), acc_phase ^ 1u)) {
+            if (!warp_wait(tempty_bar(acc), acc_phase ^ 1u)) {
                 ok = false;
                 break;
             }
             fence_after();
             const uint32_t tmem_d = tmem_base + (uint32_t)(acc * BN);
             for (int kb = 0; kb < ti.k_iters; ++kb) {
-                if (!wait_bar(full_bar(stage), phase)) {
+                if (!warp_wait(full_bar(stage), phase)) {
                     ok = false;
                     break;
                 }
@@ -1075,7 +1079,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                     const Tile ti = tile_at(t);
                     for (int kb = 0; kb < ti.k_iters; ++kb) {
                         if (kb == ti.k_iters - 1 && ti.last_rows < KB) {
-                            if (!mbar_wait(pfull_bar(st2), (wpar >> st2) & 1u, abort_flag, p.wait_ns)) {
+                            if (!__all_sync(0xffffffffu, mbar_wait(pfull_bar(st2), (wpar >> st2) & 1u, abort_flag, p.wait_ns))) {
                                 ok2 = false;
                                 break;
                             }
@@ -1139,7 +1143,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
             }
         };
         auto gu_wait = [&](int b, uint32_t parity) -> bool {
-            return mbar_wait(gu_bar0 + 8u * b, parity, abort_flag, limit);
+            return __all_sync(0xffffffffu, mbar_wait(gu_bar0 + 8u * b, parity, abort_flag, limit));
         };
         if constexpr (EPI == EPI_SWIGLU_BWD) {
             if (tile0 < total_tiles) {
@@ -1184,7 +1188,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
             };
             if (dwt) {
                 // second problem: a bf16 weight-gradient tile, [Mout, N] per group
-                if (!wait_bar(tfull_bar(acc), acc_phase)) break;
+                if (!warp_wait(tfull_bar(acc), acc_phase)) break;
                 fence_after();
                 __nv_bfloat16* out = (__nv_bfloat16*)p2.out0 + (int64_t)ti.we * p2.Mout * p2.N + (int64_t)m * p2.N;
 #pragma unroll 1
@@ -1203,7 +1207,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                     emit(1, vals, maps, cols, direct);
                 }
             } else if (SWAP && ti.ntok) {
-                if (!wait_bar(tfull_bar(acc), acc_phase)) break;
+                if (!warp_wait(tfull_bar(acc), acc_phase)) break;
                 fence_after();
                 swapped_epilogue<EPI>(N, p.F, out0, p.aux, ti, (int)rank, q, lane, tbase, half * 32, SPLIT * 32);
             } else if constexpr (EPI == EPI_SWIGLU_BWD) {
@@ -1215,7 +1219,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                 constexpr int NCH = BN / 32;
                 const int nchv = min(NCH, (F - ti.n0) / 32);  // chunks inside F (a ragged last tile)
                 if (gu_issued == gu_chunk) gu_issue(ti, 0);  // not prefetched (a fused tile came before)
-                if (!wait_bar(tfull_bar(acc), acc_phase)) break;
+                if (!warp_wait(tfull_bar(acc), acc_phase)) break;
                 fence_after();
                 bool stop = false;
 #pragma unroll 1
@@ -1266,7 +1270,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                 }
                 if (stop) break;
             } else {
-                const bool got = wait_bar(tfull_bar(acc), acc_phase);
+                const bool got = warp_wait(tfull_bar(acc), acc_phase);
                 // (short router tiles: the epilogue warps meet per tile, and give up together)
                 if (SHORT ? epilogue_any(!got) : !got) break;
                 fence_after();
