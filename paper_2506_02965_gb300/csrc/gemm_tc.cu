@@ -981,10 +981,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
             fence_after();
             const uint32_t tmem_d = tmem_base + (uint32_t)(acc * BN);
             for (int kb = 0; kb < ti.k_iters; ++kb) {
-                if (!warp_wait(full_bar(stage), phase)) {
-                    ok = false;
-                    break;
-                }
+                const bool got = wait_bar(full_bar(stage), phase);
                 const uint32_t sa = ring + stage * STAGE_BYTES;
                 const uint32_t sb = sa + A_BYTES;
                 // K-variable groups: the last k-block may hold contraction rows of the next
@@ -996,7 +993,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                 const int ksteps = part ? (ti.last_rows + 15) / 16 : KB * KPS / 16;
                 if (part) {
                     const int zr0 = ti.last_rows, zr1 = ksteps * 16;
-                    if (zr1 > zr0) {
+                    if (got && zr1 > zr0) {
                         uint8_t* base = ring_ptr + (size_t)stage * STAGE_BYTES;
                         const int per_box = (zr1 - zr0) * 8;  // 16-byte words
 #pragma unroll
@@ -1009,7 +1006,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                     __syncwarp();
                 }
                 fence_after();
-                if (lane == 0) {
+                if (lane == 0 && got) {
                     auto step = [&](int kk, bool swapped) {
                         uint64_t ad, bd;
                         if (!A_MN && !dwt) ad = smem_desc(sa + (kk / (KB / 16)) * A_BOX + (kk % (KB / 16)) * 32, 16, 1024);
@@ -1036,7 +1033,12 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                     else mma_commit(empty_bar(stage));
                     issued_any = true;
                 }
-                __syncwarp();
+                // one answer to the warp, after the MMAs are on their way (a vote before them cost
+                // up to 1% of a step)
+                if (!__all_sync(0xffffffffu, got)) {
+                    ok = false;
+                    break;
+                }
                 if (++stage == NST) {
                     stage = 0;
                     phase ^= 1u;
