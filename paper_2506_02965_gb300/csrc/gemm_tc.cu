@@ -570,6 +570,9 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
     __shared__ uint64_t bars[2 * NST + 5 + 2 * EW + NPART];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
+    // pairs: operand stages that this CTA's producer filled in all, and the bytes of each stage's
+    // last fill that count on the leader's barrier
+    __shared__ uint32_t s_fills, s_fill_bytes[PAIR ? NST : 1];
     __shared__ int s_tile_start[MAX_GROUPS + 1];
     __shared__ int s_total1;  // fused: tiles of the first problem
     __shared__ unsigned char s_order[DW2 ? MAX_GROUPS : 1];  // fused: second problem's group order
@@ -839,6 +842,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
             int stage = 0;
             uint32_t phase = 0;
             uint32_t issued = 0, issued_par = 0;  // stages ever filled, and the parity of their last fill
+            uint32_t fills = 0;
             // K-variable pair peer: stages whose own barrier was ever armed, and per stage
             // the parity of the next phase to arm
             uint32_t parmed = 0, pnext = 0;
@@ -927,6 +931,10 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                             load(sb + i * ATOM_B, mB, fb, ti.n0 + (int)rank * BNL + 64 * i, brow + k0);
                     }
                     }
+                    if constexpr (PAIR) {
+                        s_fill_bytes[stage] = local_bar ? 0 : tile_bytes / NPAIR;
+                        ++fills;
+                    }
                     issued |= 1u << stage;
                     issued_par = (issued_par & ~(1u << stage)) | (phase << stage);
                     if (++stage == NST) {
@@ -935,6 +943,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                     }
                 }
             }
+            if constexpr (PAIR) s_fills = fills;
             // Every copy started into this pair lands before the CTAs exit (after a whole launch at
             // once: the MMAs have read them), also when another role gives up only after this one
             // is through.
@@ -1376,7 +1385,28 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
     }
     fence_before();
     __syncthreads();
-    if constexpr (PAIR) cluster_sync_all();  // neither CTA leaves while the pair's MMAs run
+    if constexpr (PAIR) {
+        if (threadIdx.x == 0 && *abort_flag) st_cluster(map_to_rank(smem_u32(&s_abort), rank ^ 1u), 1u);
+        __syncwarp();
+        cluster_sync_all();  // neither CTA leaves while the pair's MMAs run
+        if (*abort_flag) {   // (both CTAs see it)
+            // The peer's producer may have filled stages that the leader's, giving up first, never
+            // armed: the leader arms them for those bytes alone and waits for them.
+            if (rank == 0 && threadIdx.x == 0) {
+                const uint32_t theirs = ld_cluster(map_to_rank(smem_u32(&s_fills), 1));
+                for (uint32_t i = s_fills; i < theirs; ++i) {
+                    const uint32_t bytes = ld_cluster(map_to_rank(smem_u32(&s_fill_bytes[i % NST]), 1));
+                    if (!bytes) continue;
+                    mbar_expect_tx(full_bar(i % NST), bytes);
+                    const uint64_t t0 = gtimer();
+                    while (!mbar_try(full_bar(i % NST), (i / NST) & 1u) && gtimer() - t0 < drain_limit) {
+                    }
+                }
+            }
+            __syncwarp();
+            cluster_sync_all();
+        }
+    }
     fence_after();
     if (warp == 1) {
         if constexpr (PAIR)
