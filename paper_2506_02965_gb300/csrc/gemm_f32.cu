@@ -6,7 +6,10 @@
 // value is split exactly into three bf16 values, x = h + m + l (each the bf16 nearest to
 // what the ones before left: 3 x 8 bits of significand cover fp32's 24), and a product is
 // the sum of the six bf16 products hh, hm, mh, mm, hl, lh; the three left out are below
-// 2^-25 of it. The tensor core's fp32 accumulator truncates, which over a long contraction
+// 2^-25 of it. Both operands are multiplied by 2^23 before the split and the sums by 2^-46
+// after it, which changes no digit: the last bit of the smallest fp32 number, 2^-149, becomes
+// bf16's smallest normal number, so that the split is exact down to zero. (Unscaled it was not
+// below 2^-110: 6e-5 off for operands of 2^-120.) The tensor core's fp32 accumulator truncates, which over a long contraction
 // loses more than an FFMA chain does, so an accumulator holds only 32 contraction terms
 // (the smallest products first) and is then added to fp32 registers with round-to-nearest.
 // Measured against 64 bits, the worst tensor of a whole fp32 step is 2.4e-7 (512 tokens,
@@ -27,8 +30,9 @@
 // 1501 tokens, d = 1000, F = 1366, E = 6, k = 3: 5.39 -> 1.13 ms (21 -> 98 TFLOP/s);
 // 512 tokens, d = 256, F = 512, E = 8, k = 2: 493 -> 133 us.
 //
-// An infinite or NaN operand makes 0 * inf terms in the split, so an output element that is
-// not finite is computed again by a plain fp32 FMA chain, which gives IEEE results.
+// An infinite or NaN operand makes 0 * inf terms in the split, and operands from 2^105 or sums
+// from 2^82 on leave the scaled range, so an output element that is not finite is computed
+// again by a plain fp32 FMA chain, which gives IEEE results.
 #include <algorithm>
 #include <type_traits>
 
@@ -100,16 +104,19 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// 8 values -> the three bf16 planes of x = h + m + l, 16 bytes each
+constexpr float kSplitScale = 8388608.f;         // 2^23
+constexpr float kSumScale = 0x1p-46f;            // of a product of two scaled operands
+// 8 values -> the three bf16 planes of 2^23 x = h + m + l, 16 bytes each
 __device__ __forceinline__ void split8(const float* v, uint4* h, uint4* m, uint4* l) {
     uint32_t* hp = reinterpret_cast<uint32_t*>(h);
     uint32_t* mp = reinterpret_cast<uint32_t*>(m);
     uint32_t* lp = reinterpret_cast<uint32_t*>(l);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const __nv_bfloat162 hh = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+        const float x0 = v[2 * i] * kSplitScale, x1 = v[2 * i + 1] * kSplitScale;
+        const __nv_bfloat162 hh = __floats2bfloat162_rn(x0, x1);
         const uint32_t hu = *reinterpret_cast<const uint32_t*>(&hh);
-        const float r0 = v[2 * i] - __uint_as_float(hu << 16), r1 = v[2 * i + 1] - __uint_as_float(hu & 0xffff0000u);
+        const float r0 = x0 - __uint_as_float(hu << 16), r1 = x1 - __uint_as_float(hu & 0xffff0000u);
         const __nv_bfloat162 mm = __floats2bfloat162_rn(r0, r1);
         const uint32_t mu = *reinterpret_cast<const uint32_t*>(&mm);
         const __nv_bfloat162 ll =
@@ -459,6 +466,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
                 }
             }
             if (!ok) break;
+#pragma unroll
+            for (int c = 0; c < CW; ++c) {
+                acc[0][c] *= kSumScale;
+                acc[1][c] *= kSumScale;
+            }
             // transpose through shared memory (32 rows x 32 columns at a time): lanes then run
             // along the columns, so that loads and stores are coalesced
             auto put = [&](int at, float v) { st[lane * 32 + (at ^ lane)] = v; };

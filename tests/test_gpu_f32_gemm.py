@@ -25,7 +25,7 @@ def L():
 
 def close(name, got, ref, mag, K):
     err = np.abs(got.double().cpu().numpy() - ref)
-    bound = (16 + K / 32) * 2.0 ** -23 * mag + 1e-38
+    bound = (16 + K / 32) * 2.0 ** -23 * mag + (2 + K / 32) * 2.0 ** -149
     assert (err <= bound).all(), (name, float((err / bound).max()))
 
 
@@ -72,6 +72,28 @@ def test_contractions_at_the_edges(L, rows, d, F):
         dA, mag = dy[r] @ w2[e], np.abs(dy[r]) @ np.abs(w2[e])
         close("dG", g["dh"][r, :F], dA * U * s * (1 + G * (1 - s)), mag * np.abs(U) * (1 + np.abs(G)), d)
         close("dU", g["dh"][r, F:], dA * G * s, mag * np.abs(G), d)
+
+
+@pytest.mark.parametrize("xe,we", [(-120, 0), (-140, 10), (-149, 20), (0, -125), (-60, -60), (-100, -50), (60, -128)])
+def test_operands_near_the_end_of_the_range(L, xe, we):
+    """h = x W1^T with all of x of about 2^xe and all of W1 of about 2^we: the bound above, and
+    what the last rounding of an fp32 number that small adds (2^-149 a step: the split's, the
+    accumulator's and each register addition's)."""
+    rows, d, F = (5, 130), 100, 33
+    rng = np.random.default_rng(1000 - xe + we)
+    f = lambda e, *s: np.ldexp(rng.standard_normal(s), e).astype(np.float32)  # noqa: E731
+    off, x, w1 = np.array([0, 5, 135], np.int32), f(xe, 135, d), f(we, 2, 2 * F, d)
+    h, a, y = (empty((135, n), torch.float32) for n in (2 * F, F, d))
+    t = lambda v: dev(v, torch.float32)  # noqa: E731
+    L.moe_expert_ffn_fwd(cfg_of(L, mi.MoEShape("f", 135, d, 2, F, 1, "f32")), t(x), dev(off, torch.int32), t(w1),
+                         t(f(0, 2, d, F)), h, a, y)
+    assert status(L) == 0
+    for e in range(2):
+        r = slice(off[e], off[e + 1])
+        xs, ws = x[r].astype(np.float64), w1[e].astype(np.float64)
+        err = np.abs(h[r].double().cpu().numpy() - xs @ ws.T)
+        bound = (16 + d / 32) * 2.0 ** -23 * (np.abs(xs) @ np.abs(ws).T) + (2 + d / 32) * 2.0 ** -149
+        assert (err <= bound).all(), float((err / bound).max())
 
 
 def test_non_finite_values_follow_ieee(L):
