@@ -324,8 +324,9 @@ moe_status moe_sgd_update(void* w, const void* dw, float* w_master, int64_t n_gr
  * last call (MOE_OK if none) in *code and clears it. */
 moe_status moe_device_status(moe_stream_t stream, int32_t* code /* HOST out */);
 
-/* Upper bound, in nanoseconds, of every bounded wait inside the tensor-core kernels
- * (default 2e9). A wait that runs out records MOE_ERR_TIMEOUT and the kernel returns. */
+/* Upper bound, in nanoseconds, of every bounded wait inside the tensor-core kernels, the fp32
+ * ones included (default 2e9). A wait that runs out records MOE_ERR_TIMEOUT and the kernel
+ * returns. */
 moe_status moe_set_wait_limit_ns(uint64_t ns);
 
 /* Tile shape of the 256-wide expert GEMMs (forward, dA, dX and the weight gradients),

@@ -32,7 +32,7 @@
 //
 // An infinite or NaN operand makes 0 * inf terms in the split, and operands from 2^105 or sums
 // from 2^82 on leave the scaled range, so an output element that is not finite is computed
-// again by a plain fp32 FMA chain, which gives IEEE results.
+// again by a plain fp32 FMA chain, which gives IEEE results (repair).
 #include <algorithm>
 #include <type_traits>
 
@@ -113,10 +113,10 @@ __device__ __forceinline__ void split8(const float* v, uint4* h, uint4* m, uint4
     uint32_t* lp = reinterpret_cast<uint32_t*>(l);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const float x0 = v[2 * i] * kSplitScale, x1 = v[2 * i + 1] * kSplitScale;
-        const __nv_bfloat162 hh = __floats2bfloat162_rn(x0, x1);
+        const __nv_bfloat162 hh = __hmul2(__floats2bfloat162_rn(v[2 * i], v[2 * i + 1]), __float2bfloat162_rn(kSplitScale));
         const uint32_t hu = *reinterpret_cast<const uint32_t*>(&hh);
-        const float r0 = x0 - __uint_as_float(hu << 16), r1 = x1 - __uint_as_float(hu & 0xffff0000u);
+        const float r0 = fmaf(v[2 * i], kSplitScale, -__uint_as_float(hu << 16)),
+                    r1 = fmaf(v[2 * i + 1], kSplitScale, -__uint_as_float(hu & 0xffff0000u));
         const __nv_bfloat162 mm = __floats2bfloat162_rn(r0, r1);
         const uint32_t mu = *reinterpret_cast<const uint32_t*>(&mm);
         const __nv_bfloat162 ll =
@@ -127,11 +127,119 @@ __device__ __forceinline__ void split8(const float* v, uint4* h, uint4* m, uint4
     }
 }
 
-// One output element by a plain FMA chain (outputs that the split made non-finite).
-__device__ float dot_plain(const float* a, int64_t sa, const float* b, int64_t sb, int K) {
-    float s = 0.f;
-    for (int k = 0; k < K; ++k) s = fmaf(a[k * sa], b[k * sb], s);
-    return s;
+__device__ __forceinline__ bool is_finite(float v) { return fabsf(v) <= 3.402823466e38f; }
+// A warp's outputs by plain chains of FMAs in order of k: y = lane l's row (of `rows` at A) times
+// RC columns (of `cols` at B). Eight k of both operands at a time go through st, the next eight
+// are in flight meanwhile. Stops early once every wanted output (a bit per column) is NaN, which
+// it then stays.
+template <bool A_MN, bool B_MN, int RC>
+__device__ __forceinline__ void fma_chains(const float* A, int64_t lda, int rows, const float* B, int64_t ldb, int cols,
+                                           int klen, uint32_t want, float* st, float (&y)[RC]) {
+    constexpr int RK = 8, NB = RK * RC / 32, LDB = RC + 4, LDA = RK + 4;
+    static_assert(RK * LDB + 32 * LDA <= ST_FLOATS, "a warp's buffer");
+    const int lane = threadIdx.x & 31;
+    float* sa = st + RK * LDB;  // [32][LDA], after B's [RK][LDB]
+    float a[RK], b[NB];
+    auto fetch = [&](int k0) {
+        // A: lane's row (MN: contiguous over the lanes), or four rows of RK consecutive k at a time
+#pragma unroll
+        for (int i = 0; i < RK; ++i) {
+            const int r = A_MN ? lane : 4 * i + lane / RK, k = k0 + (A_MN ? i : lane % RK);
+            a[i] = r < rows && k < klen ? A[A_MN ? k * lda + r : r * lda + k] : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            const int j = lane + 32 * i, k = k0 + (B_MN ? j / RC : j % RK), c = B_MN ? j % RC : j / RK;
+            b[i] = c < cols && k < klen ? B[B_MN ? k * ldb + c : c * ldb + k] : 0.f;
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < RC; ++i) y[i] = 0.f;
+    fetch(0);
+#pragma unroll 1
+    for (int k0 = 0; k0 < klen; k0 += RK) {
+        __syncwarp();  // the values before these have been read
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            const int j = lane + 32 * i;
+            st[B_MN ? j / RC * LDB + j % RC : j % RK * LDB + j / RK] = b[i];
+        }
+#pragma unroll
+        for (int i = 0; i < RK; ++i) sa[A_MN ? lane * LDA + i : (4 * i + lane / RK) * LDA + lane % RK] = a[i];
+        __syncwarp();
+        fetch(k0 + RK);
+#pragma unroll
+        for (int k = 0; k < RK; k += 4) {
+            float x[4];
+            Vec<float>::load(sa + lane * LDA + k, x);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int i = 0; i < RC; i += 4) {
+                    float w[4];
+                    Vec<float>::load(st + (k + q) * LDB + i, w);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) y[i + j] = fmaf(x[q], w[j], y[i + j]);
+                }
+        }
+        if (k0 % (4 * RK) == 0) {
+            uint32_t open = 0;
+#pragma unroll
+            for (int i = 0; i < RC; ++i) open |= y[i] == y[i] ? 1u << i : 0u;
+            if (!__any_sync(0xffffffffu, open & want)) break;
+        }
+    }
+}
+
+// The outputs of an epilogue warp (rows mrow.. of the tile, columns col0.. of either half) that it
+// has stored as not finite, computed again and stored: after the warp's last tile, when nothing
+// else is in registers, so that it costs the other outputs nothing. (dG and dU are not finite where dA is
+// not; a finite dA beside a G or U that is not comes out within rounding.) A, B: the operands of the tile's group;
+// out_row: the output row of its first. One chain per output costs about what the FFMA
+// kernel that this replaces took for any values: a step of 1501 tokens, d = 1000, F = 1366 of which
+// nearly all sums leave the range 4.1 to 7.2 ms (5.4 before; finite 1.13); NaN stop early, 1.6 to
+// 1.9 ms for all, 3.4 for a single one in dY.
+template <bool A_MN, bool B_MN, int EPI, int BN>
+static __device__ __forceinline__ void repair(const Params& p, const float* A, const float* B, int64_t out_row, int n0, int mrow,
+                                       int mrows, int klen, int col0, float* st) {
+    constexpr int RC = BN / 4;  // the warp's columns of one half
+    constexpr bool GU = EPI != EPI_STORE;  // outputs (gate, up) of a feature
+    const int lane = threadIdx.x & 31, F = EPI == EPI_SWIGLU_FWD ? p.N / 2 : p.N;
+    const int64_t lda = A_MN ? p.M : p.K, ldb = B_MN ? p.N : p.K;
+    float* out = p.out0 + (out_row + mrow + lane) * (GU ? 2 * F : F);
+    const bool row_ok = mrow + lane < mrows;
+    __syncwarp();  // the warp's stores before these
+#pragma unroll 1
+    for (int u = 0; u < 2; ++u) {
+        // RC columns from f on: features, or (forward) their gates or ups, rows n.. of B
+        const int f = n0 + col0 + (EPI == EPI_SWIGLU_FWD ? 0 : u * (BN / 2)), n = f + (EPI == EPI_SWIGLU_FWD ? u * F : 0);
+        const int cols = min(RC, F - f);
+        uint32_t want = 0;
+        if (row_ok)
+            for (int i = 0; i < cols; ++i)
+                if (!is_finite(out[n + i]) || (EPI == EPI_SWIGLU_BWD && !is_finite(out[F + n + i]))) want |= 1u << i;
+        if (!__any_sync(0xffffffffu, want)) continue;
+        float y[RC];
+        fma_chains<A_MN, B_MN, RC>(A + (A_MN ? mrow : mrow * lda), lda, mrows - mrow, B + (B_MN ? n : n * ldb), ldb, cols, klen, want,
+                               st, y);
+#pragma unroll
+        for (int i = 0; i < RC; ++i) {
+            if (!((want >> i) & 1u)) continue;
+            if constexpr (EPI == EPI_SWIGLU_BWD) {
+                const float* gu = p.aux + (out_row + mrow + lane) * 2 * F + n + i;
+                const float G = gu[0], U = gu[F], sg = sigmoidf_(G);
+                out[F + n + i] = y[i] * G * sg;
+                out[n + i] = y[i] * U * sg * (1.f + G * (1.f - sg));
+            } else {
+                out[n + i] = y[i];
+                if constexpr (EPI == EPI_SWIGLU_FWD) {  // (gates come before ups: the last to change)
+                    const float G = out[f + i], U = out[F + f + i];
+                    p.out1[(out_row + mrow + lane) * F + f + i] = G * sigmoidf_(G) * U;
+                }
+            }
+        }
+    }
+    __syncwarp();
 }
 
 template <bool A_MN, bool B_MN, bool VAR_K, int EPI, int BN>
@@ -437,6 +545,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
         float* st = reinterpret_cast<float*>(ring_ptr + NST * STAGE + NRAW * raw_bytes()) + (warp - EPI_WARP0) * ST_FLOATS;
         int b = 0;
         uint32_t bphase = 0;
+        float odd = 0.f;  // NaN once this lane has seen an output that is not finite
         for (int t = blockIdx.x; t < total; t += gridDim.x) {
             const Tile ti = tile_at(t);
             const int kiters = (ti.klen + FK - 1) / FK;
@@ -471,23 +580,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
                 acc[0][c] *= kSumScale;
                 acc[1][c] *= kSumScale;
             }
+            const int mrow = ti.m0 + q * 32;
             // transpose through shared memory (32 rows x 32 columns at a time): lanes then run
             // along the columns, so that loads and stores are coalesced
             auto put = [&](int at, float v) { st[lane * 32 + (at ^ lane)] = v; };
             auto get = [&](int r, int at) { return st[r * 32 + (at ^ r)]; };
-            auto finite = [](float v) { return fabsf(v) <= 3.402823466e38f; };
-            auto redo = [&](int m, int n) -> float {
-                const float* A = a_base(ti) + (A_MN ? (int64_t)m : (int64_t)m * p.K);
-                const float* B = b_base(ti) + (B_MN ? (int64_t)n : (int64_t)n * p.K);
-                return dot_plain(A, A_MN ? p.M : 1, B, B_MN ? p.N : 1, ti.klen);
-            };
-            // Eight rows at a time, so that their loads and stores overlap and one vote covers
-            // the check for non-finite values. (Row by row, with the check's branch at every
-            // element, a tile's epilogue took 8 us: the weight gradients of experts with few
-            // rows are all epilogue, dW2 of 78 experts of d = 1928, F = 591 at 10 rows took
-            // 362 us, now 173; dA waited for G and U row by row, 4503 rows of d = 1000,
-            // F = 1366 258 -> 163 us.)
-            const int mrow = ti.m0 + q * 32;
+            // Eight rows at a time, so that their loads and stores overlap. (Row by row, with a check
+            // for non-finite values at every element, a tile's epilogue took 8 us: the weight
+            // gradients of experts with few rows are all epilogue, dW2 of 78 experts of d = 1928,
+            // F = 591 at 10 rows took 362 us, now 173; dA waited for G and U row by row, 4503 rows
+            // of d = 1000, F = 1366 258 -> 163 us.)
             if constexpr (EPI == EPI_SWIGLU_FWD) {
                 // 16 gate columns beside the 16 up columns of the same features; a half-warp per row
 #pragma unroll
@@ -504,24 +606,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
                     for (int i0 = 0; i0 < 16; i0 += 8) {
                         const int m0 = mrow + 2 * i0 + (lane >> 4);  // rows m0, m0 + 2, ...
                         float G[8], U[8];
-                        bool ok8 = true;
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             const int r = 2 * (i0 + i) + (lane >> 4);
                             G[i] = get(r, c);
                             U[i] = get(r, 16 + c);
-                            ok8 = ok8 && finite(G[i]) && finite(U[i]);
-                        }
-                        if (!__all_sync(0xffffffffu, ok8)) {
-                            for (int i = 0; i < 8; ++i) {
-                                const int m = m0 + 2 * i;
-                                if (f >= F || m >= ti.mrows) continue;
-#pragma unroll
-                                for (int u = 0; u < 8; ++u) {
-                                    if (u == i && !finite(G[u])) G[u] = redo(m, f);
-                                    if (u == i && !finite(U[u])) U[u] = redo(m, F + f);
-                                }
-                            }
                         }
                         if (f >= F) continue;
                         float* h = p.out0 + (ti.o0 + m0) * 2 * F + f;
@@ -529,6 +618,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             if (m0 + 2 * i >= ti.mrows) break;
+                            odd = fmaf(U[i], 0.f, fmaf(G[i], 0.f, odd));
                             h[(int64_t)i * 4 * F] = G[i];
                             h[(int64_t)i * 4 * F + F] = U[i];
                             o[(int64_t)i * 2 * F] = G[i] * sigmoidf_(G[i]) * U[i];
@@ -557,24 +647,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
                                 U[i] = i < rows ? __ldg(gu + (int64_t)i * 2 * F + F) : 0.f;
                             }
                         }
-                        bool ok8 = true;
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            v[i] = get(r0 + i, lane);
-                            ok8 = ok8 && finite(v[i]);
-                        }
-                        if (!__all_sync(0xffffffffu, ok8)) {
-                            for (int i = 0; i < rows; ++i) {
-#pragma unroll
-                                for (int w = 0; w < 8; ++w)
-                                    if (w == i && !finite(v[w])) v[w] = redo(mrow + r0 + i, n);
-                            }
-                        }
+                        for (int i = 0; i < 8; ++i) v[i] = get(r0 + i, lane);
                         if constexpr (EPI == EPI_SWIGLU_BWD) {
                             float* o = p.out0 + (row0 + r0) * 2 * F + n;
 #pragma unroll
                             for (int i = 0; i < 8; ++i) {
                                 if (i >= rows) break;
+                                odd = fmaf(v[i], 0.f, odd);
                                 const float s = sigmoidf_(G[i]);
                                 o[(int64_t)i * 2 * F + F] = v[i] * G[i] * s;
                                 o[(int64_t)i * 2 * F] = v[i] * U[i] * s * (1.f + G[i] * (1.f - s));
@@ -584,11 +664,22 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
 #pragma unroll
                             for (int i = 0; i < 8; ++i) {
                                 if (i >= rows) break;
+                                odd = fmaf(v[i], 0.f, odd);
                                 o[(int64_t)i * p.N] = v[i];
                             }
                         }
                     }
                 }
+            }
+        }
+        // Outputs that are not finite are looked at again only now, when no other role of the CTA
+        // waits for this one: their chains may take longer than any wait limit.
+        if (__any_sync(0xffffffffu, odd != 0.f) && !*abort_flag) {
+#pragma unroll 1
+            for (int t = blockIdx.x; t < total; t += gridDim.x) {
+                const Tile ti = tile_at(t);
+                repair<A_MN, B_MN, EPI, BN>(p, a_base(ti), b_base(ti), VAR_K ? (int64_t)ti.we * p.M : ti.o0, ti.n0, ti.m0 + q * 32,
+                                            ti.mrows, ti.klen, hc * CW, st);
             }
         }
     }

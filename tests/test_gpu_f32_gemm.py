@@ -116,6 +116,54 @@ def test_non_finite_values_follow_ieee(L):
     assert torch.equal(h[rest], clean[rest])
 
 
+def test_large_finite_values_follow_the_fma_chain(L):
+    """Rows of x whose operands (from 2^105) or sums (from 2^82) leave the split's scaled range:
+    what a chain of d FMAs gives, each rounding a partial sum by 2^-24 of it."""
+    rows, d, F = (200,), 260, 70
+    rng = np.random.default_rng(4)
+    f = lambda *s: rng.standard_normal(s).astype(np.float32)  # noqa: E731
+    x, w1 = f(200, d), f(1, 2 * F, d) * np.float32(0.1)
+    x[3] *= np.float32(1e30)
+    x[150:] *= np.float32(2.0 ** 110)
+    h, a, y = (empty((200, n), torch.float32) for n in (2 * F, F, d))
+    t = lambda v: dev(v, torch.float32)  # noqa: E731
+    L.moe_expert_ffn_fwd(cfg_of(L, mi.MoEShape("f", 200, d, 1, F, 1, "f32")), t(x), dev([0, 200], torch.int32), t(w1),
+                         t(f(1, d, F)), h, a, y)
+    assert status(L) == 0
+    x64, w64 = x.astype(np.float64), w1[0].astype(np.float64)
+    mag = np.abs(x64) @ np.abs(w64).T
+    assert (np.abs(h.double().cpu().numpy() - x64 @ w64.T) <= (16 + d) * 2.0 ** -23 * mag).all()
+
+
+def test_non_finite_outputs_of_a_long_contraction_wait_as_long_as_they_need(L):
+    """One NaN in dY makes dW1 NaN everywhere, a row of dX and of dW2 too: each such output is a
+    chain over thousands of rows, during which the other roles wait. Even with a wait limit of
+    1 ns the call is right: the repair is no stalled wait (every other wait lasts a few us, and
+    a poll sleeps for up to 20)."""
+    rows, d, F = (6001, 50), 256, 200
+    clean = run(L, rows, d, F, seed=12)[0]
+    off = dev([0, 6001, 6051], torch.int32)
+    E, TK = 2, 6051
+    rng = np.random.default_rng(12)   # the inputs of run()
+    f = lambda *s: rng.standard_normal(s).astype(np.float32)  # noqa: E731
+    x, w1, w2, dy = f(TK, d), f(E, 2 * F, d) * np.float32(0.1), f(E, d, F) * np.float32(0.1), f(TK, d)
+    dy[4000, 7] = np.nan
+    t = {n: dev(v, torch.float32) for n, v in dict(x=x, w1=w1, w2=w2, dy=dy).items()}
+    dh, dx, dw1, dw2 = (empty(s, torch.float32) for s in ((TK, 2 * F), (TK, d), (E, 2 * F, d), (E, d, F)))
+    L.moe_set_wait_limit_ns(1)
+    try:
+        L.moe_expert_ffn_bwd(cfg_of(L, mi.MoEShape("f", TK, d, E, F, 1, "f32")), t["x"], off, t["w1"], t["w2"],
+                             clean["h"], clean["a"], t["dy"], dh, dx, dw1, dw2)
+        assert status(L) == 0
+    finally:
+        L.moe_set_wait_limit_ns(2_000_000_000)
+    rest = [i for i in range(TK) if i != 4000]
+    assert torch.isnan(dx[4000]).all() and torch.isnan(dw1[0]).all() and torch.isnan(dw2[0, 7]).all()
+    assert torch.equal(dx[rest], clean["dx"][rest]) and torch.equal(dw1[1], clean["dw1"][1])
+    assert torch.equal(dw2[1], clean["dw2"][1])
+    assert torch.equal(dw2[0, [i for i in range(d) if i != 7]], clean["dw2"][0, [i for i in range(d) if i != 7]])
+
+
 @pytest.mark.parametrize("E", [7, 8, 40])
 def test_operand_with_element_alignment(L, E):
     """The router's input gradient with dlogits (the A operand) aligned to one element only,
