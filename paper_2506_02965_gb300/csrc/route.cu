@@ -99,10 +99,9 @@ __device__ void softmax_topk_token(const float (&z)[NV], int lane, int E, int k,
 }
 
 // ----------------------------------------------------------------------------- router fwd
-// Router logits and gating on the CUDA cores: the fp32 configuration, and bf16 pools whose
-// size is not a multiple of 4 (up to 64 experts). One CTA takes TB consecutive tokens of
-// one party and all experts (padded to EP): chunks of RD_KC columns of x and W_r are staged
-// in shared memory as fp32 (the next chunk's global loads are in flight meanwhile), and
+// Router logits and gating of the fp32 configuration, up to 64 experts, on the CUDA cores. One CTA
+// takes TB consecutive tokens of one party and all experts (padded to EP): chunks of RD_KC columns
+// of x and W_r are staged in shared memory (the next chunk's global loads are in flight meanwhile), and
 // thread (ks, tg, eg) multiplies TB/4 tokens by 4 experts over the columns of its slice ks.
 // A chunk's products are summed on their own before they join the running sum, so no chain
 // of additions is longer than about d / 128 + 32. The KS slices of a logit are then added
@@ -112,19 +111,20 @@ __device__ void softmax_topk_token(const float (&z)[NV], int lane, int E, int k,
 //
 // What bounds it: with large pools the shared-memory reads (12 wavefronts per 64 FMAs of a
 // warp), with small ones the latency of the d / 128 chunk steps. The kernel that it replaces
-// (a warp per 1 to 8 tokens, W_r read from L2 by every warp) took 588 us for 3805 bf16 tokens
-// of d = 3072 with E = 63, now 71; 93 -> 28 us for 2157 of 3072 with E = 6; 51 -> 13 us for
-// 1003 of 1152 with E = 13; fp32: 19 -> 4.8 us for 512 of 256 with E = 8.
+// (a warp per 1 to 8 tokens, W_r read from L2 by every warp) took 288 us for 4096 tokens of
+// d = 2048 with E = 64, now 60; 19 -> 4.8 us for 512 of 256 with E = 8. The chunks' sums are
+// closer to 64 bits than its chains (1.3e-7 of 1.6e-7 there).
 constexpr int RD_KC = 128;         // columns per chunk
 constexpr int RD_LD = RD_KC + 4;   // row pitch in shared memory: rows start 16 bytes apart in the banks
 constexpr int RD_THREADS = 256;
 
-template <typename T, int EP, int TB>
+template <int EP, int TB>
 __global__ void __launch_bounds__(RD_THREADS, EP <= 16 && TB == 8 ? 4 : 2) route_dot_kernel(
-    const T* __restrict__ x, const T* __restrict__ wr, const float* __restrict__ bias,
+    const float* __restrict__ x, const float* __restrict__ wr, const float* __restrict__ bias,
     const int32_t* __restrict__ po, int P, int64_t Tn, int d, int E, int k, int normalize, float* logits,
     float* probs, int32_t* topk_idx, float* topk_w, int32_t* counts) {
     pdl_begin();
+    using T = float;
     constexpr int NV = (EP + 31) / 32, VN = Vec<T>::N;
     constexpr int EG = EP / 4, TM = TB / 4, KS = RD_THREADS / EP;  // 4 EG tiles of TM x 4, KS slices
     constexpr int ROWV = RD_KC / VN;                               // vectors per staged row
@@ -257,6 +257,130 @@ __global__ void __launch_bounds__(RD_THREADS, EP <= 16 && TB == 8 ? 4 : 2) route
     }
     if (parts > 1) cluster.sync();  // the parts' shared memory has been read
     if (part_no) return;
+    __syncthreads();
+    if (tid < E && s_hist[tid]) atomicAdd(&counts[party * E + tid], s_hist[tid]);
+}
+
+// Router logits and gating of bf16 pools whose size is not a multiple of 4, up to 64 experts. A CTA
+// takes TB consecutive tokens of one party and all experts (padded to EP), a warp EM = EP / 8 of
+// the experts; lane l multiplies the 16-byte vectors l, l + 32, ... of the rows (the next ones are
+// in flight meanwhile), each (token, expert) in one chain of FMAs per lane, and the 32 chains are
+// added by a butterfly. That order of summation matters: the chunked one of the fp32 kernel above
+// leaves bf16 logits up to a quarter further off 64 bits (1.07e-7 against 8.7e-8 at d = 3072, E = 63).
+//
+// What bounds it: FMA issue for large batches and pools (a step of TB = EM = 8 is 512 FMAs, 128
+// conversions and 16 loads a warp), the latency of the d / 256 steps for small ones. 3805 tokens of
+// d = 3072 with E = 63: 70 us (a warp per 1 to 8 tokens with the same sums took 308, the chunked
+// kernel 73); 16372, 3072, 43: 246 (965, 275); 1003, 1152, 13: 10.3 (34, 11.9).
+// a[i], i < N, summed over the warp's lanes by the butterfly of warp_sum, each lane keeping N / 32
+// of the sums (those from lane * N / 32 on; N < 32: sum lane / (32 / N))
+template <int N>
+__device__ __forceinline__ void warp_sums(float (&a)[N], int lane) {
+#pragma unroll
+    for (int o = 16, n = N; o > 0; o >>= 1) {
+        if (n > 1) {
+            n /= 2;
+#pragma unroll
+            for (int i = 0; i < N / 2; ++i) {
+                if (i >= n) break;
+                const float send = (lane & o) ? a[i] : a[i + n], keep = (lane & o) ? a[i + n] : a[i];
+                a[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        } else {
+            a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+        }
+    }
+}
+
+template <int EP, int TB>
+__global__ void __launch_bounds__(RD_THREADS, TB * EP >= 256 ? 1 : 2) route_chain_kernel(
+    const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ wr, const float* __restrict__ bias,
+    const int32_t* __restrict__ po, int P, int64_t Tn, int d, int E, int k, int normalize, float* logits,
+    float* probs, int32_t* topk_idx, float* topk_w, int32_t* counts) {
+    pdl_begin();
+    using T = __nv_bfloat16;
+    constexpr int NV = (EP + 31) / 32, VN = Vec<T>::N, EM = EP / (RD_THREADS / 32), N = TB * EM;
+    __shared__ float s_z[TB][EP];
+    __shared__ int s_hist[EP];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, e0 = warp * EM;
+    // the CTA's tokens: group blockIdx.x of TB tokens, enumerated party by party
+    int party = -1, n = 0;
+    int64_t t0 = 0, g = blockIdx.x;
+    for (int q = 0; q < P && party < 0; ++q) {
+        const int64_t a = po ? po[q] : 0, b = po ? po[q + 1] : Tn;
+        const int64_t ng = b > a ? (b - a + TB - 1) / TB : 0;
+        if (g < ng) {
+            party = q;
+            t0 = a + g * TB;
+            n = (int)min64(TB, b - t0);
+        }
+        g -= ng;
+    }
+    if (party < 0) return;
+    if (tid < EP) s_hist[tid] = 0;
+    const int nvec = d / VN;
+    const T *X = x + t0 * d, *W = wr + ((int64_t)party * E + e0) * d;
+    uint4 xr[TB], wv[EM];
+    auto fetch = [&](int v) {
+#pragma unroll
+        for (int i = 0; i < TB; ++i)
+            xr[i] = i < n && v < nvec ? Vec<T>::raw_load(X + (int64_t)i * d + v * VN) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int j = 0; j < EM; ++j)
+            wv[j] = e0 + j < E && v < nvec ? Vec<T>::raw_load(W + (int64_t)j * d + v * VN) : make_uint4(0, 0, 0, 0);
+    };
+    float acc[N];  // token i, expert e0 + j: i * EM + j
+#pragma unroll
+    for (int i = 0; i < N; ++i) acc[i] = 0.f;
+    if (e0 < E) {  // (a whole warp)
+        fetch(lane);
+#pragma unroll 1
+        for (int v = lane; v - lane < nvec; v += 32) {
+            uint4 xc[TB], wc[EM];
+#pragma unroll
+            for (int i = 0; i < TB; ++i) xc[i] = xr[i];
+#pragma unroll
+            for (int j = 0; j < EM; ++j) wc[j] = wv[j];
+            fetch(v + 32);
+            // the vectors' columns in order
+#pragma unroll
+            for (int c = 0; c < VN; ++c) {
+                auto value = [&](const uint4& u) {
+                    const uint32_t w = c < 2 ? u.x : c < 4 ? u.y : c < 6 ? u.z : u.w;
+                    return __uint_as_float(c % 2 ? w & 0xffff0000u : w << 16);
+                };
+                float wq[EM];
+#pragma unroll
+                for (int j = 0; j < EM; ++j) wq[j] = value(wc[j]);
+#pragma unroll
+                for (int i = 0; i < TB; ++i) {
+                    const float xq = value(xc[i]);
+#pragma unroll
+                    for (int j = 0; j < EM; ++j) acc[i * EM + j] = fmaf(xq, wq[j], acc[i * EM + j]);
+                }
+            }
+        }
+    }
+    warp_sums<N>(acc, lane);
+    constexpr int KEEP = N / 32 > 0 ? N / 32 : 1, LANES = N < 32 ? 32 / N : 1;  // sums a lane, lanes a sum
+    if (lane % LANES == 0) {
+#pragma unroll
+        for (int i = 0; i < KEEP; ++i) {
+            const int q = lane / LANES * KEEP + i;
+            s_z[q / EM][e0 + q % EM] = acc[i];
+        }
+    }
+    __syncthreads();
+    for (int tt = warp; tt < n; tt += RD_THREADS / 32) {
+        float z[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int e = lane + 32 * v;
+            z[v] = e < E ? s_z[tt][e] : 0.f;
+            if (bias && e < E) z[v] += bias[party * E + e];
+        }
+        softmax_topk_token<NV>(z, lane, E, k, normalize, t0 + tt, 0, logits, probs, topk_idx, topk_w, s_hist);
+    }
     __syncthreads();
     if (tid < E && s_hist[tid]) atomicAdd(&counts[party * E + tid], s_hist[tid]);
 }
@@ -727,9 +851,9 @@ static cudaError_t launch_gating(const RouteArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-template <typename T, int EP, int TB>
+template <int EP, int TB>
 static cudaError_t launch_route_dot_t(const RouteArgs& a, int parts, cudaStream_t s) {
-    auto kern = route_dot_kernel<T, EP, TB>;
+    auto kern = route_dot_kernel<EP, TB>;
     constexpr size_t smem =
         std::max<size_t>(2 * (size_t)(TB + EP) * RD_LD, (size_t)RD_THREADS * TB + (size_t)TB * EP) * sizeof(float);
     static bool attr = false;
@@ -751,15 +875,14 @@ static cudaError_t launch_route_dot_t(const RouteArgs& a, int parts, cudaStream_
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kern, (const T*)a.x, (const T*)a.w_router, a.bias, a.po, a.P, a.T, a.d, a.E, a.k,
+    return cudaLaunchKernelEx(&cfg, kern, (const float*)a.x, (const float*)a.w_router, a.bias, a.po, a.P, a.T, a.d, a.E, a.k,
                               a.normalize, a.logits, a.probs, a.topk_idx, a.topk_w, a.counts);
 }
 
-// E <= 64. 16 tokens per CTA, 8 while those would not give every SM two CTAs (over 32 experts
+// fp32, E <= 64. 16 tokens per CTA, 8 while those would not give every SM two CTAs (over 32 experts
 // one: the weights of a CTA are staged for its tokens alone, so fewer tokens cost more
 // shared-memory traffic). A cluster of 2, 4 or 8 CTAs per group while the groups leave more
 // than half of the SMs idle and every CTA keeps a chunk of columns.
-template <typename T>
 static cudaError_t launch_route_dot(const RouteArgs& a, cudaStream_t s) {
     if (a.T == 0) return cudaSuccess;
     const bool few = a.T < (a.E > 32 ? 1 : 2) * 16 * (int64_t)num_sms();
@@ -767,12 +890,34 @@ static cudaError_t launch_route_dot(const RouteArgs& a, cudaStream_t s) {
     const int chunks = (a.d + 127) / 128;
     int parts = 1;
     while (parts < 8 && groups * parts * 2 <= num_sms() && parts * 2 <= chunks) parts *= 2;
-#define MOE_DOT(EP) (few ? launch_route_dot_t<T, EP, 8>(a, parts, s) : launch_route_dot_t<T, EP, 16>(a, parts, s))
+#define MOE_DOT(EP) (few ? launch_route_dot_t<EP, 8>(a, parts, s) : launch_route_dot_t<EP, 16>(a, parts, s))
     if (a.E <= 8) return MOE_DOT(8);
     if (a.E <= 16) return MOE_DOT(16);
     if (a.E <= 32) return MOE_DOT(32);
     return MOE_DOT(64);
 #undef MOE_DOT
+}
+
+template <int EP, int TB>
+static cudaError_t launch_route_chain_t(const RouteArgs& a, cudaStream_t s) {
+    const unsigned grid = (unsigned)((a.T + TB - 1) / TB + (a.po ? a.P : 0));
+    (void)launch_pdl(route_chain_kernel<EP, TB>, dim3(grid), dim3(RD_THREADS), 0, s, (const __nv_bfloat16*)a.x,
+                     (const __nv_bfloat16*)a.w_router, a.bias, a.po, a.P, a.T, a.d, a.E, a.k, a.normalize, a.logits, a.probs,
+                     a.topk_idx, a.topk_w, a.counts);
+    return cudaGetLastError();
+}
+
+// bf16, E <= 64. Eight tokens a CTA (fewer read W_r more often), two up to four tokens per SM, where
+// the latency of a CTA's steps decides (600 tokens of d = 3072, E = 63: 18.4 us with two, 21.7 with
+// eight; 700: 24.7, 22.6; 100 of 2048, E = 13: 8.3, 10.3).
+static cudaError_t launch_route_chain(const RouteArgs& a, cudaStream_t s) {
+    const bool few = a.T <= 4 * (int64_t)num_sms();
+#define MOE_CHAIN(EP) (few ? launch_route_chain_t<EP, 2>(a, s) : launch_route_chain_t<EP, 8>(a, s))
+    if (a.E <= 8) return MOE_CHAIN(8);
+    if (a.E <= 16) return MOE_CHAIN(16);
+    if (a.E <= 32) return MOE_CHAIN(32);
+    return MOE_CHAIN(64);
+#undef MOE_CHAIN
 }
 
 // E > 64, fp32: the router's products x W_r[p]^T by the grouped fp32 GEMM into `logits` (groups = parties), then the gating pass reads them back, adds the
@@ -807,7 +952,7 @@ cudaError_t launch_route(const RouteArgs& a, bool bf16, bool from_logits, cudaSt
     if (a.T == 0) return cudaSuccess;
     if (bf16 && (a.E % 4 == 0 || a.E > 64)) return launch_route_tc(a, s);
     if (a.E > 64) return launch_route_wide_f32(a, s);
-    return bf16 ? launch_route_dot<__nv_bfloat16>(a, s) : launch_route_dot<float>(a, s);
+    return bf16 ? launch_route_chain(a, s) : launch_route_dot(a, s);
 }
 
 cudaError_t launch_aux_loss(const float* probs, const int32_t* counts, const int32_t* po, int P,
