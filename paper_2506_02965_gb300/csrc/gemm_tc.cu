@@ -277,12 +277,11 @@ __device__ __forceinline__ void route_epilogue_short(const Params& p, const Tile
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
 #pragma unroll
-        for (int j = 0; j < V; ++j) {
-            ez[j] = l8 + 8 * j < E ? expf(z[j] - mx) : 0.f;
-            sum += ez[j];
-        }
+        for (int j = 0; j < V; ++j) ez[j] = l8 + 8 * j < E ? expf(z[j] - mx) : 0.f;
+        // in order of the experts, as one thread adds them: the gates of a token are the same bits
+        // whatever batch it is in
 #pragma unroll
-        for (int o = 1; o < 8; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        for (int e = 0; e < BN; ++e) sum += __shfl_sync(0xffffffffu, ez[e / 8], e % 8, 8);
 #pragma unroll
         for (int j = 0; j < V; ++j) {
             const int e = l8 + 8 * j;
