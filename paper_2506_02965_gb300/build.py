@@ -18,7 +18,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmoe.so")
 SOURCES = ["route.cu", "dispatch.cu", "gemm_f32.cu", "gemm_tc.cu", "train.cu", "moe_abi.cu"]
-HEADERS = ["moe_common.cuh", "moe_internal.h", "tc_ptx.cuh"]
+HEADERS = ["device_state.h", "moe_common.cuh", "moe_internal.h", "tc_ptx.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-I" + os.path.join(ROOT, "include")]

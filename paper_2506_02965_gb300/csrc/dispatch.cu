@@ -493,21 +493,11 @@ __global__ void __launch_bounds__(256, 2) unpermute_reduce_kernel(
 }
 
 // ----------------------------------------------------------------------------- launchers
-static int dispatch_sms() {
-    static int n = 0;
-    if (!n) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 148;
-    }
-    return n;
-}
 // Warps per token: doubled while the batch has fewer than 16 warps per SM and each part still
 // gets a step of columns (rows of `vecs` 16-byte vectors, `step` of them per warp and step).
 static int warps_per_token(int64_t T, int vecs, int step) {
     int w = 1;
-    while (w < TOK_WARPS && T * w < 16 * (int64_t)dispatch_sms() && vecs > step * w) w *= 2;
+    while (w < TOK_WARPS && T * w < 16 * (int64_t)sm_count() && vecs > step * w) w *= 2;
     return w;
 }
 static unsigned token_blocks(int64_t T, int wpt) { return (unsigned)((T * wpt + TOK_WARPS - 1) / TOK_WARPS); }
@@ -643,7 +633,6 @@ cudaError_t launch_unpermute_reduce(const void* dx_perm, const int32_t* slot_of,
 static __device__ __align__(256) int32_t g_dispatch_scratch[kNoAllocScratchInts];
 
 namespace {
-constexpr int kMaxDevices = 64;
 // Device address of g_dispatch_scratch per device, looked up on the first call there.
 // Two threads that make their first call at once both look it up and store the same
 // value; the atomic makes that well defined.

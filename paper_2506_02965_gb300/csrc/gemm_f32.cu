@@ -692,17 +692,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) gemm_f32_kernel(const __grid_cons
 }
 
 // ------------------------------------------------------------------------ host side
-static int sm_count() {
-    static int n = 0;
-    if (!n) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 148;
-    }
-    return n;
-}
-
 // floats per copy that the lines of an operand allow: their length, the distance of its
 // groups and its address are multiples of it
 static int vec_of(const void* base, int64_t ld, int64_t group = 0) {
@@ -715,17 +704,16 @@ template <bool A_MN, bool B_MN, bool VAR_K, int EPI, int BN>
 static cudaError_t launch_bn(const Params& p, int64_t tiles, cudaStream_t s) {
     auto kern = gemm_f32_kernel<A_MN, B_MN, VAR_K, EPI, BN>;
     constexpr size_t smem = smem_bytes(BN);
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        // the roles' register shares must not exceed the launch's (setmaxnreg would wait forever)
+    cudaError_t e = allow_dynamic_smem<gemm_f32_kernel<A_MN, B_MN, VAR_K, EPI, BN>>(smem);
+    if (e != cudaSuccess) return e;
+    // the roles' register shares must not exceed the launch's (setmaxnreg would wait forever)
+    static std::atomic<int> regs{0};
+    if (!regs) {
         cudaFuncAttributes fa;
         if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
-        if (fa.numRegs * NTHREADS < 32 * (PROD_WARPS * REG_PROD + EPI_W * REG_EPI + 4 * REG_MMA))
-            return cudaErrorInvalidConfiguration;
-        attr = true;
+        regs = fa.numRegs;
     }
+    if (regs * NTHREADS < 32 * (PROD_WARPS * REG_PROD + EPI_W * REG_EPI + 4 * REG_MMA)) return cudaErrorInvalidConfiguration;
     const unsigned grid = (unsigned)std::min<int64_t>(tiles, sm_count());
     (void)launch_pdl(kern, dim3(grid), dim3(NTHREADS), smem, s, p);
     return cudaGetLastError();

@@ -1476,17 +1476,6 @@ static bool make_map_kblocks(CUtensorMap* m, const void* base, int64_t inner, in
 static uint64_t g_wait_ns = 2000000000ull;
 static int g_pairs = MOE_PAIRS_AUTO;  // CTA-pair tiles for the 256-wide M-variable expert GEMMs
 
-static int sm_count() {
-    static int n = 0;
-    if (!n) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 148;
-    }
-    return n;
-}
-
 // M-tiles per band of the tile order for `c` tiles in flight at once (the persistent
 // CTAs, or CTA pairs): about sqrt(c).
 static int band_for(int c) {
@@ -1518,17 +1507,15 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
     const int extra = EPI == EPI_ROUTE ? p.hist_n * 4 : epi_stage_bytes(EPI);
     const int smem_max = NST * STB + 1024 + extra_max + mma_overread(AR);
     const int smem = NST * STB + 1024 + extra + mma_overread(AR);
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    const cudaError_t e = allow_dynamic_smem<grouped_gemm_kernel<BN, B_MN, VAR_K, EPI, PAIR, DW2, OCC, EW, AR>>(smem_max);
+    if (e != cudaSuccess) return e;
     if (tiles_ub <= 0) return cudaSuccess;
     if constexpr (PAIR) {
         // persistent 2-CTA clusters: no more than can be resident at once (a cluster needs
         // both SMs of a TPC, so fewer than SMs/2 may fit)
-        static int max_clusters = 0;
+        static std::atomic<int> resident[kMaxDevices] = {};
+        const int dev = current_device();
+        int max_clusters = dev >= 0 && dev < kMaxDevices ? resident[dev].load() : 0;
         if (!max_clusters) {
             cudaLaunchConfig_t q = {};
             q.gridDim = dim3(2 * (sm_count() / 2));
@@ -1541,12 +1528,11 @@ static cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CU
             qa[0].val.clusterDim.z = 1;
             q.attrs = qa;
             q.numAttrs = 1;
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, kern, &q) != cudaSuccess || n <= 0) {
+            if (cudaOccupancyMaxActiveClusters(&max_clusters, kern, &q) != cudaSuccess || max_clusters <= 0) {
                 (void)cudaGetLastError();
-                n = sm_count() / 2;
+                max_clusters = sm_count() / 2;
             }
-            max_clusters = n;
+            if (dev >= 0 && dev < kMaxDevices) resident[dev] = max_clusters;
         }
         const int clusters = (int)std::min<int64_t>(tiles_ub, max_clusters);
         P1.band = P2.band = band_for(clusters);

@@ -8,6 +8,7 @@
 #include <string>
 
 #include "../../include/moe.h"
+#include "device_state.h"
 #include "moe_internal.h"
 
 using namespace moe;
@@ -101,8 +102,7 @@ struct SideStream {
     cudaStream_t s = nullptr;
     cudaEvent_t fork = nullptr, mid = nullptr, join = nullptr;
 };
-constexpr int kMaxDev = 64;
-SideStream g_side[kMaxDev];
+SideStream g_side[kMaxDevices];
 std::mutex g_side_mu;
 
 // Requires g_side_mu held by the caller.
@@ -110,7 +110,7 @@ cudaError_t side_stream(SideStream** out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDev) return cudaErrorInvalidDevice;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     SideStream& ss = g_side[dev];
     if (!ss.s) {
         if ((e = cudaStreamCreateWithFlags(&ss.s, cudaStreamNonBlocking)) != cudaSuccess) return e;

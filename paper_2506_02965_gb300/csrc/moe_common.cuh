@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "../../include/moe.h"
+#include "device_state.h"
 
 namespace moe {
 

@@ -823,23 +823,12 @@ static cudaError_t launch_route_bwd_reduce(const RouteBwdArgs& a, const float* p
 }
 
 // ----------------------------------------------------------------------------- launchers
-static int num_sms() {
-    static int n = 0;
-    if (!n) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 148;
-    }
-    return n;
-}
-
 // gating of logits in a.logits_in
 static cudaError_t launch_gating(const RouteArgs& a, cudaStream_t s) {
     const int E = a.E;
     const size_t smem = a.P * E <= HIST_SMEM ? (size_t)a.P * E * sizeof(int) : 0;
     const int64_t groups_ub = a.T + a.P;  // upper bound with TPW = 1
-    int blocks = (int)min64((groups_ub + 7) / 8, (int64_t)num_sms() * 8);
+    int blocks = (int)min64((groups_ub + 7) / 8, (int64_t)sm_count() * 8);
     if (blocks < 1) blocks = 1;
 #define MOE_GATE(EM, TP)                                                                              \
     (void)launch_pdl(route_kernel<EM, TP>, dim3(blocks), dim3(256), smem, s, a.bias, a.logits_in, a.po, \
@@ -856,12 +845,8 @@ static cudaError_t launch_route_dot_t(const RouteArgs& a, int parts, cudaStream_
     auto kern = route_dot_kernel<EP, TB>;
     constexpr size_t smem =
         std::max<size_t>(2 * (size_t)(TB + EP) * RD_LD, (size_t)RD_THREADS * TB + (size_t)TB * EP) * sizeof(float);
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    const cudaError_t e = allow_dynamic_smem<route_dot_kernel<EP, TB>>(smem);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(((a.T + TB - 1) / TB + (a.po ? a.P : 0)) * parts));
     cfg.blockDim = dim3(RD_THREADS);
@@ -885,11 +870,11 @@ static cudaError_t launch_route_dot_t(const RouteArgs& a, int parts, cudaStream_
 // than half of the SMs idle and every CTA keeps a chunk of columns.
 static cudaError_t launch_route_dot(const RouteArgs& a, cudaStream_t s) {
     if (a.T == 0) return cudaSuccess;
-    const bool few = a.T < (a.E > 32 ? 1 : 2) * 16 * (int64_t)num_sms();
+    const bool few = a.T < (a.E > 32 ? 1 : 2) * 16 * (int64_t)sm_count();
     const int64_t groups = (a.T + (few ? 8 : 16) - 1) / (few ? 8 : 16);
     const int chunks = (a.d + 127) / 128;
     int parts = 1;
-    while (parts < 8 && groups * parts * 2 <= num_sms() && parts * 2 <= chunks) parts *= 2;
+    while (parts < 8 && groups * parts * 2 <= sm_count() && parts * 2 <= chunks) parts *= 2;
 #define MOE_DOT(EP) (few ? launch_route_dot_t<EP, 8>(a, parts, s) : launch_route_dot_t<EP, 16>(a, parts, s))
     if (a.E <= 8) return MOE_DOT(8);
     if (a.E <= 16) return MOE_DOT(16);
@@ -911,7 +896,7 @@ static cudaError_t launch_route_chain_t(const RouteArgs& a, cudaStream_t s) {
 // the latency of a CTA's steps decides (600 tokens of d = 3072, E = 63: 18.4 us with two, 21.7 with
 // eight; 700: 24.7, 22.6; 100 of 2048, E = 13: 8.3, 10.3).
 static cudaError_t launch_route_chain(const RouteArgs& a, cudaStream_t s) {
-    const bool few = a.T <= 4 * (int64_t)num_sms();
+    const bool few = a.T <= 4 * (int64_t)sm_count();
 #define MOE_CHAIN(EP) (few ? launch_route_chain_t<EP, 2>(a, s) : launch_route_chain_t<EP, 8>(a, s))
     if (a.E <= 8) return MOE_CHAIN(8);
     if (a.E <= 16) return MOE_CHAIN(16);
@@ -1025,17 +1010,11 @@ static cudaError_t launch_route_bwd_simt(const RouteBwdArgs& a, void* ws, cudaSt
     constexpr int SLAB = RB_HALF * Vec<T>::N;
     dim3 grid((unsigned)nch, (a.E + RB_ET - 1) / RB_ET, (a.d + SLAB - 1) / SLAB);
     const size_t smem = (size_t)RB_HALF * RB_ET * Vec<T>::N * sizeof(float);
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(route_bwd_partial_kernel<T>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    cudaError_t e = allow_dynamic_smem<route_bwd_partial_kernel<T>>(smem);
+    if (e != cudaSuccess) return e;
     (void)launch_pdl(route_bwd_partial_kernel<T>, dim3(grid), dim3(2 * RB_HALF), smem, s, (const T*)a.x,
                      a.dlogits, a.po, a.P, a.T, a.d, a.E, part_dw, part_db);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = launch_route_bwd_reduce<T>(a, part_dw, part_db, RB_CH, s)) != cudaSuccess) return e;
     if (a.dx_router && a.T > 0) {  // dx_router[t] = dlogits[t] W_r[p(t)], K = E
         GemmMArgs m{};

@@ -106,17 +106,6 @@ __global__ void __launch_bounds__(256) sgd_update_kernel(T* __restrict__ w, cons
     }
 }
 
-static int sm_count_train() {
-    static int n = 0;
-    if (!n) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
-            n = 148;
-    }
-    return n;
-}
-
 cudaError_t launch_sgd_update(void* w, const void* dw, float* master, int64_t n_groups, int64_t group_elems,
                               const int32_t* counts, float lr, bool bf16, cudaStream_t s) {
     if (n_groups == 0 || group_elems == 0) return cudaSuccess;
@@ -125,7 +114,7 @@ cudaError_t launch_sgd_update(void* w, const void* dw, float* master, int64_t n_
                      ((uintptr_t)master % 16 == 0);
     // about 8 CTAs per SM over all groups, none with less than one vector per thread
     const int64_t work = vec ? group_elems / vn : group_elems;
-    int64_t bx = std::max<int64_t>(1, (8 * (int64_t)sm_count_train() + n_groups - 1) / n_groups);
+    int64_t bx = std::max<int64_t>(1, (8 * (int64_t)sm_count() + n_groups - 1) / n_groups);
     bx = std::min<int64_t>(bx, (work + 255) / 256);
     const dim3 grid((unsigned)std::max<int64_t>(bx, 1), (unsigned)n_groups);
 #define MOE_SGD(TT, V, M)                                                                      \
