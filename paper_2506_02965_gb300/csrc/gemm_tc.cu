@@ -1794,14 +1794,14 @@ cudaError_t launch_gemm_k(const GemmKArgs& g, bool bf16, cudaStream_t s) {
 
 // One launch of an M-variable GEMM with MN-major B (dA with the SwiGLU-backward
 // epilogue, or dX) and a K-variable weight-gradient GEMM over the same groups (dW2, or
-// dW1); see the DW2 kernel parameter. Falls back to two
-// launches when the shapes do not fit one 256-wide template.
+// dW1), where both fit one 256-wide template (see the DW2 kernel parameter), else two.
+bool gemm_mk_fits(const GemmMArgs& g, const GemmKArgs& k) {
+    return g.rows.offsets && k.rows.offsets && g.G == k.G && !g.b_kmajor && (g.epi == EPI_SWIGLU_BWD || g.epi == EPI_STORE) &&
+           g.N % 256 == 0 && k.N % 256 == 0 && k.M % tc::BM == 0 && k.epi == EPI_STORE && g.G <= tc::MAX_GROUPS;
+}
 cudaError_t launch_gemm_mk(const GemmMArgs& g, const GemmKArgs& k, cudaStream_t s) {
     using namespace tc;
-    const bool fits = g.rows.offsets && k.rows.offsets && g.G == k.G && !g.b_kmajor &&
-                      (g.epi == EPI_SWIGLU_BWD || g.epi == EPI_STORE) && g.N % 256 == 0 &&
-                      k.N % 256 == 0 && k.M % BM == 0 && k.epi == EPI_STORE && g.G <= MAX_GROUPS;
-    if (!fits) {
+    if (!gemm_mk_fits(g, k)) {
         cudaError_t e = launch_gemm_m(g, true, s);
         if (e != cudaSuccess) return e;
         return launch_gemm_k(k, true, s);

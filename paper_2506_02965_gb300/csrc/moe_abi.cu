@@ -122,6 +122,50 @@ cudaError_t side_stream(SideStream** out) {
     return cudaSuccess;
 }
 
+// Shapes of the routed experts' backward GEMMs (the operands are the call's):
+// dA = dY W2 with the SwiGLU-backward epilogue -> dH; dXp = dH W1; dW2[e] = dY_e^T A_e;
+// dW1[e] = dH_e^T Xp_e.
+struct BwdGemms {
+    GemmMArgs a, x;
+    GemmKArgs w2, w1;
+    // Each M-variable GEMM runs with its weight gradient in one persistent launch (one tail
+    // instead of two, and no two persistent grids contending for SMs): dA then dW2 (which needs
+    // only dY and A), dX then dW1 (which needs dH). Widths that do not fit that launch's 256-wide
+    // tiles make it two, one after the other. A GEMM that runs as CTA-pair tiles, a dX whose dW1
+    // does, and the fp32 path, instead put the weight gradient on a side stream: dW2 alongside
+    // dA, dW1 alongside dX once dH exists. (Also for widths that do not fit: whole steps of 6000
+    // tokens, d = 384, E = 8, F = 1920 289 -> 298 us; 1003, 1152, 13, 1920 252 -> 248; others of
+    // 128 mod 256 in d or F equal.)
+    bool with_a, with_x;            // on the caller's stream
+    int a_launches, x_launches;
+};
+BwdGemms bwd_gemms(const moe_config* cfg, const int32_t* offsets, const int32_t* group_expert) {
+    const bool bf16 = cfg->dtype == MOE_BF16;
+    const int d = cfg->d_model, F = cfg->d_ff;
+    BwdGemms g{};
+    g.a.G = g.x.G = g.w2.G = g.w1.G = cfg->n_experts;
+    g.a.rows = g.x.rows = g.w2.rows = g.w1.rows = GroupRows{offsets, (int)(cfg->T * cfg->top_k), 0, 0, 0};
+    g.a.group_expert = g.x.group_expert = g.w2.group_expert = g.w1.group_expert = group_expert;
+    g.a.b_group_elems = (int64_t)d * F;
+    g.a.b_kmajor = g.x.b_kmajor = false;  // W2[e] is [d, F] = [K, N], W1[e] is [2F, d]
+    g.a.N = F;
+    g.a.K = d;
+    g.a.epi = EPI_SWIGLU_BWD;
+    g.x.b_group_elems = (int64_t)2 * F * d;
+    g.x.N = d;
+    g.x.K = 2 * F;
+    g.x.epi = EPI_STORE;
+    g.w2.M = d;
+    g.w2.N = F;
+    g.w1.M = 2 * F;
+    g.w1.N = d;
+    g.with_a = bf16 && !gemm_m_uses_pairs(g.a);
+    g.with_x = bf16 && !gemm_m_uses_pairs(g.x) && !gemm_k_uses_pairs(g.w1);
+    g.a_launches = g.with_a && gemm_mk_fits(g.a, g.w2) ? 1 : 2;
+    g.x_launches = g.with_x && gemm_mk_fits(g.x, g.w1) ? 1 : 2;
+    return g;
+}
+
 }  // namespace
 
 extern "C" {
@@ -489,74 +533,37 @@ moe_status moe_expert_ffn_bwd(const moe_config* cfg, const void* x_perm, const i
         REQUIRE_VEC(dh_sh);
         REQUIRE_VEC(dx_sh);
     }
-    // dA = dY W2 with the SwiGLU-backward epilogue -> dH
-    GemmMArgs a{};
-    a.group_expert = group_expert;
-    a.G = E;
-    a.rows = GroupRows{offsets, (int)TK, 0, 0, 0};
+    BwdGemms g = bwd_gemms(cfg, offsets, group_expert);
+    GemmMArgs &a = g.a, &b = g.x;
+    GemmKArgs &w2g = g.w2, &w1g = g.w1;
     a.a = dy_perm;
     a.b = w2;
-    a.b_group_elems = (int64_t)d * F;
-    a.b_kmajor = false;  // W2[e] is [d, F] = [K, N]
-    a.N = F;
-    a.K = d;
-    a.epi = EPI_SWIGLU_BWD;
     a.aux = h_gu;
     a.out0 = dh;
-    // dXp = dH W1
-    GemmMArgs b{};
-    b.group_expert = group_expert;
-    b.G = E;
-    b.rows = GroupRows{offsets, (int)TK, 0, 0, 0};
     b.a = dh;
     b.b = w1;
-    b.b_group_elems = (int64_t)2 * F * d;
-    b.b_kmajor = false;  // W1[e] is [2F, d] = [K, N]
-    b.N = d;
-    b.K = 2 * F;
-    b.epi = EPI_STORE;
     b.out0 = dx_perm;
-    // dW2[e] = dY_e^T A_e ; dW1[e] = dH_e^T Xp_e
-    GemmKArgs w2g{};
-    w2g.group_expert = group_expert;
-    w2g.G = E;
-    w2g.rows = GroupRows{offsets, (int)TK, 0, 0, 0};
     w2g.a = dy_perm;
     w2g.b = act;
-    w2g.M = d;
-    w2g.N = F;
     w2g.out = dw2;
-    GemmKArgs w1g{};
-    w1g.group_expert = group_expert;
-    w1g.G = E;
-    w1g.rows = GroupRows{offsets, (int)TK, 0, 0, 0};
     w1g.a = dh;
     w1g.b = x_perm;
-    w1g.M = 2 * F;
-    w1g.N = d;
     w1g.out = dw1;
-    // Each M-variable GEMM runs with its weight gradient in one persistent launch (one
-    // tail instead of two, and no two persistent grids contending for SMs): dA then dW2
-    // (which needs only dY and A), dX then dW1 (which needs dH). A GEMM that runs as
-    // CTA-pair tiles, a dX whose dW1 does, and the fp32 path, instead put the weight gradient
-    // on a side stream: dW2 alongside dA, dW1 alongside dX once dH exists.
-    const bool fuse_a = bf16 && !gemm_m_uses_pairs(a);  // the same rules as moe_expert_ffn_bwd_kernels
-    const bool fuse_b = bf16 && !gemm_m_uses_pairs(b) && !gemm_k_uses_pairs(w1g);
     SideStream* ss = nullptr;
     std::unique_lock<std::mutex> side_lock(g_side_mu, std::defer_lock);
-    if (!fuse_a || !fuse_b) {
+    if (!g.with_a || !g.with_x) {
         side_lock.lock();  // held until the join wait is queued (the events are shared)
         if ((st = cuda_status(side_stream(&ss), "side stream"))) return st;
         if ((st = cuda_status(cudaEventRecord(ss->fork, s), "fork"))) return st;
         if ((st = cuda_status(cudaStreamWaitEvent(ss->s, ss->fork, 0), "fork"))) return st;
     }
-    if (fuse_a) {
+    if (g.with_a) {
         if ((st = cuda_status(launch_gemm_mk(a, w2g, s), "expert dA+dW2 gemm"))) return st;
     } else {
         if ((st = cuda_status(launch_gemm_k(w2g, bf16, ss->s), "expert dW2 gemm"))) return st;
         if ((st = cuda_status(launch_gemm_m(a, bf16, s), "expert dA gemm"))) return st;
     }
-    if (fuse_b) {
+    if (g.with_x) {
         if ((st = cuda_status(launch_gemm_mk(b, w1g, s), "expert dX+dW1 gemm"))) return st;
     } else {
         if ((st = cuda_status(cudaEventRecord(ss->mid, s), "mid"))) return st;
@@ -700,28 +707,10 @@ moe_status moe_expert_ffn_bwd_kernels(const moe_config* cfg, int32_t* count) {
     moe_status st = check_cfg(cfg);
     if (st) return st;
     REQUIRE(count);
-    const bool bf16 = cfg->dtype == MOE_BF16;
-    const int64_t TK = cfg->T * cfg->top_k;
     static const int32_t marker = 0;  // offsets mode: only its non-null-ness is looked at
-    GemmMArgs a{}, b{};
-    a.G = b.G = cfg->n_experts;
-    a.rows = b.rows = GroupRows{&marker, (int)TK, 0, 0, 0};
-    a.b_kmajor = b.b_kmajor = false;
-    a.N = cfg->d_ff;
-    a.K = cfg->d_model;
-    a.epi = EPI_SWIGLU_BWD;
-    b.N = cfg->d_model;
-    b.K = 2 * cfg->d_ff;
-    b.epi = EPI_STORE;
+    const BwdGemms g = bwd_gemms(cfg, &marker, nullptr);
     int n = 0;
-    if (TK > 0) {
-        n += (bf16 && !gemm_m_uses_pairs(a)) ? 1 : 2;
-        GemmKArgs w1g{};
-        w1g.G = cfg->n_experts;
-        w1g.M = 2 * cfg->d_ff;
-        w1g.N = cfg->d_model;
-        n += (bf16 && !gemm_m_uses_pairs(b) && !gemm_k_uses_pairs(w1g)) ? 1 : 2;
-    }
+    if (cfg->T * cfg->top_k > 0) n += g.a_launches + g.x_launches;
     if (cfg->n_shared && cfg->T > 0) n += 4;
     *count = n;
     return MOE_OK;

@@ -143,7 +143,9 @@ struct GemmKArgs {
 cudaError_t launch_gemm_m(const GemmMArgs& g, bool bf16, cudaStream_t s, const GemmMArgs* second = nullptr);
 cudaError_t launch_gemm_k(const GemmKArgs& g, bool bf16, cudaStream_t s);
 // bf16: an M-variable GEMM (MN-major B) and a K-variable GEMM over the same groups in
-// one persistent launch (the second problem's tiles after the first's)
+// one persistent launch (the second problem's tiles after the first's), or two where
+// gemm_mk_fits does not hold
+bool gemm_mk_fits(const GemmMArgs& m, const GemmKArgs& k);
 cudaError_t launch_gemm_mk(const GemmMArgs& m, const GemmKArgs& k, cudaStream_t s);
 // whether launch_gemm_m runs this GEMM as CTA-pair tiles (bf16)
 bool gemm_m_uses_pairs(const GemmMArgs& g, const GemmMArgs* second = nullptr);

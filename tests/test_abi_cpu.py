@@ -174,6 +174,20 @@ def test_backward_kernel_count_follows_the_tile_mode(L):
     assert L.moe_expert_ffn_bwd_kernels(L.make_config(0, 1024, 16, 2816, 2)) == 0
 
 
+def test_backward_kernel_count_of_widths_that_share_no_launch(L):
+    """Widths of 128 mod 256: the 256-wide form that takes a GEMM and its weight gradient in
+    one launch does not fit, whether it is F (dA with dW2; N of both) or d (dX with dW1)."""
+    assert L.moe_expert_ffn_bwd_kernels(L.make_config(1003, 1152, 13, 1920, 3)) == 4
+    assert L.moe_expert_ffn_bwd_kernels(L.make_config(800, 384, 40, 128, 2)) == 4
+    assert L.moe_expert_ffn_bwd_kernels(L.make_config(800, 384, 40, 256, 2)) == 3
+    try:
+        L.moe_set_gemm_pairs(L.MOE_PAIRS_OFF)
+        assert L.moe_expert_ffn_bwd_kernels(L.make_config(800, 512, 40, 384, 2)) == 3
+        assert L.moe_expert_ffn_bwd_kernels(L.make_config(800, 384, 40, 384, 2)) == 4
+    finally:
+        L.moe_set_gemm_pairs(L.MOE_PAIRS_AUTO)
+
+
 def test_binding_refuses_to_load_without_library(L, monkeypatch):
     monkeypatch.setattr(L, "LIB_PATH", "/nonexistent/libmoe.so")
     with pytest.raises(ImportError):
