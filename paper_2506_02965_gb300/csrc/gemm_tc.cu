@@ -1568,7 +1568,12 @@ void set_gemm_pairs(int mode) { tc::g_pairs = mode; }
 // Tiles of `tile` rows that `rows` rows in G groups make, if the router spreads them evenly:
 // each group has r = rows / G of them give or take sqrt(r), so the mean of the tiles at half
 // a deviation below and above. (The counts are on the device; a rule that waited for them
-// would synchronise.)
+// would synchronise.) An uneven router ends other tiles: over 60 shapes of 4 to 45 experts,
+// 225 to 6400 tokens the rule below takes 0.77 of the time of pairs from four rounds on, at
+// Zipf(1.2) popularity (0.47 to 1.04) as at even; of 50 whose tiles lie within a few of a whole
+// round 0.98, where a skewed batch can fall on the other side of it (2000 tokens, E = 8,
+// d = 1024, F = 2816: 105 -> 115 us of a forward; even 100 -> 99). Averaging the rounds over more
+// uneven counts moved such batches about without gain (0.99).
 static int64_t expected_tiles(const GroupRows& gr, int G, int tile) {
     if (!gr.offsets) return (int64_t)G * ((gr.rows + tile - 1) / tile);
     const double r = (double)gr.rows / G, dev = 0.5 * std::sqrt(r);
