@@ -1,7 +1,7 @@
 // Token dispatch (the "send h to the host of idx" step of Alg. 3 as one expert-major
 // buffer), the gate-weighted combine of Alg. 3 and the backward of both (Alg. 5,
-// Sec. 3.2). All memory-bound: 16-byte vector loads/stores, one warp per token or
-// per permuted row, no floating-point atomics (every result is deterministic).
+// Sec. 3.2). All memory-bound: 16-byte vector loads/stores, one to eight warps per token
+// or one per permuted row, no floating-point atomics (every result is deterministic).
 #include <algorithm>
 #include <atomic>
 

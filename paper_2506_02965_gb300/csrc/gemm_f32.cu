@@ -193,12 +193,12 @@ __device__ __forceinline__ void fma_chains(const float* A, int64_t lda, int rows
 
 // The outputs of an epilogue warp (rows mrow.. of the tile, columns col0.. of either half) that it
 // has stored as not finite, computed again and stored: after the warp's last tile, when nothing
-// else is in registers, so that it costs the other outputs nothing. (dG and dU are not finite where dA is
-// not; a finite dA beside a G or U that is not comes out within rounding.) A, B: the operands of the tile's group;
-// out_row: the output row of its first. One chain per output costs about what the FFMA
-// kernel that this replaces took for any values: a step of 1501 tokens, d = 1000, F = 1366 of which
-// nearly all sums leave the range 4.1 to 7.2 ms (5.4 before; finite 1.13); NaN stop early, 1.6 to
-// 1.9 ms for all, 3.4 for a single one in dY.
+// else is in registers, so that it costs the other outputs nothing. (dG and dU are not finite
+// where dA is not; a finite dA beside a G or U that is not comes out within rounding.) A, B: the
+// operands of the tile's group; out_row: the output row of its first. One chain per output costs
+// about what the FFMA kernel that this replaces took for any values: a step of 1501 tokens, d =
+// 1000, F = 1366 of which nearly all sums leave the range 4.1 to 7.2 ms (5.4 before; finite 1.13);
+// NaN stop early, 1.6 to 1.9 ms for all, 3.4 for a single one in dY.
 template <bool A_MN, bool B_MN, int EPI, int BN>
 static __device__ __forceinline__ void repair(const Params& p, const float* A, const float* B, int64_t out_row, int n0, int mrow,
                                        int mrows, int klen, int col0, float* st) {

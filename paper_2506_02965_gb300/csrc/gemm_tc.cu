@@ -903,32 +903,32 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
                         tma_load_3d(sa, &tmA, fb, 0, arow, kb * KPS);
                         tma_load_3d(sb, &tmB, fb, 0, brow, kb * KPS);
                     } else {
-                    if (!A_MN && !dw) {
-                        if (SWAP && trows) {
-                            for (int r = 0; r < trows; r += 32)
+                        if (!A_MN && !dw) {
+                            if (SWAP && trows) {
+                                for (int r = 0; r < trows; r += 32)
 #pragma unroll
-                                for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX + r * 128, mAs, fb, k0 + KB * i, arow + r);
+                                    for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX + r * 128, mAs, fb, k0 + KB * i, arow + r);
+                            } else {
+#pragma unroll
+                                for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX, mA, fb, k0 + KB * i, arow);
+                            }
                         } else {
 #pragma unroll
-                            for (int i = 0; i < KPS; ++i) load(sa + i * A_BOX, mA, fb, k0 + KB * i, arow);
+                            for (int i = 0; i < BM / 64; ++i) load(sa + i * ATOM, mA, fb, ti.m0 + 64 * i, arow + k0);
                         }
-                    } else {
+                        if (!B_MN) {
 #pragma unroll
-                        for (int i = 0; i < BM / 64; ++i) load(sa + i * ATOM, mA, fb, ti.m0 + 64 * i, arow + k0);
-                    }
-                    if (!B_MN) {
+                            for (int i = 0; i < KPS; ++i) {
+                                load(sb + i * B_BOX, mB, fb, k0 + KB * i, brow);
+                                // SwiGLU forward: 128 gate rows, then 128 up rows of the same features
+                                // (in a pair the leader holds the gate half and the peer the up half)
+                                if (EPI == EPI_SWIGLU_FWD && !PAIR) load(sb + i * B_BOX + 128 * 128, mB, fb, k0 + KB * i, brow + F);
+                            }
+                        } else {
 #pragma unroll
-                        for (int i = 0; i < KPS; ++i) {
-                            load(sb + i * B_BOX, mB, fb, k0 + KB * i, brow);
-                            // SwiGLU forward: 128 gate rows, then 128 up rows of the same features
-                            // (in a pair the leader holds the gate half and the peer the up half)
-                            if (EPI == EPI_SWIGLU_FWD && !PAIR) load(sb + i * B_BOX + 128 * 128, mB, fb, k0 + KB * i, brow + F);
+                            for (int i = 0; i < BNL / 64; ++i)
+                                load(sb + i * ATOM_B, mB, fb, ti.n0 + (int)rank * BNL + 64 * i, brow + k0);
                         }
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < BNL / 64; ++i)
-                            load(sb + i * ATOM_B, mB, fb, ti.n0 + (int)rank * BNL + 64 * i, brow + k0);
-                    }
                     }
                     if constexpr (PAIR) {
                         s_fill_bytes[stage] = local_bar ? 0 : tile_bytes / NPAIR;

@@ -42,7 +42,7 @@ struct RouteBwdArgs {
 };
 
 cudaError_t launch_route(const RouteArgs& a, bool bf16, bool from_logits, cudaStream_t s);
-// bf16 router logits on the tensor cores with the gating epilogue (E <= 64, E % 4 == 0)
+// bf16 router logits on the tensor cores with the gating epilogue (E > 64, or E % 4 == 0)
 cudaError_t launch_route_tc(const RouteArgs& a, cudaStream_t s);
 cudaError_t launch_aux_loss(const float* probs, const int32_t* counts, const int32_t* po, int P,
                             int64_t T, int E, int k, float alpha, float* loss, float* coef,

@@ -1,6 +1,6 @@
 // Gating function of the MoE layer (Alg. 7) and its backward, plus the per-party
-// load-balancing loss. SIMT kernels: x is read once with 16-byte
-// vector loads, logits are reduced with warp shuffles, top-k is a warp argmax.
+// load-balancing loss, on the CUDA cores (the bf16 router's GEMMs are in gemm_tc.cu): 16-byte
+// vector loads, reductions by warp shuffles, top-k as a warp argmax.
 #include <cfloat>
 
 #include <cooperative_groups.h>
@@ -905,8 +905,9 @@ static cudaError_t launch_route_chain(const RouteArgs& a, cudaStream_t s) {
 #undef MOE_CHAIN
 }
 
-// E > 64, fp32: the router's products x W_r[p]^T by the grouped fp32 GEMM into `logits` (groups = parties), then the gating pass reads them back, adds the
-// bias and overwrites them with the biased logits.
+// E > 64, fp32: the router's products x W_r[p]^T by the grouped fp32 GEMM into `logits` (groups =
+// parties), then the gating pass reads them back, adds the bias and overwrites them with the
+// biased logits.
 static cudaError_t launch_route_wide_f32(const RouteArgs& a, cudaStream_t s) {
     GemmMArgs m{};
     m.G = (a.po && a.P > 1) ? a.P : 1;
