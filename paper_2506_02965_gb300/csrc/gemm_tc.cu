@@ -988,68 +988,94 @@ __global__ void __launch_bounds__(gemm_threads(EW), OCC)
             }
             fence_after();
             const uint32_t tmem_d = tmem_base + (uint32_t)(acc * BN);
-            for (int kb = 0; kb < ti.k_iters; ++kb) {
-                const bool got = wait_bar(full_bar(stage), phase);
-                const uint32_t sa = ring + stage * STAGE_BYTES;
-                const uint32_t sb = sa + A_BYTES;
-                // K-variable groups: the last k-block may hold contraction rows of the next
-                // group. Only K=16 steps that contain valid rows are issued, and inside the
-                // last of them the A rows past the group's end are zeroed (A alone suffices:
-                // their products with any finite B row vanish).
-                const bool dwt = DW2 && ti.dw;
-                const bool part = (VAR_K || dwt) && kb == ti.k_iters - 1 && ti.last_rows < KB;
-                const int ksteps = part ? (ti.last_rows + 15) / 16 : KB * KPS / 16;
-                if (part) {
-                    const int zr0 = ti.last_rows, zr1 = ksteps * 16;
-                    if (got && zr1 > zr0) {
-                        uint8_t* base = ring_ptr + (size_t)stage * STAGE_BYTES;
-                        const int per_box = (zr1 - zr0) * 8;  // 16-byte words
+            const bool dwt = DW2 && ti.dw;
+            // the MMAs of a k-block in stage `st`, and its release (one thread)
+            auto issue = [&](int st, int kb, int ksteps, bool part) {
+                const uint32_t sa = ring + st * STAGE_BYTES, sb = sa + A_BYTES;
+                auto step = [&](int kk, bool swapped) {
+                    uint64_t ad, bd;
+                    if (!A_MN && !dwt) ad = smem_desc(sa + (kk / (KB / 16)) * A_BOX + (kk % (KB / 16)) * 32, 16, 1024);
+                    else ad = smem_desc(sa + (kk / (KB / 16)) * A_BOX + (kk % (KB / 16)) * 2048, ATOM, 1024);
+                    if (!B_MN) bd = smem_desc(sb + (kk / (KB / 16)) * B_BOX + (kk % (KB / 16)) * 32, 16, 1024);
+                    else bd = smem_desc(sb + kk * 2048, ATOM_B, 1024);
+                    if (SWAP && swapped) mma_bf16_pair(tmem_d, bd, ad, idesc_s, (kb | kk) ? 1u : 0u);
+                    else if constexpr (PAIR) mma_bf16_pair(tmem_d, ad, bd, IDESC, (kb | kk) ? 1u : 0u);
+                    else mma_bf16(tmem_d, ad, bd, dwt ? IDESC_DW : IDESC, (kb | kk) ? 1u : 0u);
+                };
+                // whole k-blocks without a check per step (with one, the issuing thread
+                // held back the weight-gradient launches by up to 20%)
+                if (SWAP && ti.ntok) {
 #pragma unroll
-                        for (int b = 0; b < BM / 64; ++b) {
-                            uint4* z = reinterpret_cast<uint4*>(base + b * ATOM + zr0 * 128);
-                            for (int i = lane; i < per_box; i += 32) z[i] = make_uint4(0, 0, 0, 0);
-                        }
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    }
-                    __syncwarp();
-                }
-                fence_after();
-                if (lane == 0 && got) {
-                    auto step = [&](int kk, bool swapped) {
-                        uint64_t ad, bd;
-                        if (!A_MN && !dwt) ad = smem_desc(sa + (kk / (KB / 16)) * A_BOX + (kk % (KB / 16)) * 32, 16, 1024);
-                        else ad = smem_desc(sa + (kk / (KB / 16)) * A_BOX + (kk % (KB / 16)) * 2048, ATOM, 1024);
-                        if (!B_MN) bd = smem_desc(sb + (kk / (KB / 16)) * B_BOX + (kk % (KB / 16)) * 32, 16, 1024);
-                        else bd = smem_desc(sb + kk * 2048, ATOM_B, 1024);
-                        if (SWAP && swapped) mma_bf16_pair(tmem_d, bd, ad, idesc_s, (kb | kk) ? 1u : 0u);
-                        else if constexpr (PAIR) mma_bf16_pair(tmem_d, ad, bd, IDESC, (kb | kk) ? 1u : 0u);
-                        else mma_bf16(tmem_d, ad, bd, dwt ? IDESC_DW : IDESC, (kb | kk) ? 1u : 0u);
-                    };
-                    // whole k-blocks without a check per step (with one, the issuing thread
-                    // held back the weight-gradient launches by up to 20%)
-                    if (SWAP && ti.ntok) {
+                    for (int kk = 0; kk < KB * KPS / 16; ++kk) step(kk, true);
+                } else if (!part) {
 #pragma unroll
-                        for (int kk = 0; kk < KB * KPS / 16; ++kk) step(kk, true);
-                    } else if (!part) {
-#pragma unroll
-                        for (int kk = 0; kk < KB * KPS / 16; ++kk) step(kk, false);
-                    } else {
+                    for (int kk = 0; kk < KB * KPS / 16; ++kk) step(kk, false);
+                } else {
 #pragma unroll 1
-                        for (int kk = 0; kk < ksteps; ++kk) step(kk, false);
+                    for (int kk = 0; kk < ksteps; ++kk) step(kk, false);
+                }
+                if constexpr (PAIR) mma_commit_pair(empty_bar(st), 3);  // both producers
+                else mma_commit(empty_bar(st));
+                issued_any = true;
+            };
+            // One answer to the warp, whether a wait gave up: after the MMAs of a k-block are on their
+            // way (before them it cost up to 1% of a step), or, where a stage is a single k-block of
+            // a pair (dA: 247 -> 263 us by that vote) and one thread waits and issues (245; the other
+            // forms lose 1 to 5% by that), at the tile's end. After a wait that gave up nothing more
+            // is issued or released: what the other CTA of a pair would then copy is armed by no one.
+            if constexpr (PAIR && !VAR_K && KPS == 1) {
+                if (lane == 0) {
+                    int st = stage;
+                    uint32_t ph = phase;
+                    for (int kb = 0; kb < ti.k_iters; ++kb) {
+                        if (!wait_bar(full_bar(st), ph)) {
+                            ok = false;
+                            break;
+                        }
+                        fence_after();
+                        issue(st, kb, KB * KPS / 16, false);
+                        if (++st == NST) {
+                            st = 0;
+                            ph ^= 1u;
+                        }
                     }
-                    if constexpr (PAIR) mma_commit_pair(empty_bar(stage), 3);  // both producers
-                    else mma_commit(empty_bar(stage));
-                    issued_any = true;
                 }
-                // one answer to the warp, after the MMAs are on their way (a vote before them cost
-                // up to 1% of a step)
-                if (!__all_sync(0xffffffffu, got)) {
-                    ok = false;
-                    break;
-                }
-                if (++stage == NST) {
-                    stage = 0;
-                    phase ^= 1u;
+                phase ^= (uint32_t)((stage + ti.k_iters) / NST) & 1u;
+                stage = (stage + ti.k_iters) % NST;
+                ok = __all_sync(0xffffffffu, ok);
+            } else {
+                for (int kb = 0; kb < ti.k_iters; ++kb) {
+                    const bool got = wait_bar(full_bar(stage), phase);
+                    // K-variable groups: the last k-block may hold contraction rows of the next
+                    // group. Only K=16 steps that contain valid rows are issued, and inside the
+                    // last of them the A rows past the group's end are zeroed (A alone suffices:
+                    // their products with any finite B row vanish).
+                    const bool part = (VAR_K || dwt) && kb == ti.k_iters - 1 && ti.last_rows < KB;
+                    const int ksteps = part ? (ti.last_rows + 15) / 16 : KB * KPS / 16;
+                    if (part) {
+                        const int zr0 = ti.last_rows, zr1 = ksteps * 16;
+                        if (got && zr1 > zr0) {
+                            uint8_t* base = ring_ptr + (size_t)stage * STAGE_BYTES;
+                            const int per_box = (zr1 - zr0) * 8;  // 16-byte words
+#pragma unroll
+                            for (int b = 0; b < BM / 64; ++b) {
+                                uint4* z = reinterpret_cast<uint4*>(base + b * ATOM + zr0 * 128);
+                                for (int i = lane; i < per_box; i += 32) z[i] = make_uint4(0, 0, 0, 0);
+                            }
+                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        }
+                        __syncwarp();
+                    }
+                    fence_after();
+                    if (lane == 0 && got) issue(stage, kb, ksteps, part);
+                    if (!__all_sync(0xffffffffu, got)) {
+                        ok = false;
+                        break;
+                    }
+                    if (++stage == NST) {
+                        stage = 0;
+                        phase ^= 1u;
+                    }
                 }
             }
             if (!ok) break;
