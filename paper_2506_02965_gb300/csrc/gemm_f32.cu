@@ -12,10 +12,10 @@
 // below 2^-110: 6e-5 off for operands of 2^-120.) The tensor core's fp32 accumulator truncates, which over a long contraction
 // loses more than an FFMA chain does, so an accumulator holds only 32 contraction terms
 // (the smallest products first) and is then added to fp32 registers with round-to-nearest.
-// Measured against 64 bits, the worst tensor of a whole fp32 step is 2.4e-7 (512 tokens,
-// d = 256, F = 512) and 5e-7 (1501 tokens, d = 1000, F = 1366) off; the FFMA kernels that
-// this replaces were 7.1e-7 and 1.5e-6 off, and accumulators of 64 terms (1.5% faster)
-// 8.3e-7 and 1.1e-6.
+// Measured against 64 bits, the worst tensor of a whole fp32 step is 4.2e-7 (512 tokens, d = 256,
+// F = 512) and 3.1e-7 (1501 tokens, d = 1000, F = 1366) off, where the FFMA kernels that this
+// replaces were 8.7e-7 and 1.2e-6 off on the same inputs (another seed: 2.5e-7 and 3.1e-7 for
+// 7.1e-7 and 1.3e-6). Accumulators of 64 terms (1.5% faster) were further off than those.
 //
 // Roles (one persistent CTA per SM, 128 x BN tiles): 16 producer warps copy fp32 into
 // shared memory up to two stages ahead (cp.async), split it and write three swizzled bf16
@@ -23,12 +23,13 @@
 // stage into one of four TMEM accumulators; 8 warps add the accumulators into registers and
 // run the epilogue. cp.async and not TMA because lines need only 4-byte alignment (any d_ff).
 //
-// What bounds it: shared-memory bandwidth. A 32-deep stage of a 128 x 128 tile is 32 KB of
-// fp32 written and read, 48 KB of planes written, and 96 KB of operand reads by the MMAs;
-// the counters show the LSU pipe at 41% and the tensor pipe's reads at 47% (accumulating an
-// eighth as often, or issuing one MMA of six, changed the time by 10% and 4%). Whole fp32 steps:
-// 1501 tokens, d = 1000, F = 1366, E = 6, k = 3: 5.39 -> 1.13 ms (21 -> 98 TFLOP/s);
-// 512 tokens, d = 256, F = 512, E = 8, k = 2: 493 -> 133 us.
+// What bounds it: no single unit. A 32-deep stage of a 128 x 128 tile is 32 KB of fp32 written and
+// read, 48 KB of planes written, and 96 KB of operand reads by the MMAs; in the counters
+// instructions issue in 56-66% of the cycles (most of them the split's), loads and stores take
+// 33-44% of the shared-memory wavefronts, the tensor pipe is 24-35% busy, DRAM 4-9%. (Accumulating
+// an eighth as often, or issuing one MMA of six, changed the time by 10% and 4%.) Whole fp32 steps:
+// 1501 tokens, d = 1000, F = 1366, E = 6, k = 3: 5.40 -> 1.14 ms (21 -> 97 TFLOP/s);
+// 512 tokens, d = 256, F = 512, E = 8, k = 2: 494 -> 128 us.
 //
 // An infinite or NaN operand makes 0 * inf terms in the split, and operands from 2^105 or sums
 // from 2^82 on leave the scaled range, so an output element that is not finite is computed

@@ -1,7 +1,8 @@
 """The fp32 grouped GEMMs (three-way bf16 split on the tensor cores) at the edges of their
 tiles and copies: contractions around the 32-term stage, lines
 of 4-, 8- and 16-byte alignment, row counts around the 128-row tile, empty experts, one and
-several tiles per CTA; and infinities, NaN and the largest finite values.
+several tiles per CTA; operands and sums at both ends of the range, infinities and NaN; an
+operand that is aligned to its elements only.
 
 Bound per element of a contraction c = sum a_i b_i: the split leaves out terms below
 3 * 2^-25 |a_i b_i|; each of the 12 accumulation steps per 32 terms and each register
