@@ -191,7 +191,8 @@ moe_status moe_gather_rows(const void* src, const int32_t* rows, int64_t n_rows,
  *   act [TK,F] out; y_perm [TK,d] out.
  * Shared experts (all NULL when S == 0): x [T,d]; ws1 [S,2Fs,d]; ws2 [S,d,Fs];
  *   h_gu_sh [S,T,2Fs] out; act_sh [S,T,Fs] out; y_sh [S,T,d] out.
- * bf16: tcgen05 tensor-core GEMMs, fp32 accumulation in TMEM, bf16 outputs.
+ * bf16: tcgen05 tensor-core GEMMs, fp32 accumulation in TMEM, bf16 outputs. fp32: tensor cores
+ * on exact three-way bf16 splits of both operands, fp32 results (here and in the backward).
  * group_expert [E] i32 (from moe_dispatch_owner) or NULL: segment g of x_perm (rows
  *   [offsets[g], offsets[g+1])) belongs to expert group_expert[g] (NULL: to expert g).
  */
@@ -204,7 +205,8 @@ moe_status moe_expert_ffn_fwd(const moe_config* cfg, const void* x_perm, const i
 /* Number of CUDA kernels one moe_expert_ffn_bwd call with this configuration launches
  * (host only, no device work): per weight, the input-gradient GEMM and the weight
  * gradient in one persistent launch, or in two (CTA-pair tiles, moe_set_gemm_pairs,
- * and the fp32 path), plus four for the shared experts; 0 GEMMs when T*k == 0. */
+ * widths of 128 mod 256, which that launch does not take, and the fp32 path), plus four
+ * for the shared experts; 0 GEMMs when T*k == 0. */
 moe_status moe_expert_ffn_bwd_kernels(const moe_config* cfg, int32_t* count /* HOST out */);
 
 /*
